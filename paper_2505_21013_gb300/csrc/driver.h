@@ -130,7 +130,9 @@ struct Group {
   size_t cap_halo = 0;
   const int *halo_off = nullptr, *halo_col = nullptr, *halo_ref = nullptr;
   int halo_cap = 0;
-  GridBar* d_bar = nullptr;
+  TeamJob* d_jobs = nullptr;  // job table of the team launches
+  size_t cap_jobs = 0;
+  GridBar* d_bar = nullptr;   // [2]: of the lockstep and single-scene launches, of the team launches
   cudaStream_t st = nullptr;
   Staging staging;
   KernelTimer* timer = nullptr;
@@ -155,6 +157,8 @@ struct Group {
     h_bar = nullptr;
     d_halo = nullptr;
     cap_halo = 0;
+    d_jobs = nullptr;
+    cap_jobs = 0;
     cap_n = cap_tt = cap_vt = cap_bt = cap_pt = cap_et = cap_proj = 0;
   }
   template <typename X>
@@ -215,21 +219,21 @@ struct Group {
       d_pcgtiles = alloc<TileRef>(cap_pt);
       d_touchtiles = alloc<TileRef>(cap_bt);
       d_flags = alloc<unsigned long long>(XCH_MAX_CTAS_HOST);
-      d_bar = alloc<GridBar>(1);
+      d_bar = alloc<GridBar>(2);
       if (!d_desc || !d_ctl || !d_ttiles || !d_vtiles || !d_btiles || !d_ptiles || !d_etiles ||
           !d_projtiles || !d_ids || !d_bar || !d_pcgtiles || !d_touchtiles) {
         set_error("cudaMalloc failed for a scene group");
         return PPN_ERR_OOM;
       }
       PPN_CU(cudaMallocHost(&h_ctl, sizeof(Ctl) * cap_n));
-      PPN_CU(cudaMallocHost(&h_bar, sizeof(GridBar)));
+      PPN_CU(cudaMallocHost(&h_bar, 2 * sizeof(GridBar)));
     }
     pcg_ids.clear();
     pcg_ntiles = 0;
     pcg_smem_bytes = 0;
     pcg_sr = false;
-    std::memset(h_bar, 0, sizeof(GridBar));
-    PPN_CU(cudaMemset(d_bar, 0, sizeof(GridBar)));
+    std::memset(h_bar, 0, 2 * sizeof(GridBar));
+    PPN_CU(cudaMemset(d_bar, 0, 2 * sizeof(GridBar)));
     PPN_CU(cudaMemcpy(d_ttiles, tt.data(), sizeof(TileRef) * tt.size(), cudaMemcpyHostToDevice));
     PPN_CU(cudaMemcpy(d_vtiles, vt.data(), sizeof(TileRef) * vt.size(), cudaMemcpyHostToDevice));
     PPN_CU(cudaMemcpy(d_btiles, bt.data(), sizeof(TileRef) * bt.size(), cudaMemcpyHostToDevice));
@@ -279,7 +283,7 @@ struct Group {
   }
   ppn_status sync_ctl() {
     PPN_CU(cudaMemcpyAsync(h_ctl, d_ctl, sizeof(Ctl) * S.size(), cudaMemcpyDeviceToHost, st));
-    PPN_CU(cudaMemcpyAsync(h_bar, d_bar, sizeof(GridBar), cudaMemcpyDeviceToHost, st));
+    PPN_CU(cudaMemcpyAsync(h_bar, d_bar, 2 * sizeof(GridBar), cudaMemcpyDeviceToHost, st));
     PPN_CU(cudaStreamSynchronize(st));
     staging.reset();
     if (timer) timer->collect();
@@ -364,6 +368,10 @@ struct Driver {
     G.set_active(on);
     ppn_status rc = G.upload_desc();
     if (rc) return rc;
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (G.S.size() > 1 && (rc = solve_teams(ids, b_from_g))) return rc;
+      if (ids.empty()) return PPN_OK;
+    }
     // slots of at most PCG_MAX_SCENES scenes per launch
     for (size_t b = 0; b < ids.size(); b += PCG_MAX_SCENES) {
       const size_t e = std::min(ids.size(), b + PCG_MAX_SCENES);
@@ -442,6 +450,116 @@ struct Driver {
         G.tune_slots = sl;
       }
     }
+    return PPN_OK;
+  }
+
+  // The halo tables of scene s alone, one or two tiles per CTA (two = 0, 1), built at the scene's
+  // first team launch of that form and kept with it.  False when its rows do not fit.
+  bool team_tables(SceneImpl<T>& s, int two, int n_sm) {
+    auto& t = s.team[two];
+    if (t.state) return t.state > 0;
+    t.state = -1;
+    const int size = two ? (s.n_ptiles + 1) / 2 : s.n_ptiles;
+    if (size > n_sm || s.nv >= (1 << HALO_ROW_BITS)) return false;
+    int slots = 0;  // most block slots of one CTA (as plan_smem counts them)
+    for (int b = 0; b < size; ++b) {
+      const int t0 = (int)(((long long)b * s.n_ptiles) / size), t1 = (int)(((long long)(b + 1) * s.n_ptiles) / size);
+      const int r1 = std::min(s.nv, t1 * PCG_TILE);
+      int n = 0;
+      for (int g = t0 * PCG_TILE; g < r1; g += 16) {
+        int m = 0;
+        for (int r = g; r < std::min(r1, g + 16); ++r) m = std::max(m, (int)(s.h_row_ptr[r + 1] - s.h_row_ptr[r]));
+        n += 32 * ((m + 1) / 2);
+      }
+      slots = std::max(slots, n);
+    }
+    const int rows = (s.n_ptiles + size - 1) / size * PCG_TILE;
+    if (pcg_sr_smem_bytes(rows, slots, 0, SR_HALO) > (size_t)227 * 1024) return false;
+    std::vector<int> tab;
+    const int nh = build_halo_tables({{s.nv, s.h_row_ptr.data(), s.h_col.data()}}, size, tab);
+    if (nh < 0) return false;
+    const size_t smem = pcg_sr_smem_bytes(rows, slots, nh, SR_HALO);
+    // (leaves room for the kernel's static shared memory)
+    if (smem > (size_t)220 * 1024) return false;
+    t.d_tab = (int*)dev_alloc(s.dalloc, sizeof(int) * tab.size());
+    if (!t.d_tab) {
+      cudaGetLastError();
+      t.state = 0;  // (memory may be free again later)
+      return false;
+    }
+    if (cudaMemcpyAsync(t.d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, G.st) != cudaSuccess ||
+        cudaStreamSynchronize(G.st) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    t.size = size;
+    t.slots = slots;
+    t.halo = nh;
+    t.smem = smem;
+    t.off = t.d_tab;
+    t.col = t.d_tab + 2 * (size + 1);
+    t.ref = t.col + tab[2 * size];
+    t.state = 1;
+    return true;
+  }
+
+  // A group of scenes: those whose rows fit a team of CTAs go into one team launch (k_pcg_team) and
+  // leave `ids`.  Two tiles per CTA use an SM's time best (4.5 us per iteration of two tiles, 3.1
+  // of one); one tile per CTA is taken while all scenes' tiles fit the device at once (9 scenes of
+  // 1k to 13k tets: 10.2 -> 7.1 ms per step against the lockstep form).  The jobs run longest
+  // first, by the scenes' last iteration counts.  A layout switch in the environment
+  // (tests) keeps the lockstep forms.
+  ppn_status solve_teams(std::vector<int>& ids, int b_from_g) {
+    for (const char* e : {"PPN_PCG_STD", "PPN_PCG_GLOBAL", "PPN_PCG_STREAM", "PPN_PCG_SR_GLOBAL", "PPN_PCG_NO_HALO"})
+      if (std::getenv(e)) return PPN_OK;
+    int dev = 0, n_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    long long tiles = 0;
+    for (int i : ids) tiles += G.S[i]->n_ptiles;
+    const int two = tiles > n_sm;
+    std::vector<int> in, out;
+    size_t smem = 0;
+    for (int i : ids) {
+      if (team_tables(*G.S[i], two, n_sm)) {
+        in.push_back(i);
+        smem = std::max(smem, G.S[i]->team[two].smem);
+      } else {
+        out.push_back(i);
+      }
+    }
+    const int max_grid = in.empty() ? 0 : pcg_team_max_grid(dev, smem);
+    int need = 0;
+    for (int i : in) need = std::max(need, G.S[i]->team[two].size);
+    if (max_grid < need || max_grid == 0) return PPN_OK;
+    std::stable_sort(in.begin(), in.end(), [&](int a, int b) {
+      const SceneImpl<T>&x = *G.S[a], &y = *G.S[b];
+      return x.last_cg != y.last_cg ? x.last_cg > y.last_cg : x.n_ptiles > y.n_ptiles;
+    });
+    std::vector<TeamJob> jobs;
+    int ticket = 0;
+    for (int i : in) {
+      SceneImpl<T>& s = *G.S[i];
+      const auto& t = s.team[two];
+      jobs.push_back({i, ticket, t.size, s.n_ptiles, t.slots, t.halo, t.off, t.col, t.ref});
+      ticket += t.size;
+      s.last_pcg_layout = SR_HALO;
+    }
+    if (!G.d_jobs || jobs.size() > G.cap_jobs) {
+      G.d_jobs = G.template alloc<TeamJob>(G.cap_n);
+      G.cap_jobs = G.d_jobs ? G.cap_n : 0;
+      if (!G.d_jobs) return PPN_OK;  // (the lockstep forms)
+    }
+    ppn_status rc = G.upload(G.d_jobs, jobs.data(), sizeof(TeamJob) * jobs.size());
+    if (rc) return rc;
+    TeamLaunch L{G.d_jobs, (int)jobs.size(), G.d_bar + 1, std::min(max_grid, ticket), b_from_g, smem};
+    cudaError_t err = cudaSuccess;
+    timed(FAM_PCG, 0.0, [&] { err = launch_pcg_team(reinterpret_cast<const SceneDev<float>*>(G.d_desc), L, G.st); });
+    if (err != cudaSuccess) {
+      set_error(std::string("PCG launch: ") + cudaGetErrorString(err));
+      return PPN_ERR_CUDA;
+    }
+    ids = out;
     return PPN_OK;
   }
 
@@ -1046,6 +1164,7 @@ struct Driver {
     h.ind = c.pcg_ind != 0;
     h.precond_fail = c.pcg_precond_fail;
     h.pcg_iters_last = c.pcg_iters;
+    G.S[i]->last_cg = c.pcg_iters;
     h.cur.pcg_attempts += 1;
     h.cur.cg_iters += c.pcg_iters;
     ppn_attempt a;
@@ -1073,8 +1192,10 @@ struct Driver {
         return PPN_ERR_TIMEOUT;
       }
     }
-    if (G.h_bar->timeout) {
-      const GridBar& b = *G.h_bar;
+    for (int k = 0; k < 2; ++k) {
+      if (!G.h_bar[k].timeout) continue;
+      const GridBar b = G.h_bar[k];
+      cudaMemsetAsync(G.d_bar, 0, 2 * sizeof(GridBar), G.st);  // reported once
       set_error("PCG grid wait timed out (wait " + std::to_string(b.to_site) + " at CG iteration " +
                 std::to_string(b.to_iter) + " in CTA " + std::to_string(b.to_cta) + ": word " +
                 std::to_string(b.to_slot) + "/" + std::to_string(b.to_index) + " last seen with stamp " +

@@ -93,6 +93,27 @@ struct PcgLaunch {
   size_t pword_bytes[PCG_MAX_SCENES];
 };
 
+// Team launch (single-reduction kernel, halo layout): every scene of a batch is a job solved by
+// a team of `size` CTAs of its own; the jobs' members are numbered one job after the other.
+struct TeamJob {
+  int scene;             // index into the scene table
+  int ticket;            // number of the team's first member
+  int size;              // its CTAs
+  int n_tiles;           // the scene's PCG row tiles
+  int slots, halo_cap;   // shared-memory capacities (block slots, halo rows) of the scene's tables
+  const int *halo_off, *halo_col, *halo_ref;  // as PcgLaunch's, for the scene alone over `size` CTAs
+};
+struct TeamLaunch {
+  const TeamJob* jobs;   // device
+  int n_jobs;
+  GridBar* bar;
+  int grid;              // co-resident CTAs
+  int use_b_from_g;
+  size_t smem_bytes;     // of the largest job
+};
+int pcg_team_max_grid(int device, size_t smem);
+cudaError_t launch_pcg_team(const SceneDev<float>* scenes, const TeamLaunch& L, cudaStream_t st);
+
 // dynamic shared memory of the resident PCG layout for ni rows and nb blocks
 size_t pcg_smem_bytes(int ni, int nb, int fsize);
 // co-resident grid of the resident PCG kernel with `smem` dynamic bytes (0: does not fit)

@@ -132,6 +132,7 @@ template <typename T>
 SceneImpl<T>::~SceneImpl() {
   if (stream) cudaStreamSynchronize(stream);
   for (void* p : allocs) dev_free(dalloc, p);
+  for (TeamTables& t : team) dev_free(dalloc, t.d_tab);
   if (h_ctl) cudaFreeHost(h_ctl);
   if (ev_a) cudaEventDestroy(ev_a);
   if (ev_b) cudaEventDestroy(ev_b);

@@ -1,0 +1,53 @@
+"""Team launches of the linear solver: in a batch every scene is solved by a team of
+CTAs of its own, instead of all scenes in lockstep over the whole grid.  Each scene's
+sums keep their order, so the steps equal those of the lockstep forms bit for bit
+(PPN_PCG_NO_HALO keeps the batch on them)."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+P = pytest.importorskip("paper_2505_21013_gb300")
+from ppn_inputs import cube_scene, twisting_beam_scene  # noqa: E402
+
+
+def beam(nx, ny, nz, seed, omega=4.0):
+    return twisting_beam_scene(nx, ny, nz, h=0.02, E=1e5, nu=0.45, omega=omega, dt=1 / 30, seed=seed)
+
+
+SETS = {
+    # all tiles fit the device at once: one 128-row tile per CTA (rows: 27, 128, 144, 910, 1331)
+    "one_tile": [cube_scene(3, seed=1), beam(4, 4, 8, 2), beam(4, 4, 9, 3), beam(7, 10, 13, 4, 20.0), cube_scene(11, seed=5)],
+    # more tiles than SMs: two tiles per CTA, teams of 1 to 13 CTAs, some queued behind others
+    "two_tiles": [beam(8, 8, 48 + k, 10 + k) for k in range(6)] + [cube_scene(3, seed=20), beam(4, 8, 8, 21)],
+    # a scene too large for a team (its rows do not fit two tiles per SM) beside two small ones
+    "too_large": [cube_scene(4, seed=30), cube_scene(35, seed=31), beam(5, 5, 12, 32)],
+}
+# the device has fewer SMs than the second set has tiles
+SETS["two_tiles"] += [beam(8, 8, 40, 40 + k) for k in range(4)]
+
+
+def run(specs, mode):
+    scs = [P.Scene.from_spec(s, precision=P.PREC_MIXED) for s in specs]
+    for n in range(2):
+        for sc, s in zip(scs, specs):
+            sc.set_targets(s.targets_at(n))
+        rc, st = P.ppn_step_batch(scs, [mode] * len(scs), 1e-4)
+        assert rc == 0
+    out = [sc.get_displacement()[0] for sc in scs]
+    layouts = [P.PCG_LAYOUTS[sc.info()["pcg_layout"]] for sc in scs]
+    for sc in scs:
+        sc.close()
+    return out, layouts, [(x["newton_iters"], x["total_cg_iters"], x["total_projections"]) for x in st]
+
+
+@pytest.mark.parametrize("name", list(SETS))
+def test_teams_equal_the_lockstep_forms(name, monkeypatch):
+    u, layouts, st = run(SETS[name], P.MODE_PPN)
+    monkeypatch.setenv("PPN_PCG_NO_HALO", "1")
+    u0, layouts0, st0 = run(SETS[name], P.MODE_PPN)
+    assert st == st0
+    assert all(np.array_equal(a, b) for a, b in zip(u, u0))
+    assert "halo" not in layouts0
+    assert [x for x in layouts if x != "halo"] == ([] if name != "too_large" else [layouts[1]])
