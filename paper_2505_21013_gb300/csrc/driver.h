@@ -113,6 +113,8 @@ struct Group {
   int pcg_ntiles = 0;
   size_t pcg_smem_bytes = 0;  // > 0: resident PCG layout chosen for that table
   int pcg_smem_blocks = 0, pcg_smem_grid = 0;
+  size_t rd_smem_bytes = 0;  // > 0: the unit kernel takes the standard resident kernel's place
+  int rd_slots = 0, rd_halo = 0, rd_grid = 0;
   bool pcg_sr = false;          // the single-reduction FP32 kernel was chosen for that table
   int pcg_sr_mode = 0;          // its layout (SR_RES, SR_STREAM, SR_GLOBAL)
   // layout chosen per launch by the tuner (SR_STREAM and SR_GLOBAL both fit)
@@ -231,6 +233,7 @@ struct Group {
     pcg_ids.clear();
     pcg_ntiles = 0;
     pcg_smem_bytes = 0;
+    rd_smem_bytes = 0;
     pcg_sr = false;
     std::memset(h_bar, 0, 2 * sizeof(GridBar));
     PPN_CU(cudaMemset(d_bar, 0, 2 * sizeof(GridBar)));
@@ -437,6 +440,22 @@ struct Driver {
             err = launch_pcg_sr(reinterpret_cast<const SceneDev<float>*>(G.d_desc), L, G.st);
             return;
           }
+        } else if (G.rd_smem_bytes) {
+          const SceneImpl<T>& s = *G.S[sl[0]];
+          RdLaunch<double> R{};
+          R.scene = reinterpret_cast<const SceneDev<double>*>(G.d_desc) + sl[0];
+          R.nv = s.nv;
+          R.n_units = (s.nv + 31) / 32;
+          R.grid = G.rd_grid;
+          R.slots = G.rd_slots;
+          R.halo_cap = G.rd_halo;
+          R.b_from_g = b_from_g;
+          R.resident = 1;
+          R.bar = G.d_bar;
+          R.unit_words = s.d.pword;
+          R.smem_bytes = G.rd_smem_bytes;
+          err = launch_pcg_rd<double>(R, G.st);
+          return;
         }
         err = L.smem_bytes ? launch_pcg_smem<T>(G.d_desc, L, G.st) : launch_pcg<T>(G.d_desc, L, G.st);
       });
@@ -582,6 +601,7 @@ struct Driver {
   // layout fits, else the global-memory kernel.
   void plan_smem(const std::vector<int>& sl, const std::vector<TileRef>& tt) {
     G.pcg_smem_bytes = 0;
+    G.rd_smem_bytes = 0;
     G.pcg_sr = false;
     G.pcg_tune = false;
     G.halo_off = G.halo_col = G.halo_ref = nullptr;
@@ -693,6 +713,46 @@ struct Driver {
     G.pcg_smem_bytes = bytes;
     G.pcg_smem_blocks = max_blocks;
     G.pcg_smem_grid = grid;
+    if constexpr (sizeof(T) == sizeof(double))
+      if (sl.size() == 1) plan_units(*G.S[sl[0]], dev, n_sm);
+  }
+
+  // FP64, one scene: the unit kernel (pcg_rd.cu) in place of the standard resident one (same
+  // bits) when its layout fits: rows in 32-row units over all SMs, where 128-row tiles leave
+  // most SMs idle and 5.4 us of FP64 work per SpMV on the others.  125 rows: 22 -> 10.5 us per CG
+  // iteration, 6480 rows: 23.2 -> 12.3.  PPN_PCG_NO_UNITS=1 keeps the standard kernel (tests).
+  void plan_units(const SceneImpl<T>& s, int dev, int n_sm) {
+    if (std::getenv("PPN_PCG_NO_UNITS") || s.n_ptiles > 512) return;
+    const int nu = (s.nv + 31) / 32, grid = std::min(nu, n_sm);
+    const int rows = 32 * ((nu + grid - 1) / grid);
+    if (rows > 160) return;
+    int slots = 0, halo = 0;
+    std::vector<int> mark(s.nv, -1);
+    for (int b = 0; b < grid; ++b) {
+      const int r0 = 32 * (int)(((long long)b * nu) / grid), re = 32 * (int)(((long long)(b + 1) * nu) / grid);
+      const int r1 = std::min(s.nv, re);
+      int n = 0, h = 0;
+      for (int g = r0; g < r1; g += 16) {
+        int m = 0;
+        for (int r = g; r < std::min(r1, g + 16); ++r) m = std::max(m, (int)(s.h_row_ptr[r + 1] - s.h_row_ptr[r]));
+        n += 32 * ((m + 1) / 2);
+      }
+      for (int64_t k = s.h_row_ptr[r0]; k < s.h_row_ptr[r1]; ++k) {
+        const int j = s.h_col[k];
+        if ((j < r0 || j >= re) && mark[j] != b) {
+          mark[j] = b;
+          ++h;
+        }
+      }
+      slots = std::max(slots, n);
+      halo = std::max(halo, h);
+    }
+    const size_t bytes = pcg_rd_smem_bytes<double>(nu, rows, slots, true, halo);
+    if (bytes > (size_t)224 * 1024 || pcg_rd_max_grid<double>(dev, bytes, true) < grid) return;
+    G.rd_smem_bytes = bytes;
+    G.rd_slots = slots;
+    G.rd_halo = halo;
+    G.rd_grid = grid;
   }
 
   // Start a time step for the flagged slots (their H[i].mode and H[i].tol set):

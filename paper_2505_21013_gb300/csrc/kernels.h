@@ -136,6 +136,30 @@ cudaError_t launch_wait_probe(const unsigned long long* w, int n, unsigned long 
 template <typename T>
 cudaError_t launch_pcg_smem(const SceneDev<T>* scenes, const PcgLaunch& L, cudaStream_t st);
 
+// Textbook recurrences, one scene per launch, rows in 32-row units over the CTAs, direction
+// replicated on the halo (pcg_rd.cu).  double: the arithmetic of launch_pcg_smem<double>;
+// float: that of launch_pcg<float> with four lanes per row.
+template <typename T>
+struct RdLaunch {
+  const SceneDev<T>* scene;        // device
+  int nv, n_units;                 // rows, units of 32 rows
+  int grid;                        // CTAs (co-resident); unit u of CTA b: [b n_units / grid, (b + 1) n_units / grid)
+  int slots, halo_cap;             // most block slots and halo rows of one CTA
+  int b_from_g;                    // as PcgLaunch's (float: b in r)
+  int resident;                    // float: blocks in shared memory, else read from L2 every iteration
+  GridBar* bar;
+  unsigned long long* unit_words;  // 16 words per unit
+  unsigned long long* z_words;     // float: 4 words per row (double: the scene's z and q arrays)
+  size_t smem_bytes;
+};
+template <typename T> size_t pcg_rd_smem_bytes(int n_units, int rows, int slots, bool resident, int halo);
+template <typename T> int pcg_rd_max_grid(int device, size_t smem, bool resident);
+template <typename T> cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st);
+// most block slots and halo rows of one CTA for a device-resident pattern (float form); the two
+// results must be zero before; nothing is done when *error is set
+cudaError_t launch_rd_plan(const int* row_ptr, const int* col, int n, int grid, const int* error, int* most_slots,
+                           int* most_halo, cudaStream_t st);
+
 // Occupancy-limited cooperative grid size for the chosen row group width.
 int pcg_max_grid(int group, int device);
 

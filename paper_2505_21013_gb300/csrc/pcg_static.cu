@@ -30,9 +30,10 @@
 // call waits for its stream before returning.  Separate processes have
 // separate arenas.
 //
-// The solver is the global-memory cooperative kernel of pcg.cu (group of four
-// lanes per row), so the arithmetic is the one a scene's solve performs with
-// that kernel.  Nothing here changes the scene path.
+// The solver is the unit kernel of pcg_rd.cu, or the global-memory cooperative
+// kernel of pcg.cu (group of four lanes per row) for patterns the former does not
+// take.  Both give the same bits, those of a scene's solve with the latter.
+// Nothing here changes the scene path.
 #include <cuda.h>
 
 #include <algorithm>
@@ -101,7 +102,8 @@ Arena carve(unsigned char* base, int n, int t) {
 
 struct DeviceSetup {
   unsigned char* base = nullptr;  // device address of g_pcg_static
-  int grid = 0;                   // co-resident CTAs of the solver
+  int grid = 0;                   // co-resident CTAs of the global-memory solver
+  int n_sm = 0;
   unsigned long long ctx = 0;     // id of the context the address belongs to (0: unknown)
 };
 std::mutex g_lock;
@@ -210,6 +212,8 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
       return fail(PPN_ERR_CUDA, std::string("ppn_pcg_solve_static: cudaGetSymbolAddress: ") + cudaGetErrorString(e));
     const int grid = pcg_max_grid(4, dev);
     if (grid <= 0) return fail(PPN_ERR_CUDA, "ppn_pcg_solve_static: solver occupancy query failed");
+    if (cudaDeviceGetAttribute(&D.n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || D.n_sm <= 0)
+      return fail(PPN_ERR_CUDA, "ppn_pcg_solve_static: device query failed");
     D.grid = grid;
     D.base = (unsigned char*)p;
     D.ctx = ctx;
@@ -229,6 +233,9 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   const int nb = (std::max(n_rows, n_tiles) + 255) / 256;
   k_static_prep<<<nb, 256, 0, st>>>(row_ptr, col, n_rows, nnzb, A.diag, A.tiles, n_tiles, A.ctl);
   PPN_STATIC_CU(cudaGetLastError());
+  // the unit kernel's shared-memory needs for this pattern (two counters of the control block)
+  const int n_units = (n_rows + 31) / 32, rd_grid = std::min(n_units, D.n_sm);
+  PPN_STATIC_CU(launch_rd_plan(row_ptr, col, n_rows, rd_grid, &A.ctl->error, &A.ctl->n_new, &A.ctl->n_touched, st));
   Ctl c{};
   PPN_STATIC_CU(cudaMemcpyAsync(&c, A.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   PPN_STATIC_CU(cudaStreamSynchronize(st));
@@ -255,8 +262,22 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   s.pcg_tol2 = rel_tol * rel_tol;
   s.pcg_max_iter = max_iter > 0 ? max_iter : std::max(1000, 3 * n_rows);
   s.active = 1;
+  // The unit kernel (pcg_rd.cu; same bits) where its rows' vectors fit in shared memory, with the blocks
+  // resident too when they fit: 32000 rows 24.9 -> 13.2 us per CG iteration, 546 rows 19.5 -> 6.9; a
+  // pattern with too many halo rows per CTA keeps the global-memory kernel.
+  RdLaunch<float> R{};
+  const int rd_rows = 32 * ((n_units + rd_grid - 1) / rd_grid);
+  bool units = rd_rows <= 512 && c.n_touched <= 4096;
+  for (int resident = 1; units && resident >= 0; --resident) {
+    R.smem_bytes = pcg_rd_smem_bytes<float>(n_units, rd_rows, c.n_new, resident != 0, c.n_touched);
+    R.resident = resident;
+    if (R.smem_bytes <= (size_t)224 * 1024 && pcg_rd_max_grid<float>(dev, R.smem_bytes, resident != 0) >= rd_grid) break;
+    if (resident == 0) units = false;
+  }
+  const bool copy_b = !units || (reinterpret_cast<uintptr_t>(b) & 15u);
+  if (!copy_b) s.r = const_cast<float4*>(reinterpret_cast<const float4*>(b));  // read only by the solver
   PPN_STATIC_CU(cudaMemcpyAsync(A.desc, &s, sizeof(s), cudaMemcpyHostToDevice, st));
-  PPN_STATIC_CU(cudaMemcpyAsync(A.r, b, sizeof(float4) * n_rows, cudaMemcpyDeviceToDevice, st));
+  if (copy_b) PPN_STATIC_CU(cudaMemcpyAsync(A.r, b, sizeof(float4) * n_rows, cudaMemcpyDeviceToDevice, st));
 
   PcgLaunch L{};
   L.n_tiles = n_tiles;
@@ -267,7 +288,20 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   L.grid = std::min(D.grid, n_tiles);
   L.group = 4;
   L.use_b_from_g = 0;
-  PPN_STATIC_CU(launch_pcg<float>(A.desc, L, st));
+  if (units) {
+    R.scene = A.desc;
+    R.nv = n_rows;
+    R.n_units = n_units;
+    R.grid = rd_grid;
+    R.slots = c.n_new;
+    R.halo_cap = c.n_touched;
+    R.bar = A.bar;
+    R.z_words = reinterpret_cast<unsigned long long*>(A.z);      // 32 bytes per row: z and the q after it
+    R.unit_words = reinterpret_cast<unsigned long long*>(A.d0);  // 128 bytes per 32 rows
+    PPN_STATIC_CU(launch_pcg_rd<float>(R, st));
+  } else {
+    PPN_STATIC_CU(launch_pcg<float>(A.desc, L, st));
+  }
   GridBar bar{};
   PPN_STATIC_CU(cudaMemcpyAsync(&c, A.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   PPN_STATIC_CU(cudaMemcpyAsync(&bar, A.bar, sizeof(GridBar), cudaMemcpyDeviceToHost, st));

@@ -1,0 +1,81 @@
+"""The unit kernel of the linear solver (32-row units, direction replicated on the halo)
+against the kernels whose arithmetic it keeps: FP64 scenes against the standard resident
+kernel, the allocation-free solve against the global-memory kernel.  Same sums in the
+same order, so the iterates are equal bit for bit at every size: fewer rows than a unit,
+exact and ragged units and tiles, one and several units per CTA, more tiles than lanes."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+P = pytest.importorskip("paper_2505_21013_gb300")
+from ppn_inputs import kuhn_grid, twisting_beam_scene  # noqa: E402
+
+# rows: 8, 32, 45, 128, 156, 1024, 4864 (152 units), 6480 (two units on some CTAs), 10290 (several)
+DIMS = [(2, 2, 2), (2, 4, 4), (3, 3, 5), (4, 4, 8), (3, 4, 13), (8, 8, 16), (16, 16, 19), (12, 12, 45), (14, 15, 49)]
+
+
+def springs(dims, seed, indefinite=False):
+    """An SPD (or, shifted, indefinite) block system on the pattern of a tet grid."""
+    X, tets = kuhn_grid(*dims, h=0.1, jitter=0.01, seed=seed)
+    n = len(X)
+    rng = np.random.default_rng(seed)
+    a = np.zeros((n, n), bool) if n < 200 else None
+    pairs = np.concatenate([tets[:, [i, j]] for i in range(4) for j in range(4)]).astype(np.int64)
+    key = np.unique(np.concatenate([pairs[:, 0] * n + pairs[:, 1], np.arange(n) * (n + 1)]))
+    del a
+    i, j = key // n, key % n
+    d = X[j] - X[i]
+    w = np.exp(rng.uniform(-1, 1, len(key)))
+    sym = np.minimum(i, j) * n + np.maximum(i, j)  # the same weight both ways
+    w = w[np.searchsorted(key, sym)]
+    K = -w[:, None, None] * (d[:, :, None] * d[:, None, :] * 100 + 0.1 * np.eye(3))
+    K[i == j] = 0
+    D = np.zeros((n, 3, 3))
+    np.add.at(D, i, -K)
+    K[i == j] = D + (-0.6 if indefinite else 0.05) * np.eye(3)
+    row_ptr = np.concatenate([[0], np.cumsum(np.bincount(i, minlength=n))])
+    return X, row_ptr, j.astype(np.int32), K, rng.standard_normal((n, 3))
+
+
+@pytest.mark.parametrize("indefinite", [False, True])
+@pytest.mark.parametrize("dims", DIMS)
+def test_fp64_scenes(dims, indefinite, monkeypatch):
+    spec = twisting_beam_scene(*dims, h=0.1, seed=3)
+    sc = P.Scene.from_spec(spec, precision=P.PREC_FP64)
+    rp, col = sc.probe_pattern()
+    _, rp2, col2, K, b = springs(dims, 5, indefinite)
+    assert np.array_equal(rp, rp2) and np.array_equal(col, col2)
+    x, info = sc.probe_pcg(K, b, rel_tol=1e-7)
+    sc.close()
+    monkeypatch.setenv("PPN_PCG_NO_UNITS", "1")
+    sc = P.Scene.from_spec(spec, precision=P.PREC_FP64)
+    x0, info0 = sc.probe_pcg(K, b, rel_tol=1e-7)
+    sc.close()
+    assert info == info0 and (info["ind"] or not indefinite)
+    assert np.array_equal(x, x0), (np.abs(x - x0).max(), info)
+
+
+@pytest.mark.parametrize("dims", DIMS + [(20, 20, 80), (27, 30, 70), (32, 32, 64)])
+def test_allocation_free_solve(dims, monkeypatch):
+    # the scene's solve through the global-memory kernel is the reference; 32000 rows keep their
+    # blocks in shared memory, 56700 and 65536 (the most that is taken) read them from L2
+    spec = twisting_beam_scene(*dims, h=0.1, seed=3)
+    _, rp, col, K, b = springs(dims, 6)
+    monkeypatch.setenv("PPN_PCG_GLOBAL", "1")
+    sc = P.Scene.from_spec(spec, precision=P.PREC_MIXED)
+    x0, info0 = sc.probe_pcg(K, b, rel_tol=1e-5)
+    sc.close()
+    dev = torch.device("cuda", 0)
+    n = len(rp) - 1
+    b4 = np.zeros((n, 4), np.float32)
+    b4[:, :3] = b
+    d_rp, d_col = torch.tensor(rp.astype(np.int32), device=dev), torch.tensor(col, device=dev)
+    d_val = torch.tensor(np.ascontiguousarray(K.reshape(-1, 9).T.astype(np.float32)), device=dev)
+    d_x = torch.tensor(b4, device=dev)  # the solution may take the right-hand side's place
+    info = P.ppn.pcg_solve_static(d_rp.data_ptr(), d_col.data_ptr(), d_val.data_ptr(), n, len(col), d_x.data_ptr(),
+                                  d_x.data_ptr(), rel_tol=1e-5)
+    assert info == info0
+    assert np.array_equal(d_x[:, :3].cpu().numpy().astype(np.float64), x0)
