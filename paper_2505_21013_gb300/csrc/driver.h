@@ -114,7 +114,8 @@ struct Group {
   size_t pcg_smem_bytes = 0;  // > 0: resident PCG layout chosen for that table
   int pcg_smem_blocks = 0, pcg_smem_grid = 0;
   size_t rd_smem_bytes = 0;  // > 0: the unit kernel takes the standard resident kernel's place
-  int rd_slots = 0, rd_halo = 0, rd_grid = 0;
+  int rd_slots = 0, rd_halo = 0;
+  RdPlan rd_plan{};
   bool pcg_sr = false;          // the single-reduction FP32 kernel was chosen for that table
   int pcg_sr_mode = 0;          // its layout (SR_RES, SR_STREAM, SR_GLOBAL)
   // layout chosen per launch by the tuner (SR_STREAM and SR_GLOBAL both fit)
@@ -444,15 +445,13 @@ struct Driver {
           const SceneImpl<T>& s = *G.S[sl[0]];
           RdLaunch<double> R{};
           R.scene = reinterpret_cast<const SceneDev<double>*>(G.d_desc) + sl[0];
-          R.nv = s.nv;
-          R.n_units = (s.nv + 31) / 32;
-          R.grid = G.rd_grid;
+          R.plan = G.rd_plan;
           R.slots = G.rd_slots;
           R.halo_cap = G.rd_halo;
           R.b_from_g = b_from_g;
           R.resident = 1;
           R.bar = G.d_bar;
-          R.unit_words = s.d.pword;
+          R.words = s.d.pword;
           R.smem_bytes = G.rd_smem_bytes;
           err = launch_pcg_rd<double>(R, G.st);
           return;
@@ -719,13 +718,13 @@ struct Driver {
 
   // FP64, one scene: the unit kernel (pcg_rd.cu) in place of the standard resident one (same
   // bits) when its layout fits: rows in 32-row units over all SMs, where 128-row tiles leave
-  // most SMs idle and 5.4 us of FP64 work per SpMV on the others.  125 rows: 22 -> 10.5 us per CG
-  // iteration, 6480 rows: 23.2 -> 12.3.  PPN_PCG_NO_UNITS=1 keeps the standard kernel (tests).
+  // most SMs idle and 5.4 us of FP64 work per SpMV on the others.  125 rows: 22 -> 8.9 us per CG
+  // iteration, 6480 rows: 23.2 -> 10.6.  PPN_PCG_NO_UNITS=1 keeps the standard kernel (tests).
   void plan_units(const SceneImpl<T>& s, int dev, int n_sm) {
     if (std::getenv("PPN_PCG_NO_UNITS") || s.n_ptiles > 512) return;
-    const int nu = (s.nv + 31) / 32, grid = std::min(nu, n_sm);
-    const int rows = 32 * ((nu + grid - 1) / grid);
-    if (rows > 160) return;
+    const RdPlan plan = rd_plan(s.nv, 32, n_sm);
+    if (plan.rows() > RD_ROWS_MAX_F64) return;
+    const int nu = plan.n_posts, grid = plan.grid;
     int slots = 0, halo = 0;
     std::vector<int> mark(s.nv, -1);
     for (int b = 0; b < grid; ++b) {
@@ -747,12 +746,12 @@ struct Driver {
       slots = std::max(slots, n);
       halo = std::max(halo, h);
     }
-    const size_t bytes = pcg_rd_smem_bytes<double>(nu, rows, slots, true, halo);
+    const size_t bytes = pcg_rd_smem_bytes<double>(plan, slots, true, halo);
     if (bytes > (size_t)224 * 1024 || pcg_rd_max_grid<double>(dev, bytes, true) < grid) return;
     G.rd_smem_bytes = bytes;
     G.rd_slots = slots;
     G.rd_halo = halo;
-    G.rd_grid = grid;
+    G.rd_plan = plan;
   }
 
   // Start a time step for the flagged slots (their H[i].mode and H[i].tol set):

@@ -139,25 +139,37 @@ cudaError_t launch_pcg_smem(const SceneDev<T>* scenes, const PcgLaunch& L, cudaS
 // Textbook recurrences, one scene per launch, rows in 32-row units over the CTAs, direction
 // replicated on the halo (pcg_rd.cu).  double: the arithmetic of launch_pcg_smem<double>;
 // float: that of launch_pcg<float> with four lanes per row.
+struct RdPlan {
+  int nv;         // rows
+  int post_rows;  // rows of one post of the exchanges: 32 (a unit) or 128 (a tile; float only)
+  int n_posts;
+  int grid;       // CTAs (co-resident); CTA b owns the posts [b n_posts / grid, (b + 1) n_posts / grid)
+  __host__ __device__ int rows() const { return (n_posts + grid - 1) / grid * post_rows; }  // of the largest CTA
+};
+inline RdPlan rd_plan(int nv, int post_rows, int n_sm) {
+  RdPlan p{nv, post_rows, (nv + post_rows - 1) / post_rows, 0};
+  p.grid = p.n_posts < n_sm ? p.n_posts : n_sm;
+  return p;
+}
+constexpr int RD_ROWS_MAX_F64 = 160;  // (three threads per row)
 template <typename T>
 struct RdLaunch {
-  const SceneDev<T>* scene;        // device
-  int nv, n_units;                 // rows, units of 32 rows
-  int grid;                        // CTAs (co-resident); unit u of CTA b: [b n_units / grid, (b + 1) n_units / grid)
-  int slots, halo_cap;             // most block slots and halo rows of one CTA
-  int b_from_g;                    // as PcgLaunch's (float: b in r)
-  int resident;                    // float: blocks in shared memory, else read from L2 every iteration
+  const SceneDev<T>* scene;   // device
+  RdPlan plan;
+  int slots, halo_cap;        // most block slots and halo rows of one CTA
+  int b_from_g;               // as PcgLaunch's (float: b in r)
+  int resident;               // float: blocks in shared memory, else read from L2 every iteration
   GridBar* bar;
-  unsigned long long* unit_words;  // 16 words per unit
-  unsigned long long* z_words;     // float: 4 words per row (double: the scene's z and q arrays)
+  unsigned long long* words;  // 32 words per post
+  unsigned long long* z_words;  // float: 3 words per row (double: the scene's z and q arrays)
   size_t smem_bytes;
 };
-template <typename T> size_t pcg_rd_smem_bytes(int n_units, int rows, int slots, bool resident, int halo);
+template <typename T> size_t pcg_rd_smem_bytes(const RdPlan& p, int slots, bool resident, int halo);
 template <typename T> int pcg_rd_max_grid(int device, size_t smem, bool resident);
 template <typename T> cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st);
 // most block slots and halo rows of one CTA for a device-resident pattern (float form); the two
 // results must be zero before; nothing is done when *error is set
-cudaError_t launch_rd_plan(const int* row_ptr, const int* col, int n, int grid, const int* error, int* most_slots,
+cudaError_t launch_rd_plan(const int* row_ptr, const int* col, const RdPlan& plan, const int* error, int* most_slots,
                            int* most_halo, cudaStream_t st);
 
 // Occupancy-limited cooperative grid size for the chosen row group width.

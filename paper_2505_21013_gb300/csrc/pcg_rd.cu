@@ -15,12 +15,17 @@
 //     not once per gathered block; what crosses CTAs is z of the halo rows;
 //   - in FP64 the SpMV and the updates go component by component over the threads, so that
 //     all four sub-partitions of an SM work on 32 rows; sums run only where rows are;
+//   - a warp's FP64 instruction holds its sub-partition for 64 cycles whatever its lanes do:
+//     levels of a tree that add only zeros are left out, comparisons look at the bits, both
+//     sums of the FP32 form share one warp's tree, and rows past the end hold zeros (a branch
+//     there ran the last CTA's sums once per side: 546 rows, 6.2 -> 5.5 us per CG iteration);
 //   - every value crosses the grid as 64-bit words that carry 32 bits and a 32-bit stamp
 //     (single-copy atomic: a word with the expected stamp carries the value, no fence).
 // Fixed order.  A unit's sum is the warp's tree over its rows (FP64 scenes: d.q by 16-row
 // halves), a tile's sum its units in order, a scene's sum the tiles lane-strided over a
-// warp and its tree: the order of the kernels named above.  A unit's words are rewritten
-// two exchanges later, after every CTA has read them.  All waits are bounded.
+// warp and its tree: the order of the kernels named above.  What is posted is a unit's
+// sums, or a whole tile's where a CTA has several tiles anyway (RdPlan).  A post's words are
+// rewritten two exchanges later, after every CTA has read them.  All waits are bounded.
 #include <algorithm>
 #include <type_traits>
 
@@ -34,7 +39,11 @@ namespace {
 
 constexpr int RD_NT = 512;  // threads per CTA
 constexpr int RD_NW = RD_NT / 32;
-constexpr int RD_LINE = 16;  // 64-bit words per unit (a 128-byte line): d.q at 0, r.z and r.r at 4, failed blocks at 8
+// 64-bit words per post: two 128-byte lines that one CTA writes, one per exchange (d.q, then the
+// failed blocks of the set-up; r.z and r.r).  Packing several posts' words in a line measured slower
+// (32000 rows, the d.q exchange 7.4 -> 13 k cycles), and so did both exchanges' words in one line (546
+// rows, r.z 4.6 -> 5.9 k cycles): every poll of a line delays the stores to it.
+constexpr int RD_LINE = 32, RD_DQ = 0, RD_FAIL = 8, RD_RZ = 16;
 
 template <typename T>
 struct RdCfg;
@@ -51,7 +60,8 @@ struct RdCfg<float> {
 
 template <typename T>
 struct RdSmem {
-  double *w, *t;            // the units' and the tiles' sums of an exchange
+  double *w, *t;            // the posts' and the tiles' sums of an exchange
+  double* u;                // the CTA's unit sums (posts of whole tiles)
   int *lrp, *lkb, *lgb;     // local row pointers, first global block of each row, first slot step of each group
   int *lcol, *href;         // local columns by slot; halo rows
   T* lval;                  // blocks by slot step: nine runs of 32 values
@@ -67,7 +77,7 @@ struct RdSmem {
 __host__ __device__ inline size_t rd_up16(size_t b) { return (b + 15) & ~size_t(15); }
 
 template <typename T>
-__host__ __device__ inline size_t rd_carve(char* base, int nu, int rows, int slots, bool resident, int nh, int hs,
+__host__ __device__ inline size_t rd_carve(char* base, int n_posts, int n_tiles, int rows, int slots, bool resident, int nh, int hs,
                                            RdSmem<T>* out) {
   size_t off = 0;
   auto take = [&](size_t b) {
@@ -78,8 +88,9 @@ __host__ __device__ inline size_t rd_carve(char* base, int nu, int rows, int slo
   RdSmem<T> s{};
   constexpr bool D = sizeof(T) == 8;
   const int gr = 32 / RdCfg<T>::G;
-  s.w = (double*)take(sizeof(double) * 2 * nu);
-  s.t = (double*)take(sizeof(double) * 2 * ((nu + 3) / 4));
+  s.w = (double*)take(sizeof(double) * 2 * n_posts);
+  s.t = (double*)take(sizeof(double) * 2 * n_tiles);
+  s.u = (double*)take(sizeof(double) * 2 * (rows / 32));
   s.lrp = (int*)take(sizeof(int) * (rows + 1));
   s.lkb = (int*)take(sizeof(int) * rows);
   s.lgb = (int*)take(sizeof(int) * (rows / gr + 1));
@@ -111,8 +122,8 @@ __host__ __device__ inline size_t rd_carve(char* base, int nu, int rows, int slo
   return off;
 }
 
-// the units [u0, u1) of CTA b
-__host__ __device__ inline int rd_unit(int b, int nu, int grid) { return (int)(((long long)b * nu) / grid); }
+// the posts [rd_post0(b), rd_post0(b + 1)) of CTA b
+__host__ __device__ inline int rd_post0(int b, int n_posts, int grid) { return (int)(((long long)b * n_posts) / grid); }
 
 // smallest power of two >= 2 n (at least 64)
 __host__ __device__ inline int rd_hash_size(int n) {
@@ -148,9 +159,45 @@ __device__ __forceinline__ void rd_post(unsigned long long* p, unsigned s, doubl
 __device__ __forceinline__ double rd_join(unsigned long long a, unsigned long long b) {
   return __longlong_as_double((long long)((a << 32) | (b & 0xffffffffull)));
 }
-// three products summed as k_pcg_s<double> sums them (d.q and r.z of a row)
+// three products summed as the kernels named above sum them
 __device__ __forceinline__ double rd_dot(double a0, double b0, double a1, double b1, double a2, double b2) {
   return __fma_rn(a2, b2, __fma_rn(a0, b0, __dmul_rn(a1, b1)));
+}
+__device__ __forceinline__ float rd_dot(float a0, float b0, float a1, float b1, float a2, float b2) {
+  return __fmaf_rn(a2, b2, __fmaf_rn(a0, b0, __fmul_rn(a1, b1)));
+}
+// after_dq and after_rz with their comparisons on the bits: FP64 compares cost as much as adds
+__device__ __forceinline__ bool rd_nan(double v) {
+  return ((unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ void rd_after_dq(SState<double>& s, double dq) {
+  s.dq = dq;
+  if (rd_nan(dq)) {
+    s.nonfinite = 1;
+    s.done = 1;
+  } else if (__double_as_longlong(dq) <= 0) {  // negative or zero of either sign
+    s.ind = 1;
+    s.done = 1;
+  } else {
+    s.alpha = s.rz / dq;
+  }
+}
+// stop: the squared tolerance times the squared norm of b (not negative, as r2)
+__device__ __forceinline__ void rd_after_rz(SState<double>& s, double rz, double r2, double stop, int max_iter) {
+  s.iters += 1;
+  s.rr = r2;
+  if (rd_nan(r2) || rd_nan(rz)) {
+    s.nonfinite = 1;
+    s.done = 1;
+  } else if (!rd_nan(stop) && __double_as_longlong(r2) <= __double_as_longlong(stop)) {
+    s.done = 1;
+  } else if (s.iters >= max_iter) {
+    s.hitmax = 1;
+    s.done = 1;
+  } else {
+    s.beta = rz / s.rz;
+    s.rz = rz;
+  }
 }
 // A tile sum as k_pcg_s<double> exchanges it (hi and lo words with 16 stamp bits each):
 // exact for every ordinary value; an infinite sum becomes a NaN and the last bits of a
@@ -166,11 +213,11 @@ __device__ __forceinline__ double rd_exchanged(double v) {
 }  // namespace
 
 template <typename T>
-size_t pcg_rd_smem_bytes(int nu, int rows, int slots, bool resident, int nh) {
-  return rd_carve<T>(nullptr, nu, rows, slots, resident, nh, rd_hash_size(nh), nullptr);
+size_t pcg_rd_smem_bytes(const RdPlan& p, int slots, bool resident, int nh) {
+  return rd_carve<T>(nullptr, p.n_posts, (p.nv + 127) / 128, p.rows(), slots, resident, nh, rd_hash_size(nh), nullptr);
 }
-template size_t pcg_rd_smem_bytes<double>(int, int, int, bool, int);
-template size_t pcg_rd_smem_bytes<float>(int, int, int, bool, int);
+template size_t pcg_rd_smem_bytes<double>(const RdPlan&, int, bool, int);
+template size_t pcg_rd_smem_bytes<float>(const RdPlan&, int, bool, int);
 
 // RES: the blocks stay in shared memory; else they are read from L2 every iteration
 template <typename T, bool RES>
@@ -180,19 +227,24 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
   extern __shared__ __align__(16) char dyn[];
   __shared__ SceneLite<T> S;
   __shared__ SState<double> st;
+  __shared__ double s_sum[2], s_stop;
+  __shared__ int s_bad[RD_NW];
   __shared__ int s_to, s_nh, s_fail, s_scan[RD_NW];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int grid = (int)gridDim.x, nu = A.n_units, n_tiles = (nu + 3) / 4;
-  const int u0 = rd_unit((int)blockIdx.x, nu, grid), u1 = rd_unit((int)blockIdx.x + 1, nu, grid);
-  const int row0 = 32 * u0, rows = 32 * (u1 - u0);  // (rows past the scene's last one are idle)
+  const int grid = (int)gridDim.x, n_posts = A.plan.n_posts, n_tiles = (A.plan.nv + PCG_TILE - 1) / PCG_TILE;
+  const int p0 = rd_post0((int)blockIdx.x, n_posts, grid), p1 = rd_post0((int)blockIdx.x + 1, n_posts, grid);
+  const int per = D ? 32 : A.plan.post_rows;        // rows per post: a unit (32) or a tile (128)
+  const int row0 = per * p0, rows = per * (p1 - p0);  // (rows past the scene's last one are idle)
+  unsigned long long* const my_words = A.words + (size_t)p0 * RD_LINE;
   const int hs = rd_hash_size(A.halo_cap);
   RdSmem<T> L;
-  rd_carve<T>(dyn, nu, rows, A.slots, RES, A.halo_cap, hs, &L);
+  rd_carve<T>(dyn, n_posts, n_tiles, rows, A.slots, RES, A.halo_cap, hs, &L);
   GridBar* bar = A.bar;
   if (tid == 0) {
     load_lite(S, *A.scene);
     s_to = s_nh = s_fail = 0;
   }
+  if (tid < RD_NW) s_bad[tid] = 0;
   for (int h = tid; h < hs; h += RD_NT) L.hkey[h] = -1;
   __syncthreads();
   const int nv = S.nv;
@@ -306,13 +358,16 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
     if (tid == 0) atomicExch(&bar->timeout, 1);
     return true;
   };
-  // The scene's sums of NQ quantities, VU values per unit and quantity, from the units' words at
-  // word offset `at` of their lines: unit sums to shared memory, tile sums in unit order, then one
-  // warp.  f(sums) runs in one thread; every thread returns after it.
-  auto sums = [&](unsigned s, int at, auto nq_, auto vu_, auto&& meanwhile, auto&& f) {
+  // The scene's sums of NQ quantities from the posts' words at word offset `at` (VU values per
+  // quantity): to shared memory, a tile's units in order, then one warp per quantity.  Levels of the
+  // warp's tree that would only add the zeros of lanes without a tile are left out: a warp's FP64
+  // instruction costs 64 cycles whatever its lanes do.  f(sums) runs in one thread; every thread
+  // returns after it.
+  auto sums = [&](unsigned s, int at, auto nq_, auto vu_, auto&& first, auto&& f) {
     constexpr int NQ = decltype(nq_)::value, VU = decltype(vu_)::value, NV = NQ * VU;
-    for (int u = tid; u < nu; u += RD_NT) {
-      const unsigned long long* p = A.unit_words + (size_t)u * RD_LINE + at;
+    first();
+    for (int u = tid; u < n_posts; u += RD_NT) {
+      const unsigned long long* p = A.words + (size_t)u * RD_LINE + at;
       unsigned long long w[2 * NV];
 #pragma unroll
       for (int q = 0; q < NV; ++q) rd_ld2(p + 2 * q, w[2 * q], w[2 * q + 1]);
@@ -322,76 +377,100 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
         L.w[NV * u + q] = rd_join(w[2 * q], w[2 * q + 1]);
       }
     }
-    meanwhile();
     __syncthreads();
     if (s_to) return;
-    for (int x = tid; x < NQ * n_tiles; x += RD_NT) {
-      const int t = x % n_tiles, q = x / n_tiles, n = min(4, nu - 4 * t);
-      // tile sums: (NQ = 2: value q of each unit; NQ = 1: the unit's VU values in row order)
-      double a;
-      if constexpr (NQ == 1 && VU == 2) {
-        a = 0.0;
-        for (int u = 0; u < 2 * n; ++u) a += L.w[8 * t + u];
-      } else {
-        const double* w = L.w + 4 * NQ * t + q;
-        a = w[0];
-        for (int u = 1; u < n; ++u) a += w[NQ * u];
+    // the sum of tile t of quantity q (values of units past the last one are zero)
+    auto tile_sum = [&](int t, int q) {
+      if (per == PCG_TILE) return L.w[NQ * t + q];
+      constexpr int NA = NQ == 1 ? 4 * VU : 4, step = NQ == 1 ? 1 : NV;
+      const double* w = L.w + 4 * NV * t + (NQ == 1 ? 0 : q);
+      const int n = min(4, n_posts - 4 * t) * (NQ == 1 ? VU : 1);
+      double v[NA];
+#pragma unroll
+      for (int u = 0; u < NA; ++u) v[u] = u < n ? w[step * u] : 0.0;
+#pragma unroll
+      for (int u = 1; u < NA; ++u) v[0] += v[u];
+      return D ? rd_exchanged(v[0]) : v[0];
+    };
+    const bool two = n_tiles > 32 && per != PCG_TILE;  // tile sums by all threads first
+    if (two) {
+      for (int x = tid; x < NQ * n_tiles; x += RD_NT) L.t[x] = tile_sum(x % n_tiles, x / n_tiles);
+      __syncthreads();
+    }
+    if (warp < NQ) {
+      double acc = 0.0;
+      if (lane < n_tiles) {
+        acc = two ? L.t[warp * n_tiles + lane] : tile_sum(lane, warp);
+        for (int k = lane + 32; k < n_tiles; k += 32) acc += two ? L.t[warp * n_tiles + k] : L.w[NQ * k + warp];
       }
-      L.t[q * n_tiles + t] = D ? rd_exchanged(a) : a;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (o < n_tiles) acc += __shfl_down_sync(0xffffffffu, acc, o);  // (uniform)
+      if (lane == 0) {
+        s_sum[warp] = acc;
+        if (NQ == 1) f(s_sum);
+      }
     }
     __syncthreads();
-    if (warp == 0) {
-      double acc[NQ];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-      for (int t = lane; t < n_tiles; t += 32)
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q] += L.t[q * n_tiles + t];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) acc[q] = warp_sum(acc[q]);
-      if (lane == 0) f(acc);
+    if (NQ > 1) {
+      if (tid == 0) f(s_sum);
+      __syncthreads();
     }
+  };
+  // unit lu's sum v (in one lane) of quantity q: posted at once, or kept for its tile's post
+  auto unit_sum = [&](int lu, int q, int at, unsigned s, double v) {
+    if (per == PCG_TILE)
+      L.u[2 * lu + q] = v;
+    else
+      rd_post(my_words + (size_t)lu * RD_LINE + at, s, v);
+  };
+  // the posts of whole tiles: nq sums of four units each, in unit order
+  auto post_tiles = [&](int nq, int at, unsigned s) {
+    if (per != PCG_TILE) return;
     __syncthreads();
+    for (int x = tid; x < nq * (rows / PCG_TILE); x += RD_NT) {
+      const int q = x % nq, t = x / nq;
+      const double* u = L.u + 8 * t + q;
+      rd_post(my_words + (size_t)t * RD_LINE + at + 2 * q, s, ((u[0] + u[2]) + u[4]) + u[6]);
+    }
   };
   using I1 = std::integral_constant<int, 1>;
   using I2 = std::integral_constant<int, 2>;
   auto nothing = [] {};
 
-  // z of the own rows out (stamp s), z of the halo rows in
-  auto post_z = [&](int i, int c, T z, unsigned s) {
-    if constexpr (D) {
-      rd_post(reinterpret_cast<unsigned long long*>(c < 2 ? S.z + i : S.q + i) + 2 * (c & 1), s, z);
-    } else {
-      (void)c, (void)z, (void)i;
-    }
+  // z of the own rows out (stamp s), z of the halo rows in (before the sums' words, which are posted
+  // later, and by the last threads first, which have no such words to wait for)
+  // The words lie by component, so that a warp's rows store and load whole runs.
+  auto z_pair = [&](int c, int i) {  // double: the two words of component c of row i
+    return reinterpret_cast<unsigned long long*>(c < 2 ? S.z : S.q) + 2 * ((size_t)(c & 1) * nv + i);
   };
   auto read_halo = [&](unsigned s) {
     if constexpr (D) {
-      T* dst[3] = {L.zx, L.zy, L.zz};
-      for (int x = tid; x < 3 * nh; x += RD_NT) {
-        const int h = x / 3, c = x - 3 * h, i = L.href[h];
-        const unsigned long long* p =
-            reinterpret_cast<const unsigned long long*>(c < 2 ? S.z + i : S.q + i) + 2 * (c & 1);
+      for (int x = RD_NT - 1 - tid; x < 3 * nh; x += RD_NT) {
+        const int c = (x >= nh) + (x >= 2 * nh), h = x - c * nh;
+        const unsigned long long* p = z_pair(c, L.href[h]);
         unsigned long long a, b;
         rd_ld2(p, a, b);
         wait2(p, s, a, b);
-        dst[c][rows + h] = rd_join(a, b);
+        (c == 0 ? L.zx : c == 1 ? L.zy : L.zz)[rows + h] = rd_join(a, b);
       }
     } else {
-      for (int h = tid; h < nh; h += RD_NT) {
-        const unsigned long long* p = A.z_words + 4 * (size_t)L.href[h];
-        unsigned long long a, b, c = ld_relaxed_u64(p + 2);
-        rd_ld2(p, a, b);
-        wait2(p, s, a, b);
-        for (unsigned spins = 0; !has(c, s); ++spins) {
+      for (int h = RD_NT - 1 - tid; h < nh; h += RD_NT) {
+        const unsigned long long* p = A.z_words + L.href[h];
+        unsigned long long w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) w[c] = ld_relaxed_u64(p + (size_t)c * nv);
+        for (unsigned spins = 0; !(has(w[0], s) && has(w[1], s) && has(w[2], s)); ++spins) {
           if (spins > kWaitSpins || *(volatile int*)&s_to) {
             s_to = 1;
             break;
           }
-          c = ld_relaxed_u64(p + 2);
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            if (!has(w[c], s)) w[c] = ld_relaxed_u64(p + (size_t)c * nv);
         }
-        L.z4[rows + h] = make_float4(__uint_as_float((unsigned)a), __uint_as_float((unsigned)b),
-                                     __uint_as_float((unsigned)c), 0.0f);
+        L.z4[rows + h] = make_float4(__uint_as_float((unsigned)w[0]), __uint_as_float((unsigned)w[1]),
+                                     __uint_as_float((unsigned)w[2]), 0.0f);
       }
     }
   };
@@ -401,8 +480,9 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
   const int my_c = D ? tid / rows : 0, my_item = D ? tid - my_c * rows : tid;
   const int my_i = row0 + my_item;
   const bool own = (D ? tid < 3 * rows : tid < rows) && my_i < nv;
-  T x[3] = {(T)0, (T)0, (T)0}, r[3] = {(T)0, (T)0, (T)0}, P[9];
-  unsigned long long* my_line = A.unit_words + (size_t)(u0 + warp) * RD_LINE;  // (of unit u0 + warp)
+  T x[3] = {(T)0, (T)0, (T)0}, r[3] = {(T)0, (T)0, (T)0}, P[9];  // (zero where there is no row: no branch
+#pragma unroll                                                   // splits a warp before its sums)
+  for (int c = 0; c < 9; ++c) P[c] = (T)0;
 
   // z = P r, r.z and r.r of the own rows, posted with stamp s
   auto precondition = [&](unsigned s) {
@@ -413,12 +493,9 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       if (tid < 3 * rows) lr[my_item] = r[0];
       __syncthreads();
       if (tid < 3 * rows) {
-        T z = (T)0;
-        if (own) {
-          const T r0 = L.rx[my_item], r1 = L.ry[my_item], rr2 = L.rz[my_item];
-          z = P[0] * r0 + P[1] * r1 + P[2] * rr2;
-          post_z(my_i, my_c, z, s);
-        }
+        const T r0 = L.rx[my_item], r1 = L.ry[my_item], rr2 = L.rz[my_item];
+        const T z = rd_dot(P[0], r0, P[1], r1, P[2], rr2);
+        if (own) rd_post(z_pair(my_c, my_i), s, z);
         lz[my_item] = z;
       }
       __syncthreads();
@@ -432,34 +509,34 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
           const T z0 = L.zx[item], z1 = L.zy[item], z2 = L.zz[item];
           v = rd_dot(r0, z0, r1, z1, rr2, z2);
         } else {
-          v = r0 * r0 + r1 * r1 + rr2 * rr2;
+          v = rd_dot(r0, r0, r1, r1, rr2, rr2);
         }
         v = warp_sum(v);
-        if (lane == 0) rd_post(A.unit_words + (size_t)(u0 + u) * RD_LINE + (w < units ? 4 : 6), s, v);
+        if (lane == 0) unit_sum(u, w < units ? 0 : 1, RD_RZ + (w < units ? 0 : 2), s, v);
       }
     } else {
       if (warp < rows / 32) {  // (warp-uniform)
-        double rz = 0.0, r2 = 0.0;
+        const T z0 = rd_dot(P[0], r[0], P[1], r[1], P[2], r[2]);
+        const T z1 = rd_dot(P[3], r[0], P[4], r[1], P[5], r[2]);
+        const T z2 = rd_dot(P[6], r[0], P[7], r[1], P[8], r[2]);
         if (own) {
-          const T z0 = P[0] * r[0] + P[1] * r[1] + P[2] * r[2];
-          const T z1 = P[3] * r[0] + P[4] * r[1] + P[5] * r[2];
-          const T z2 = P[6] * r[0] + P[7] * r[1] + P[8] * r[2];
-          unsigned long long* p = A.z_words + 4 * (size_t)my_i;
-          rd_st2(p, rd_word(s, __float_as_uint(z0)), rd_word(s, __float_as_uint(z1)));
-          st_relaxed_u64(p + 2, rd_word(s, __float_as_uint(z2)));
-          L.z4[tid] = make_float4(z0, z1, z2, 0.0f);
-          rz = (double)(r[0] * z0 + r[1] * z1 + r[2] * z2);
-          r2 = (double)(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-        } else {
-          L.z4[tid] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          unsigned long long* p = A.z_words + my_i;
+          st_relaxed_u64(p, rd_word(s, __float_as_uint(z0)));
+          st_relaxed_u64(p + nv, rd_word(s, __float_as_uint(z1)));
+          st_relaxed_u64(p + 2 * (size_t)nv, rd_word(s, __float_as_uint(z2)));
         }
-        rz = warp_sum(rz);
-        r2 = warp_sum(r2);
-        if (lane == 0) {
-          rd_post(my_line + 4, s, rz);
-          rd_post(my_line + 6, s, r2);
-        }
+        L.z4[tid] = make_float4(z0, z1, z2, 0.0f);
+        const double rz = (double)rd_dot(r[0], z0, r[1], z1, r[2], z2);
+        const double r2 = (double)rd_dot(r[0], r[0], r[1], r[1], r[2], r[2]);
+        // both trees in one warp: lanes 0-15 take the halves of r.z, lanes 16-31 those of r.r
+        // (warp_sum pairs lane l with l + 16 first, then both halves alike)
+        const double give = lane < 16 ? r2 : rz, keep = lane < 16 ? rz : r2;
+        double v = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0) unit_sum(warp, lane >> 4, RD_RZ + (lane >> 3), s, v);
       }
+      post_tiles(2, RD_RZ, s);
     }
   };
 
@@ -487,7 +564,7 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       }
     }
     const unsigned bad = __ballot_sync(0xffffffffu, !ok);
-    if (lane == 0 && warp < rows / 32) st_relaxed_u64(my_line + 8, rd_word(epoch, (unsigned)__popc(bad)));
+    if (lane == 0 && bad) atomicAdd(&s_bad[32 * warp / per], __popc(bad));
     for (int item = tid; item < n_items; item += RD_NT) {
       if constexpr (D)
         L.dx[item] = L.dy[item] = L.dz[item] = (T)0;
@@ -511,9 +588,11 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       }
     }
     precondition(epoch);
-    // the failed blocks of every unit (one thread each), then the start of the recurrences
-    for (int u = tid; u < nu; u += RD_NT) {
-      const unsigned long long* p = A.unit_words + (size_t)u * RD_LINE + 8;
+    __syncthreads();  // (the counts)
+    if (tid < p1 - p0) st_relaxed_u64(my_words + (size_t)tid * RD_LINE + RD_FAIL, rd_word(epoch, (unsigned)s_bad[tid]));
+    // the failed blocks of every post, then the start of the recurrences
+    for (int u = tid; u < n_posts; u += RD_NT) {
+      const unsigned long long* p = A.words + (size_t)u * RD_LINE + RD_FAIL;
       unsigned long long w = ld_relaxed_u64(p);
       for (unsigned spins = 0; !has(w, epoch); ++spins) {
         if (spins > kWaitSpins || *(volatile int*)&s_to) {
@@ -524,8 +603,10 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       }
       if ((unsigned)w) atomicAdd(&s_fail, (int)(unsigned)w);
     }
-    sums(epoch, 4, I2{}, I1{}, [&] { read_halo(epoch); },
-         [&](const double* v) { init_state(st, v[0], v[1], (double)s_fail); });
+    sums(epoch, RD_RZ, I2{}, I1{}, [&] { read_halo(epoch); }, [&](const double* v) {
+      init_state(st, v[0], v[1], (double)s_fail);
+      s_stop = (double)S.tol2 * st.rr0;
+    });
     if (gave_up()) return;
   }
 
@@ -561,7 +642,7 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
             const int cl = L.lcol[(j0 + j) * 32 + lane];
             const T* v = L.lval + (j0 + j) * 288 + 96 * c + lane;
             const T dj0 = L.dx[cl], dj1 = L.dy[cl], dj2 = L.dz[cl];
-            a += v[0] * dj0 + v[32] * dj1 + v[64] * dj2;
+            a += rd_dot(v[0], dj0, v[32], dj1, v[64], dj2);
           }
         a += __shfl_xor_sync(0xffffffffu, a, 16);
         if (h == 0) (c == 0 ? L.qx : c == 1 ? L.qy : L.qz)[item] = a;
@@ -586,9 +667,9 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
               for (int c = 0; c < 9; ++c) v[c] = __ldg(S.val + c * nnzb + kb + G * j + h);
             }
             const T dj0 = d.x, dj1 = d.y, dj2 = d.z;
-            ax += v[0] * dj0 + v[1] * dj1 + v[2] * dj2;
-            ay += v[3] * dj0 + v[4] * dj1 + v[5] * dj2;
-            az += v[6] * dj0 + v[7] * dj1 + v[8] * dj2;
+            ax += rd_dot(v[0], dj0, v[1], dj1, v[2], dj2);
+            ay += rd_dot(v[3], dj0, v[4], dj1, v[5], dj2);
+            az += rd_dot(v[6], dj0, v[7], dj1, v[8], dj2);
           }
 #pragma unroll
         for (int o = 16; o >= 8; o >>= 1) {
@@ -609,29 +690,30 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       const T ax = L.qx[tid], ay = L.qy[tid], az = L.qz[tid];
       if constexpr (D) {
         const T d0 = L.dx[tid], d1 = L.dy[tid], d2 = L.dz[tid];
-        T dq = rd_dot(d0, ax, d1, ay, d2, az);
+        T dq = row0 + tid < nv ? rd_dot(d0, ax, d1, ay, d2, az) : (T)0;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) dq += __shfl_xor_sync(0xffffffffu, dq, o);
-        if ((lane & 15) == 0) rd_post(my_line + (lane >> 3), epoch, dq);
+        if ((lane & 15) == 0) rd_post(my_words + (size_t)warp * RD_LINE + RD_DQ + (lane >> 3), epoch, dq);
       } else {
         const float4 di = L.d4[tid];
-        double dq = (double)(di.x * ax + di.y * ay + di.z * az);
+        double dq = row0 + tid < nv ? (double)rd_dot(di.x, ax, di.y, ay, di.z, az) : 0.0;
         dq = warp_sum(dq);
-        if (lane == 0) rd_post(my_line, epoch, dq);
+        if (lane == 0) unit_sum(warp, 0, RD_DQ, epoch, dq);
       }
     }
-    sums(epoch, 0, I1{}, std::integral_constant<int, DQ>{}, nothing, [&](const double* v) { after_dq(st, v[0]); });
+    if constexpr (!D) post_tiles(1, RD_DQ, epoch);
+    sums(epoch, RD_DQ, I1{}, std::integral_constant<int, DQ>{}, nothing, [&](const double* v) { rd_after_dq(st, v[0]); });
     if (gave_up()) return;
     if (st.done) break;
 
     // ---------------- x += alpha d, r -= alpha q, z = P r
     ++epoch;
-    if (own) {
-      const T alpha = (T)st.alpha;
+    const T alpha = own ? (T)st.alpha : (T)0;
+    T d_own = (T)0;
+    if (tid < (D ? 3 : 1) * rows) {  // (the rows past the scene's last one stay zero)
       if constexpr (D) {
-        const T d = (my_c == 0 ? L.dx : my_c == 1 ? L.dy : L.dz)[my_item];
+        d_own = (my_c == 0 ? L.dx : my_c == 1 ? L.dy : L.dz)[my_item];
         const T q = (my_c == 0 ? L.qx : my_c == 1 ? L.qy : L.qz)[my_item];
-        x[0] += alpha * d;
         r[0] = r[0] - alpha * q;
       } else {
         const float4 di = L.d4[tid];
@@ -644,8 +726,9 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       }
     }
     precondition(epoch);
-    sums(epoch, 4, I2{}, I1{}, [&] { read_halo(epoch); },
-         [&](const double* v) { after_rz(st, v[0], v[1], S.tol2, S.max_iter); });
+    if (D && tid < 3 * rows) x[0] += alpha * d_own;  // (off the chain to the sums; idle warps would hold the FP64 pipe)
+    sums(epoch, RD_RZ, I2{}, I1{}, [&] { read_halo(epoch); },
+         [&](const double* v) { rd_after_rz(st, v[0], v[1], s_stop, S.max_iter); });
     if (gave_up()) return;
   }
 
@@ -668,8 +751,8 @@ __global__ void k_rd_clear(RdLaunch<T> A, int nv) {
   const int n_thr = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
   if (t0 == 0) *A.bar = GridBar{};
   const ulonglong2 zero = make_ulonglong2(0, 0);
-  ulonglong2* w = reinterpret_cast<ulonglong2*>(A.unit_words);
-  for (int k = t0; k < A.n_units * (RD_LINE / 2); k += n_thr) w[k] = zero;
+  ulonglong2* w = reinterpret_cast<ulonglong2*>(A.words);
+  for (int k = t0; k < A.plan.n_posts * (RD_LINE / 2); k += n_thr) w[k] = zero;
   if constexpr (sizeof(T) == 8) {
     ulonglong2 *z = reinterpret_cast<ulonglong2*>(A.scene->z), *q = reinterpret_cast<ulonglong2*>(A.scene->q);
     for (int k = t0; k < 2 * nv; k += n_thr) z[k] = q[k] = zero;
@@ -679,10 +762,9 @@ __global__ void k_rd_clear(RdLaunch<T> A, int nv) {
   }
 }
 
-// Block slots and halo rows of the largest CTA when n rows go to `grid` CTAs in 32-row units, for
-// a device-resident pattern; a CTA with more than HS / 2 halo rows reports more than any plan
+// Block slots and halo rows of the largest CTA of a plan, for a device-resident pattern; a CTA with more than HS / 2 halo rows reports more than any plan
 // takes.  Skips a pattern that `error` says is malformed.
-__global__ void __launch_bounds__(RD_NT) k_rd_plan(const int* row_ptr, const int* col, int n, int n_units, int g_lanes,
+__global__ void __launch_bounds__(RD_NT) k_rd_plan(const int* row_ptr, const int* col, RdPlan plan, int g_lanes,
                                                    const int* error, int* most_slots, int* most_halo) {
   constexpr int HS = 8192;
   __shared__ int key[HS];
@@ -692,9 +774,9 @@ __global__ void __launch_bounds__(RD_NT) k_rd_plan(const int* row_ptr, const int
   for (int h = tid; h < HS; h += RD_NT) key[h] = -1;
   if (tid == 0) s_nh = s_steps = 0;
   __syncthreads();
-  const int row0 = 32 * rd_unit((int)blockIdx.x, n_units, (int)gridDim.x);
-  const int rend = 32 * rd_unit((int)blockIdx.x + 1, n_units, (int)gridDim.x);
-  const int r1 = min(n, rend);
+  const int row0 = plan.post_rows * rd_post0((int)blockIdx.x, plan.n_posts, plan.grid);
+  const int rend = plan.post_rows * rd_post0((int)blockIdx.x + 1, plan.n_posts, plan.grid);
+  const int r1 = min(plan.nv, rend);
   for (int g = row0 + gr * tid; g < r1; g += gr * RD_NT) {
     int m = 0;
     for (int r = g; r < min(r1, g + gr); ++r) m = max(m, row_ptr[r + 1] - row_ptr[r]);
@@ -719,9 +801,9 @@ __global__ void __launch_bounds__(RD_NT) k_rd_plan(const int* row_ptr, const int
   }
 }
 
-cudaError_t launch_rd_plan(const int* row_ptr, const int* col, int n, int grid, const int* error, int* most_slots,
+cudaError_t launch_rd_plan(const int* row_ptr, const int* col, const RdPlan& plan, const int* error, int* most_slots,
                            int* most_halo, cudaStream_t st) {
-  k_rd_plan<<<grid, RD_NT, 0, st>>>(row_ptr, col, n, (n + 31) / 32, RdCfg<float>::G, error, most_slots, most_halo);
+  k_rd_plan<<<plan.grid, RD_NT, 0, st>>>(row_ptr, col, plan, RdCfg<float>::G, error, most_slots, most_halo);
   return cudaGetLastError();
 }
 
@@ -748,10 +830,11 @@ template int pcg_rd_max_grid<float>(int, size_t, bool);
 
 template <typename T>
 cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st) {
-  const int nv = L.nv;
-  if (!L.scene || !L.bar || !L.unit_words || nv <= 0 || L.n_units != (nv + 31) / 32 || L.grid < 1 ||
-      L.grid > L.n_units || (L.n_units + L.grid - 1) / L.grid * 32 > (sizeof(T) == 8 ? RD_NT / 96 * 32 : RD_NT) ||
-      (sizeof(T) == 4 && !L.z_words))
+  const RdPlan& p = L.plan;
+  const int nv = p.nv;
+  if (!L.scene || !L.bar || !L.words || nv <= 0 || (p.post_rows != 32 && (p.post_rows != PCG_TILE || sizeof(T) == 8)) ||
+      p.n_posts != (nv + p.post_rows - 1) / p.post_rows || p.grid < 1 || p.grid > p.n_posts ||
+      p.rows() > (sizeof(T) == 8 ? RD_ROWS_MAX_F64 : RD_NT) || (sizeof(T) == 4 && !L.z_words))
     return cudaErrorInvalidValue;
   k_rd_clear<T><<<std::min(152, 1 + nv / 128), 256, 0, st>>>(L, nv);
   cudaError_t e = cudaGetLastError();
@@ -761,7 +844,7 @@ cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   RdLaunch<T> a = L;
   void* args[] = {(void*)&a};
-  return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(RD_NT), args, L.smem_bytes, st);
+  return cudaLaunchCooperativeKernel(k, dim3(p.grid), dim3(RD_NT), args, L.smem_bytes, st);
 }
 template cudaError_t launch_pcg_rd<double>(const RdLaunch<double>&, cudaStream_t);
 template cudaError_t launch_pcg_rd<float>(const RdLaunch<float>&, cudaStream_t);

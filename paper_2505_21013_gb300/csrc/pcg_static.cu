@@ -50,6 +50,10 @@ namespace {
 constexpr int kMaxRows = PPN_PCG_STATIC_MAX_ROWS;
 constexpr int kMaxTiles = (kMaxRows + PCG_TILE - 1) / PCG_TILE;
 constexpr int kMaxDevices = 64;
+// rows up to which the unit kernel posts 32-row units (a CTA each up to the SM count): more CTAs for
+// the rows (2000 rows 7.5 -> 6.6 us per CG iteration against tiles); beyond, whole tiles: fewer words
+// for every CTA to poll (32000 rows 13.2 -> 10.1)
+constexpr int kUnitPostRows = 4864;
 constexpr int kErrPattern = 4;  // Ctl::error bit: the caller's BSR pattern is malformed
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -234,8 +238,8 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   k_static_prep<<<nb, 256, 0, st>>>(row_ptr, col, n_rows, nnzb, A.diag, A.tiles, n_tiles, A.ctl);
   PPN_STATIC_CU(cudaGetLastError());
   // the unit kernel's shared-memory needs for this pattern (two counters of the control block)
-  const int n_units = (n_rows + 31) / 32, rd_grid = std::min(n_units, D.n_sm);
-  PPN_STATIC_CU(launch_rd_plan(row_ptr, col, n_rows, rd_grid, &A.ctl->error, &A.ctl->n_new, &A.ctl->n_touched, st));
+  const RdPlan plan = rd_plan(n_rows, n_rows <= kUnitPostRows ? 32 : PCG_TILE, D.n_sm);
+  PPN_STATIC_CU(launch_rd_plan(row_ptr, col, plan, &A.ctl->error, &A.ctl->n_new, &A.ctl->n_touched, st));
   Ctl c{};
   PPN_STATIC_CU(cudaMemcpyAsync(&c, A.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   PPN_STATIC_CU(cudaStreamSynchronize(st));
@@ -263,15 +267,14 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   s.pcg_max_iter = max_iter > 0 ? max_iter : std::max(1000, 3 * n_rows);
   s.active = 1;
   // The unit kernel (pcg_rd.cu; same bits) where its rows' vectors fit in shared memory, with the blocks
-  // resident too when they fit: 32000 rows 24.9 -> 13.2 us per CG iteration, 546 rows 19.5 -> 6.9; a
+  // resident too when they fit: 32000 rows 24.9 -> 9.4 us per CG iteration, 546 rows 19.5 -> 5.5, 65536 rows 33 -> 15.5; a
   // pattern with too many halo rows per CTA keeps the global-memory kernel.
   RdLaunch<float> R{};
-  const int rd_rows = 32 * ((n_units + rd_grid - 1) / rd_grid);
-  bool units = rd_rows <= 512 && c.n_touched <= 4096;
+  bool units = plan.rows() <= 512 && c.n_touched <= 4096;
   for (int resident = 1; units && resident >= 0; --resident) {
-    R.smem_bytes = pcg_rd_smem_bytes<float>(n_units, rd_rows, c.n_new, resident != 0, c.n_touched);
+    R.smem_bytes = pcg_rd_smem_bytes<float>(plan, c.n_new, resident != 0, c.n_touched);
     R.resident = resident;
-    if (R.smem_bytes <= (size_t)224 * 1024 && pcg_rd_max_grid<float>(dev, R.smem_bytes, resident != 0) >= rd_grid) break;
+    if (R.smem_bytes <= (size_t)224 * 1024 && pcg_rd_max_grid<float>(dev, R.smem_bytes, resident != 0) >= plan.grid) break;
     if (resident == 0) units = false;
   }
   const bool copy_b = !units || (reinterpret_cast<uintptr_t>(b) & 15u);
@@ -290,14 +293,12 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   L.use_b_from_g = 0;
   if (units) {
     R.scene = A.desc;
-    R.nv = n_rows;
-    R.n_units = n_units;
-    R.grid = rd_grid;
+    R.plan = plan;
     R.slots = c.n_new;
     R.halo_cap = c.n_touched;
     R.bar = A.bar;
-    R.z_words = reinterpret_cast<unsigned long long*>(A.z);      // 32 bytes per row: z and the q after it
-    R.unit_words = reinterpret_cast<unsigned long long*>(A.d0);  // 128 bytes per 32 rows
+    R.z_words = reinterpret_cast<unsigned long long*>(A.z);      // 24 bytes per row: z and the q after it
+    R.words = reinterpret_cast<unsigned long long*>(A.d0);    // 256 bytes per 32 or 128 rows
     PPN_STATIC_CU(launch_pcg_rd<float>(R, st));
   } else {
     PPN_STATIC_CU(launch_pcg<float>(A.desc, L, st));
