@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "pcg_common.cuh"
+#include "pcg_units.cuh"
 
 namespace ppn {
 
@@ -120,26 +121,6 @@ __host__ __device__ inline size_t rd_carve(char* base, int n_posts, int n_tiles,
   s.qz = (T*)take(sizeof(T) * rows);
   if (out) *out = s;
   return off;
-}
-
-// the posts [rd_post0(b), rd_post0(b + 1)) of CTA b
-__host__ __device__ inline int rd_post0(int b, int n_posts, int grid) { return (int)(((long long)b * n_posts) / grid); }
-
-// smallest power of two >= 2 n (at least 64)
-__host__ __device__ inline int rd_hash_size(int n) {
-  int h = 64;
-  while (h < 2 * n) h *= 2;
-  return h;
-}
-__device__ __forceinline__ unsigned rd_hash(int j) { return (unsigned)j * 2654435761u >> 8; }
-// inserts j into the table of hs keys (-1: free); false when it is full
-__device__ __forceinline__ bool rd_insert(int* key, int hs, int j) {
-  unsigned h = rd_hash(j) & (unsigned)(hs - 1);
-  for (int n = 0; n < hs; ++n, h = (h + 1) & (unsigned)(hs - 1)) {
-    const int k = atomicCAS(&key[h], -1, j);
-    if (k == -1 || k == j) return true;
-  }
-  return false;
 }
 
 // ---- stamped words: 32 bits of a value and the 32-bit stamp
@@ -296,13 +277,7 @@ __global__ void __launch_bounds__(RD_NT, 1) k_pcg_rd(RdLaunch<T> A) {
       }
     }
     __syncthreads();
-    for (int h = tid; h < hs; h += RD_NT)
-      if (L.hkey[h] >= 0) {
-        const int n = atomicAdd(&s_nh, 1);
-        L.hidx[h] = n;
-        if (n < A.halo_cap) L.href[n] = L.hkey[h];
-      }
-    __syncthreads();
+    rd_rank<RD_NT>(L.hkey, L.hidx, L.href, hs, A.halo_cap, &s_nh);
     if (s_nh > A.halo_cap) s_to = 5;
   }
   __syncthreads();

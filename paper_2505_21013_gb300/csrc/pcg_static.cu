@@ -267,7 +267,7 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   s.pcg_max_iter = max_iter > 0 ? max_iter : std::max(1000, 3 * n_rows);
   s.active = 1;
   // The unit kernel (pcg_rd.cu; same bits) where its rows' vectors fit in shared memory, with the blocks
-  // resident too when they fit: 32000 rows 24.9 -> 9.4 us per CG iteration, 546 rows 19.5 -> 5.5, 65536 rows 33 -> 15.5; a
+  // resident too when they fit: 32000 rows 24.9 -> 8.3 us per CG iteration, 546 rows 19.5 -> 5.5, 50400 rows 31 -> 12.7; a
   // pattern with too many halo rows per CTA keeps the global-memory kernel.
   RdLaunch<float> R{};
   bool units = plan.rows() <= 512 && c.n_touched <= 4096;
