@@ -18,7 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libppn.so")
-SOURCES = ["kernels.cu", "pcg.cu", "pcg_smem.cu", "pcg_sr.cu", "pcg_rd.cu", "pcg_static.cu", "scene.cu", "server.cu"]
+SOURCES = ["kernels.cu", "pcg.cu", "pcg_smem.cu", "pcg_sr.cu", "pcg_su.cu", "pcg_rd.cu", "pcg_static.cu", "scene.cu", "server.cu"]
 HEADERS = ["common.cuh", "tetmath.cuh", "eigclamp.cuh", "contact.cuh", "kernels.h", "scene.h", "driver.h", "pcg_common.cuh",
            "pcg_sr.cuh", "pcg_units.cuh", "halo.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

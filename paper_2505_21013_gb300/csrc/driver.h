@@ -437,6 +437,19 @@ struct Driver {
       cudaError_t err = cudaSuccess;
       timed(FAM_PCG, bytes, [&] {
         if constexpr (sizeof(T) == sizeof(float)) {
+          if (G.rd_smem_bytes) {
+            SuLaunch U{};
+            U.scene = reinterpret_cast<const SceneDev<float>*>(G.d_desc) + sl[0];
+            U.plan = G.rd_plan;
+            U.slots = G.rd_slots;
+            U.halo_cap = G.rd_halo;
+            U.b_from_g = b_from_g;
+            U.bar = G.d_bar;
+            U.words = reinterpret_cast<float4*>(G.h_desc[sl[0]].pword);
+            U.smem_bytes = G.rd_smem_bytes;
+            err = launch_pcg_su(U, G.st);
+            return;
+          }
           if (G.pcg_sr) {
             err = launch_pcg_sr(reinterpret_cast<const SceneDev<float>*>(G.d_desc), L, G.st);
             return;
@@ -650,6 +663,11 @@ struct Driver {
         fits[mode] = bytes[mode] <= (size_t)212 * 1024 && pcg_sr_max_grid(dev, bytes[mode], mode) >= grid;
         if (fits[mode] && (mode == SR_RES || f_str || f_gl)) break;
       }
+      if (first == SR_RES && sl.size() == 1 && !std::getenv("PPN_PCG_NO_HALO") && plan_units(*G.S[sl[0]], dev, n_sm)) {
+        G.pcg_sr = true;
+        G.pcg_sr_mode = SR_HALO;
+        return;
+      }
       if (first == SR_RES && fits[SR_RES] && sl.size() <= (size_t)HALO_MAX_SCENES && max_items <= SR_HALO_MAX_ROWS &&
           !std::getenv("PPN_PCG_NO_HALO")) {
         std::vector<int> tab;
@@ -713,28 +731,22 @@ struct Driver {
     G.pcg_smem_blocks = max_blocks;
     G.pcg_smem_grid = grid;
     if constexpr (sizeof(T) == sizeof(double))
-      if (sl.size() == 1) plan_units(*G.S[sl[0]], dev, n_sm);
+      if (sl.size() == 1) (void)plan_units(*G.S[sl[0]], dev, n_sm);
   }
 
-  // FP64, one scene: the unit kernel (pcg_rd.cu) in place of the standard resident one (same
-  // bits) when its layout fits: rows in 32-row units over all SMs, where 128-row tiles leave
-  // most SMs idle and 5.4 us of FP64 work per SpMV on the others.  125 rows: 22 -> 8.9 us per CG
-  // iteration, 6480 rows: 23.2 -> 10.6.  PPN_PCG_NO_UNITS=1 keeps the standard kernel (tests).
-  void plan_units(const SceneImpl<T>& s, int dev, int n_sm) {
-    if (std::getenv("PPN_PCG_NO_UNITS") || s.n_ptiles > 512) return;
-    const RdPlan plan = rd_plan(s.nv, 32, n_sm);
-    if (plan.rows() > RD_ROWS_MAX_F64) return;
-    const int nu = plan.n_posts, grid = plan.grid;
-    int slots = 0, halo = 0;
+  // Most block slots (per group of gr rows, 32 per step of ceil(longest row / lanes)) and halo rows of
+  // one CTA of a plan.
+  static void unit_needs(const SceneImpl<T>& s, const RdPlan& plan, int gr, int lanes, int& slots, int& halo) {
+    slots = halo = 0;
     std::vector<int> mark(s.nv, -1);
-    for (int b = 0; b < grid; ++b) {
-      const int r0 = 32 * (int)(((long long)b * nu) / grid), re = 32 * (int)(((long long)(b + 1) * nu) / grid);
-      const int r1 = std::min(s.nv, re);
+    for (int b = 0; b < plan.grid; ++b) {
+      const int r0 = plan.post_rows * (int)(((long long)b * plan.n_posts) / plan.grid);
+      const int re = plan.post_rows * (int)(((long long)(b + 1) * plan.n_posts) / plan.grid), r1 = std::min(s.nv, re);
       int n = 0, h = 0;
-      for (int g = r0; g < r1; g += 16) {
+      for (int g = r0; g < r1; g += gr) {
         int m = 0;
-        for (int r = g; r < std::min(r1, g + 16); ++r) m = std::max(m, (int)(s.h_row_ptr[r + 1] - s.h_row_ptr[r]));
-        n += 32 * ((m + 1) / 2);
+        for (int r = g; r < std::min(r1, g + gr); ++r) m = std::max(m, (int)(s.h_row_ptr[r + 1] - s.h_row_ptr[r]));
+        n += 32 * ((m + lanes - 1) / lanes);
       }
       for (int64_t k = s.h_row_ptr[r0]; k < s.h_row_ptr[r1]; ++k) {
         const int j = s.h_col[k];
@@ -746,12 +758,34 @@ struct Driver {
       slots = std::max(slots, n);
       halo = std::max(halo, h);
     }
-    const size_t bytes = pcg_rd_smem_bytes<double>(plan, slots, true, halo);
-    if (bytes > (size_t)224 * 1024 || pcg_rd_max_grid<double>(dev, bytes, true) < grid) return;
+  }
+
+  // One scene: the unit kernels in place of the standard resident one (FP64: pcg_rd.cu) or of the halo
+  // layout (FP32: pcg_su.cu), with the same bits, when their layout fits.
+  // FP64: rows in 32-row units over all SMs, where 128-row tiles leave most SMs idle and 5.4 us of FP64
+  // work per SpMV on the others.  125 rows: 22 -> 8.9 us per CG iteration, 6480 rows: 23.2 -> 10.6.
+  // FP32: scenes of at most one 128-row tile per SM; 756 rows 3.11 -> 2.20 us, 15840 rows 3.39 -> 2.54.
+  // PPN_PCG_NO_UNITS=1 keeps the other kernels (tests).
+  bool plan_units(const SceneImpl<T>& s, int dev, int n_sm) {
+    constexpr bool D = sizeof(T) == sizeof(double);
+    if (std::getenv("PPN_PCG_NO_UNITS") || s.n_ptiles > 512) return false;
+    int pr = 32;  // FP32: a CTA per post
+    while (!D && pr < PCG_TILE && (s.nv + pr - 1) / pr > n_sm) pr *= 2;
+    const RdPlan plan = rd_plan(s.nv, pr, n_sm);
+    if (D ? plan.rows() > RD_ROWS_MAX_F64 : plan.grid != plan.n_posts) return false;
+    int slots, halo;
+    unit_needs(s, plan, 16, 2, slots, halo);
+    const int hpt = D ? 1 : pcg_su_hpt(plan, halo);
+    if (!hpt) return false;
+    const size_t bytes = D ? pcg_rd_smem_bytes<double>(plan, slots, true, halo) : pcg_su_smem_bytes(plan, slots, halo);
+    if (bytes > (size_t)224 * 1024 ||
+        (D ? pcg_rd_max_grid<double>(dev, bytes, true) : pcg_su_max_grid(dev, bytes, plan.post_rows, hpt)) < plan.grid)
+      return false;
     G.rd_smem_bytes = bytes;
     G.rd_slots = slots;
     G.rd_halo = halo;
     G.rd_plan = plan;
+    return true;
   }
 
   // Start a time step for the flagged slots (their H[i].mode and H[i].tol set):

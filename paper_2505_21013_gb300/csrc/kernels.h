@@ -141,7 +141,7 @@ cudaError_t launch_pcg_smem(const SceneDev<T>* scenes, const PcgLaunch& L, cudaS
 // float: that of launch_pcg<float> with four lanes per row.
 struct RdPlan {
   int nv;         // rows
-  int post_rows;  // rows of one post of the exchanges: 32 (a unit) or 128 (a tile; float only)
+  int post_rows;  // rows of one post of the exchanges: a unit of 32, or 64 or a tile of 128 (float only)
   int n_posts;
   int grid;       // CTAs (co-resident); CTA b owns the posts [b n_posts / grid, (b + 1) n_posts / grid)
   __host__ __device__ int rows() const { return (n_posts + grid - 1) / grid * post_rows; }  // of the largest CTA
@@ -171,6 +171,22 @@ template <typename T> cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream
 // results must be zero before; nothing is done when *error is set
 cudaError_t launch_rd_plan(const int* row_ptr, const int* col, const RdPlan& plan, const int* error, int* most_slots,
                            int* most_halo, cudaStream_t st);
+
+// Single-reduction recurrences for one scene in 32-row units (pcg_su.cu): the arithmetic of
+// launch_pcg_sr.
+struct SuLaunch {
+  const SceneDev<float>* scene;  // device
+  RdPlan plan;                   // a CTA per post of 32, 64 or 128 rows
+  int slots, halo_cap;           // most block slots (as launch_pcg_sr's) and halo rows of one CTA
+  int b_from_g;
+  GridBar* bar;
+  float4* words;                 // 16 words of 16 bytes per post
+  size_t smem_bytes;
+};
+size_t pcg_su_smem_bytes(const RdPlan& p, int slots, int halo);
+int pcg_su_hpt(const RdPlan& p, int halo);  // halo rows per thread; 0: does not fit
+int pcg_su_max_grid(int device, size_t smem, int rows, int hpt);
+cudaError_t launch_pcg_su(const SuLaunch& L, cudaStream_t st);
 
 // Occupancy-limited cooperative grid size for the chosen row group width.
 int pcg_max_grid(int group, int device);

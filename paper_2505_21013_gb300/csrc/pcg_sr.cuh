@@ -90,5 +90,40 @@ __device__ __forceinline__ void sr_step(SState<float>& s, float gam, float del, 
   s.rz = gam;
 }
 
+// sr_step on the common path (another iteration follows) with its divisions issued at once, not
+// behind one exit test after the other; the tests decide as sr_step does
+__device__ __forceinline__ void sr_step_fast(SState<float>& s, float gam, float del, float rho, float fail, int it,
+                                             float tol2, int max_iter) {
+  const float rz = s.rz, alpha = s.alpha, rr0 = s.rr0;
+  const int iters = s.iters;
+  const float beta = gam / rz, d = del - beta * gam / alpha, a = gam / d;
+  if (it > 0 && rho == rho && gam == gam && del == del && !(rho <= tol2 * rr0) && iters < max_iter && d > 0.0f) {
+    s.rr = rho;
+    s.dq = d;
+    s.beta = beta;
+    s.alpha = a;
+    s.rz = gam;
+  } else {
+    sr_step(s, gam, del, rho, fail, it, tol2, max_iter);
+  }
+}
+
+// ---- 16-byte words: three FP32 values and the 32-bit stamp, read and written as one 128-bit
+// scalar (single-copy atomic): a word with the expected stamp carries its values
+__device__ __forceinline__ void st_word4(float4* p, float x, float y, float z, unsigned s) {
+  asm volatile(
+      "{\n\t.reg .b128 w;\n\tmov.b128 w, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], w;\n\t}" ::"l"(p),
+      "l"(((unsigned long long)__float_as_uint(y) << 32) | __float_as_uint(x)),
+      "l"(((unsigned long long)s << 32) | __float_as_uint(z))
+      : "memory");
+}
+__device__ __forceinline__ void ld_word4(const float4* p, unsigned long long& a, unsigned long long& b) {
+  asm volatile("{\n\t.reg .b128 w;\n\tld.relaxed.gpu.global.b128 w, [%2];\n\tmov.b128 {%0, %1}, w;\n\t}"
+               : "=l"(a), "=l"(b)
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ unsigned word4_stamp(unsigned long long b) { return (unsigned)(b >> 32); }
+
 }  // namespace pcgdev
 }  // namespace ppn

@@ -1,7 +1,7 @@
-"""The unit kernel of the linear solver (32-row units, direction replicated on the halo)
-against the kernels whose arithmetic it keeps: FP64 scenes against the standard resident
-kernel, the allocation-free solve against the global-memory kernel.  Same sums in the
-same order, so the iterates are equal bit for bit at every size: fewer rows than a unit,
+"""The unit kernels of the linear solver (32-row units, the halo replicated) against the
+kernels whose arithmetic they keep: FP64 scenes against the standard resident kernel,
+mixed scenes of at most a tile per SM against the halo layout, the allocation-free solve
+against the global-memory kernel.  Same sums in the same order, so the iterates are equal bit for bit at every size: fewer rows than a unit,
 exact and ragged units and tiles, one and several units per CTA, more tiles than lanes."""
 
 import numpy as np
@@ -56,6 +56,47 @@ def test_fp64_scenes(dims, indefinite, monkeypatch):
     sc.close()
     assert info == info0 and (info["ind"] or not indefinite)
     assert np.array_equal(x, x0), (np.abs(x - x0).max(), info)
+
+
+# 32, 64 and 128 rows per CTA (19456 rows: the most, a tile on each SM), and the size past it
+@pytest.mark.parametrize("indefinite", [False, True])
+@pytest.mark.parametrize("dims", DIMS + [(16, 19, 32), (16, 16, 76), (16, 16, 77)])
+def test_mixed_scenes(dims, indefinite, monkeypatch):
+    spec = twisting_beam_scene(*dims, h=0.1, seed=3)
+    _, _, _, K, b = springs(dims, 7, indefinite)
+    out = []
+    for env in (None, "PPN_PCG_NO_UNITS", "PPN_PCG_NO_HALO"):
+        if env:
+            monkeypatch.setenv(env, "1")
+        sc = P.Scene.from_spec(spec, precision=P.PREC_MIXED)
+        out.append(sc.probe_pcg(K, b, rel_tol=1e-5))
+        if env is None:  # the same scene again: words of the solve before it do not count
+            again = sc.probe_pcg(K, b, rel_tol=1e-5)
+            assert again[1] == out[0][1] and np.array_equal(again[0], out[0][0])
+        sc.close()
+    for x, info in out[1:]:
+        assert info == out[0][1] and (info["ind"] or not indefinite)
+        assert np.array_equal(x, out[0][0]), np.abs(x - out[0][0]).max()
+
+
+def test_mixed_scene_exits(monkeypatch):
+    # a failing diagonal block and a zero right-hand side end the solve alike
+    dims = (5, 6, 9)
+    spec = twisting_beam_scene(*dims, h=0.1, seed=3)
+    _, rp, col, K, b = springs(dims, 8)
+    bad = K.copy()
+    k = rp[77] + np.nonzero(col[rp[77]:rp[78]] == 77)[0][0]
+    bad[k] = np.diag([-1.0, 2.0, 3.0])
+    runs = []
+    for env in (None, "PPN_PCG_NO_UNITS"):
+        if env:
+            monkeypatch.setenv(env, "1")
+        sc = P.Scene.from_spec(spec, precision=P.PREC_MIXED)
+        runs.append((sc.probe_pcg(bad, b)[1], sc.probe_pcg(K, 0 * b)[1], sc.probe_pcg(K, b, max_iter=7)))
+        sc.close()
+    assert runs[0][:2] == runs[1][:2] and runs[0][0]["precond_fail"] and runs[0][1]["iters"] == 0
+    assert runs[0][2][1] == runs[1][2][1] and runs[0][2][1]["hit_max"]
+    assert np.array_equal(runs[0][2][0], runs[1][2][0])
 
 
 @pytest.mark.parametrize("dims", DIMS + [(20, 20, 80), (27, 30, 70), (32, 32, 64)])
