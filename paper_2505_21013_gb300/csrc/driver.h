@@ -505,11 +505,11 @@ struct Driver {
       slots = std::max(slots, n);
     }
     const int rows = (s.n_ptiles + size - 1) / size * PCG_TILE;
-    if (pcg_sr_smem_bytes(rows, slots, 0, SR_HALO) > (size_t)227 * 1024) return false;
+    if (pcg_sr_smem_bytes(rows, slots, 0, s.n_ptiles, SR_HALO) > (size_t)227 * 1024) return false;
     std::vector<int> tab;
     const int nh = build_halo_tables({{s.nv, s.h_row_ptr.data(), s.h_col.data()}}, size, tab);
     if (nh < 0) return false;
-    const size_t smem = pcg_sr_smem_bytes(rows, slots, nh, SR_HALO);
+    const size_t smem = pcg_sr_smem_bytes(rows, slots, nh, s.n_ptiles, SR_HALO);
     // (leaves room for the kernel's static shared memory)
     if (smem > (size_t)220 * 1024) return false;
     t.d_tab = (int*)dev_alloc(s.dalloc, sizeof(int) * tab.size());
@@ -659,7 +659,7 @@ struct Driver {
       bool fits[3] = {false, false, false};
       size_t bytes[3];
       for (int mode = first; mode <= SR_GLOBAL; ++mode) {
-        bytes[mode] = pcg_sr_smem_bytes(max_items, mode == SR_RES ? max_slots : 0, 0, mode);
+        bytes[mode] = pcg_sr_smem_bytes(max_items, mode == SR_RES ? max_slots : 0, 0, 0, mode);
         fits[mode] = bytes[mode] <= (size_t)212 * 1024 && pcg_sr_max_grid(dev, bytes[mode], mode) >= grid;
         if (fits[mode] && (mode == SR_RES || f_str || f_gl)) break;
       }
@@ -668,11 +668,11 @@ struct Driver {
         G.pcg_sr_mode = SR_HALO;
         return;
       }
-      if (first == SR_RES && fits[SR_RES] && sl.size() <= (size_t)HALO_MAX_SCENES && max_items <= SR_HALO_MAX_ROWS &&
+      if (first == SR_RES && fits[SR_RES] && sl.size() == 1 && max_items <= SR_HALO_MAX_ROWS &&
           !std::getenv("PPN_PCG_NO_HALO")) {
         std::vector<int> tab;
         const int nh = build_halo(sl, grid, tab);
-        const size_t hb = nh < 0 ? 0 : pcg_sr_smem_bytes(max_items, max_slots, nh, SR_HALO);
+        const size_t hb = nh < 0 ? 0 : pcg_sr_smem_bytes(max_items, max_slots, nh, n_tiles, SR_HALO);
         if (nh >= 0 && hb <= (size_t)227 * 1024 && pcg_sr_max_grid(dev, hb, SR_HALO) >= grid) {
           if (tab.size() > G.cap_halo) {
             if (G.d_halo) {  // (cudaFree waits for launches that may still read it)

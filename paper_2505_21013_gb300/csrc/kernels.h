@@ -122,12 +122,12 @@ int pcg_smem_max_grid(int group, int device, size_t smem, int fsize);
 // shared memory (SR_RES); vectors in shared memory, blocks streamed (SR_STREAM);
 // both in global memory (SR_GLOBAL); as SR_RES plus a replicated halo, which
 // removes the neighbour exchange (SR_HALO).  Shared memory for ni rows / nb
-// blocks / nh halo rows, co-resident grid, launch.
+// blocks / nh halo rows / n_tiles tiles of the launch, co-resident grid, launch.
 constexpr int SR_RES = 0, SR_STREAM = 1, SR_GLOBAL = 2, SR_HALO = 3;
 // SR_HALO keeps each row's CG state in the registers of one thread: a CTA holds at
 // most one SpMV pass of rows (512 threads, two lanes per row)
 constexpr int SR_HALO_MAX_ROWS = 256;
-size_t pcg_sr_smem_bytes(int ni, int nb, int nh, int mode);
+size_t pcg_sr_smem_bytes(int ni, int nb, int nh, int n_tiles, int mode);
 int pcg_sr_max_grid(int device, size_t smem, int mode);
 cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cudaStream_t st);
 // one warp waits (at most `limit` polling rounds) for n stamped words to reach `stamp`; *out = 1 if it ran out

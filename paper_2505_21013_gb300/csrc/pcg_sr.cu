@@ -80,11 +80,14 @@ __device__ __forceinline__ int spmv_lane(int tid) { return (tid & 31) / (32 / SP
 // lane that multiplies it, so that every shared-memory load of the SpMV (a column, one of
 // a block's nine values) reads 32 consecutive words, free of bank conflicts.  A group
 // has ceil(longest row / 2) steps; the slots past a shorter row's end stay unused.  Slot
-// q = 32 (lgb[g] + j) + lane; value c of the block in slot q is at lval[288 (q / 32) + 32 c + q % 32].
+// q = 32 (lgb[g] + j) + lane; a step's 288 floats are 32 x 16 bytes (values 0..3), 32 x 16 bytes (values
+// 4..7) and 32 x 4 bytes (value 8).
 __device__ __forceinline__ int blk_slot(const int* lgb, int item, int k) {
   return (lgb[item >> 4] + (k >> 1)) * 32 + 16 * (k & 1) + (item & 15);
 }
-__device__ __forceinline__ int slot_val(int q, int c) { return (q >> 5) * 288 + 32 * c + (q & 31); }
+__device__ __forceinline__ int slot_val(int q, int c) {
+  return (q >> 5) * 288 + (c < 8 ? 128 * (c >> 2) + 4 * (q & 31) + (c & 3) : 256 + (q & 31));
+}
 
 struct SrLayout {
   float* lws;    // [(ni / PCG_TILE + 1) * 16 * NQ] partial sums per 16-row group (8 per tile)
@@ -99,12 +102,13 @@ struct SrLayout {
   float4* lu4;   // SR_HALO: [ni + nh] u of the own rows, then of the halo rows (w while it arrives)
   float *hr, *hs, *hP;  // SR_HALO: [nh * 3], [nh * 3], [nh * 6] r, s and inverse of the halo rows
   int* href;     // SR_HALO: [nh] halo rows (slot << HALO_ROW_BITS | row)
+  float* ltw;    // SR_HALO: [3][tiles of the scene] sums of the iteration's tile words
 };
 
 __host__ __device__ inline size_t up16(size_t b) { return (b + 15) & ~size_t(15); }
 
 // the layout's pieces in carving order (nullptr base: sizes only)
-__host__ __device__ inline size_t carve_sr(char* base, int ni, int nb, int nh, int mode, SrLayout* L) {
+__host__ __device__ inline size_t carve_sr(char* base, int ni, int nb, int nh, int nt, int mode, SrLayout* L) {
   const int ntl = ni / PCG_TILE + 1;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -133,6 +137,7 @@ __host__ __device__ inline size_t carve_sr(char* base, int ni, int nb, int nh, i
     l.hs = (float*)take(sizeof(float) * 3 * nh);
     l.hP = (float*)take(sizeof(float) * 6 * nh);
     l.href = (int*)take(sizeof(int) * nh);
+    l.ltw = (float*)take(sizeof(float) * 3 * nt);
   }
   if (L) *L = l;
   return off;
@@ -177,7 +182,9 @@ __device__ __forceinline__ int ld_stream(const int* a, unsigned long long pol) {
 
 }  // namespace
 
-size_t pcg_sr_smem_bytes(int ni, int nb, int nh, int mode) { return carve_sr(nullptr, ni, nb, nh, mode, nullptr); }
+size_t pcg_sr_smem_bytes(int ni, int nb, int nh, int n_tiles, int mode) {
+  return carve_sr(nullptr, ni, nb, nh, n_tiles, mode, nullptr);
+}
 
 // The solve by CTA `cta` of the `grid` CTAs that share the tile table.  TEAM: the table is every
 // tile of the one scene scene_ids[0], whose CTAs are the members of a team (k_pcg_team).  False
@@ -193,7 +200,8 @@ __device__ __forceinline__ bool sr_solve(
   // scene runs on (no progress-flag wait); the same operations in the same order
   const int n_scenes = ONE ? 1 : n_scenes_arg;
   constexpr bool HALO = MODE == SR_HALO, RES = MODE == SR_RES || HALO, GV = MODE == SR_GLOBAL;
-  constexpr int MS = HALO ? HALO_MAX_SCENES : PCG_MAX_SCENES;  // scenes of one launch
+  static_assert(ONE || !HALO, "the halo layout solves one scene");
+  constexpr int MS = HALO ? 1 : PCG_MAX_SCENES;  // scenes of one launch
   constexpr int GP = SP_GP;             // lanes per BSR row in the SpMV
   constexpr int RPP = NTP / GP;         // rows per SpMV pass
   // blocks per lane per gather round: from shared memory four (more in flight lengthen the
@@ -220,7 +228,7 @@ __device__ __forceinline__ bool sr_solve(
   const int ntl = t1 - t0;
   const int n_items = ntl * PCG_TILE;
   SrLayout L;
-  carve_sr(dyn, n_items, nb_cap, nh_cap, MODE, &L);
+  carve_sr(dyn, n_items, nb_cap, nh_cap, n_tiles, MODE, &L);
   // SR_HALO: this CTA's first block in halo_col, its halo rows in halo_ref
   const int blk0 = HALO ? halo_off[2 * cta] : 0;
   const int h0 = HALO ? halo_off[2 * cta + 1] : 0;
@@ -231,6 +239,7 @@ __device__ __forceinline__ bool sr_solve(
     s_hi = -1;
     s_seen = 0;
     s_wslot = s_widx = -1;
+    if (HALO) s_sum[0][3] = 0.0f;  // (set by a tile with failed blocks)
   }
   for (int si = tid; si < n_scenes; si += NTP) {
     load_lite(sl[si], scenes[scene_ids[si]]);
@@ -368,55 +377,83 @@ __device__ __forceinline__ bool sr_solve(
   // SR_HALO: w of the halo rows hb, hb + dh, ... (stamp s, buffer par) into their u slots,
   // which the SpMV has finished reading; one row at a time (two rows' loads in flight
   // measured slower in this register-bound kernel)
-  auto halo_w = [&](int hb, int dh, unsigned s, int par) {
-    auto rec = [&](int h, int& slot, int& row) -> const unsigned long long* {
-      const int ref = L.href[h];
-      slot = ONE ? 0 : ref >> HALO_ROW_BITS;
-      row = ref & ((1 << HALO_ROW_BITS) - 1);
-      if (st[slot].done) return nullptr;
-      return reinterpret_cast<const unsigned long long*>(sl[slot].zrec) + ((size_t)par * sl[slot].nv + row) * 4;
-    };
-    auto wait = [&](const unsigned long long* wr, unsigned long long* w, int slot, int row) {
-      for (unsigned spins = 0; !(W::has(w[0], s) && W::has(w[1], s) && W::has(w[2], s)); ++spins) {
-        if (spins > kWaitSpins || *(volatile int*)&s_to) {
-          if (!s_to) {
-            s_to = 3;
-            s_seen = (unsigned)((W::has(w[0], s) ? (W::has(w[1], s) ? w[2] : w[1]) : w[0]) >> 32);
-            s_wslot = slot;
-            s_widx = row;
-          }
-          break;
+  // SR_HALO: a tile's words in buffer par: gamma, delta, rho; failed blocks (set-up).  A line per tile.
+  auto tile_word = [&](int par, int tile) {
+    return reinterpret_cast<float4*>(sl[0].pword) + ((size_t)par * sl[0].n_ptiles + tile) * 8;
+  };
+  // bounded wait for a 16-byte word of stamp s (the values in a and b); site, index: the timeout record
+  auto wait4 = [&](const float4* p, unsigned s, unsigned long long& a, unsigned long long& b, int site, int index) {
+    for (unsigned spins = 0; word4_stamp(b) != s; ++spins) {
+      if (spins > kWaitSpins || *(volatile int*)&s_to) {
+        if (!s_to) {
+          s_to = site;
+          s_seen = word4_stamp(b);
+          s_wslot = 0;
+          s_widx = index;
         }
-        ld_relaxed_v2_u64(wr, w[0], w[1]);
-        w[2] = ld_relaxed_u64(wr + 2);
+        break;
       }
-    };
+      ld_word4(p, a, b);
+    }
+  };
+  // SR_HALO: the reduction, and meanwhile the halo rows' w.  A tile's three sums come as one 16-byte
+  // word: thread t polls tile t's (at most two tiles per CTA: fewer than threads), then every thread its
+  // halo rows' words, which are posted earlier; warp 0 sums in tile order (lane-strided, then the tree)
+  // and does the scalar step.
+  auto reduce_halo = [&](unsigned s, int it) -> bool {
+    const SceneLite<float>& S = sl[0];
+    const int n = S.n_ptiles, par = it & 1;
+    const float4* tw = tile_word(par, tid);
+    unsigned long long a = 0, b = 0, fa = 0, fb = 0;
+    if (tid < n) {
+      ld_word4(tw, a, b);
+      if (it == 0) ld_word4(tw + 1, fa, fb);
+    }
 #pragma unroll 1
-    for (int h = hb; h < nh; h += dh) {
-      int sa, ra;
-      const unsigned long long* wa = rec(h, sa, ra);
-      unsigned long long a[3];
-      if (wa) {
-        ld_relaxed_v2_u64(wa, a[0], a[1]);
-        a[2] = ld_relaxed_u64(wa + 2);
-        wait(wa, a, sa, ra);
-        L.lu4[n_items + h] = make_float4(W::join(a), W::join(a + 1), W::join(a + 2), 0.0f);
+    for (int h = tid; h < nh; h += NTP) {
+      const int row = L.href[h] & ((1 << HALO_ROW_BITS) - 1);
+      const float4* p = reinterpret_cast<const float4*>(S.zrec) + (size_t)par * S.nv + row;
+      unsigned long long wa, wb;
+      ld_word4(p, wa, wb);
+      wait4(p, s, wa, wb, 3, row);
+      L.lu4[n_items + h] = make_float4(__uint_as_float((unsigned)wa), __uint_as_float((unsigned)(wa >> 32)),
+                                       __uint_as_float((unsigned)wb), 0.0f);
+    }
+    if (tid < n) {
+      wait4(tw, s, a, b, 2, tid);
+      L.ltw[tid] = __uint_as_float((unsigned)a);
+      L.ltw[n + tid] = __uint_as_float((unsigned)(a >> 32));
+      L.ltw[2 * n + tid] = __uint_as_float((unsigned)b);
+      if (it == 0) {
+        wait4(tw + 1, s, fa, fb, 2, tid);
+        if (__uint_as_float((unsigned)fa) > 0.0f) s_sum[0][3] = 1.0f;
       }
     }
+    __syncthreads();
+    if (s_to) return false;
+    if (warp == 0) {
+      float acc[3] = {0.0f, 0.0f, 0.0f};
+      for (int t = lane32; t < n; t += 32)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) acc[q] += L.ltw[q * n + t];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+      if (lane32 == 0)
+        sr_step_fast(st[0], acc[0], acc[1], acc[2], it == 0 ? s_sum[0][3] : 0.0f, it, s_tol2[0], sl[0].max_iter);
+    }
+    __syncthreads();
+    return true;
   };
   // every CTA sums the tile words (buffer par) of quantities [0, nq) of every live scene
   // in tile order.  Once a scene of the launch has finished, a CTA may have no live tile
   // left and post nothing; one warp then also waits until every CTA has started this
   // iteration (progress flag >= s), so that no CTA is ever a whole iteration behind
   // another, which the parity buffers rely on.  (While every scene is live, every CTA
-  // posts every iteration and the tile words alone ensure it.)  SR_HALO: the
-  // halo's w words are read meanwhile, by the warps without other work when they are at
-  // least half of the CTA, else by every warp first.
+  // posts every iteration and the tile words alone ensure it.)
   auto reduce = [&](int nq, unsigned s, int par) -> bool {
     const int npw = n_scenes * nq + 1;  // warps with words to wait for (the last: the flags)
-    if constexpr (HALO) {
-      if (npw > NW / 2) halo_w(tid, NTP, s, par);
-    }
     for (int x = warp; x < npw; x += NW) {
       if (x == npw - 1) {
         if constexpr (!ONE) {
@@ -471,9 +508,6 @@ __device__ __forceinline__ bool sr_solve(
       acc = warp_sum(acc);
       if (lane32 == 0) s_sum[si][q] = acc;
     }
-    if constexpr (HALO) {
-      if (npw <= NW / 2 && warp >= npw) halo_w((warp - npw) * 32 + lane32, (NW - npw) * 32, s, par);
-    }
     __syncthreads();
     return !s_to;
   };
@@ -506,6 +540,15 @@ __device__ __forceinline__ bool sr_solve(
     const SceneLite<float>& S = sl[sc];
     if (st[sc].done) return;
     const float* w = L.lws + NQ * 8 * lt;
+    if constexpr (HALO) {
+      float v[NQ];
+      for (int q = 0; q < nq; ++q)
+        v[q] = ((w[q] + w[NQ + q]) + (w[2 * NQ + q] + w[3 * NQ + q])) +
+               ((w[4 * NQ + q] + w[5 * NQ + q]) + (w[6 * NQ + q] + w[7 * NQ + q]));
+      st_word4(tile_word(par, tr.tile), v[0], v[1], v[2], s);
+      if (nq == NQ) st_word4(tile_word(par, tr.tile) + 1, v[3], 0.0f, 0.0f, s);
+      return;
+    }
     const size_t ws = (size_t)pword_stride(S.n_ptiles);
     unsigned long long* wbase = S.pword + ((size_t)par * NQ * S.n_ptiles + tr.tile) * ws;
     for (int q = 0; q < nq; ++q) {
@@ -545,10 +588,10 @@ __device__ __forceinline__ bool sr_solve(
             for (int u = 0; u < U; ++u) {
               const int j = jb + u;
               if (GP * j + lane < len) {
-                const float* v = L.lval + (j0 + j) * 288 + lane32;
-                float a[9];
-#pragma unroll
-                for (int c = 0; c < 9; ++c) a[c] = v[32 * c];
+                const float* v = L.lval + (j0 + j) * 288;
+                const float4 v0 = reinterpret_cast<const float4*>(v)[lane32];
+                const float4 v1 = reinterpret_cast<const float4*>(v + 128)[lane32];
+                const float a[9] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w, v[256 + lane32]};
                 blk_mv(a, vj[u].x, vj[u].y, vj[u].z, ax, ay, az);
               }
             }
@@ -604,14 +647,7 @@ __device__ __forceinline__ bool sr_solve(
             r[0] = rv.x, r[1] = rv.y, r[2] = rv.z;
             u[0] = uv.x, u[1] = uv.y, u[2] = uv.z;
           } else if constexpr (HALO) {
-            unsigned long long w[3];
-            W::split(ax, s, w);
-            W::split(ay, s, w + 1);
-            W::split(az, s, w + 2);
-            unsigned long long* wr =
-                reinterpret_cast<unsigned long long*>(sl[slot].zrec) + ((size_t)par * sl[slot].nv + i) * 4;
-            st_relaxed_v2_u64(wr, w[0], w[1]);
-            st_relaxed_u64(wr + 2, w[2]);
+            st_word4(reinterpret_cast<float4*>(sl[slot].zrec) + (size_t)par * sl[slot].nv + i, ax, ay, az, s);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
               u[c] = ou[c];
@@ -814,23 +850,27 @@ __device__ __forceinline__ bool sr_solve(
     const unsigned s = W::stamp((unsigned)it + 1);
     if constexpr (HALO) {
       __syncthreads();  // set-up, or the previous update, before the SpMV
-      if (!TEAM && tid == 0) st_relaxed_u64(flags + cta, (unsigned long long)it + 1);  // progress
     } else {
       // ---- u released to the neighbours (set-up wrote u_0; later iterations below)
       publish_flag((unsigned long long)it + 1);
       if (!wait_flags((unsigned long long)it + 1)) return fail_out(it);
     }
     spmv(s, it & 1, it == 0 ? NQ : 3);  // w = A u, and the tile partials posted
-    if (!reduce(it == 0 ? NQ : 3, s, it & 1)) return fail_out(it);
-    // one thread per scene (n_scenes <= MS < NTP); the barrier also finds whether all are done
-    int done = 1;
-    if (tid < n_scenes) {
-      if (!st[tid].done)
-        sr_step(st[tid], s_sum[tid][0], s_sum[tid][1], s_sum[tid][2], it == 0 ? s_sum[tid][3] : 0.0f, it,
-                s_tol2[tid], sl[tid].max_iter);
-      done = st[tid].done;
+    if constexpr (HALO) {
+      if (!reduce_halo(s, it)) return fail_out(it);
+      if (st[0].done) break;
+    } else {
+      if (!reduce(it == 0 ? NQ : 3, s, it & 1)) return fail_out(it);
+      // one thread per scene (n_scenes <= MS < NTP); the barrier also finds whether all are done
+      int done = 1;
+      if (tid < n_scenes) {
+        if (!st[tid].done)
+          sr_step(st[tid], s_sum[tid][0], s_sum[tid][1], s_sum[tid][2], it == 0 ? s_sum[tid][3] : 0.0f, it,
+                  s_tol2[tid], sl[tid].max_iter);
+        done = st[tid].done;
+      }
+      if (__syncthreads_and(done)) break;
     }
-    if (__syncthreads_and(done)) break;
     // ---- p = u + beta p, s = w + beta s; x += alpha p, r -= alpha s, u = M r (published)
     if constexpr (HALO) {
       if (o_row >= 0 && !st[o_slot].done) {
@@ -1026,14 +1066,14 @@ static const void* sr_kernel(int mode, bool one) {
     case SR_RES: return one ? (const void*)k_pcg_sr<SR_RES, true> : (const void*)k_pcg_sr<SR_RES, false>;
     case SR_STREAM: return one ? (const void*)k_pcg_sr<SR_STREAM, true> : (const void*)k_pcg_sr<SR_STREAM, false>;
     case SR_GLOBAL: return one ? (const void*)k_pcg_sr<SR_GLOBAL, true> : (const void*)k_pcg_sr<SR_GLOBAL, false>;
-    default: return (const void*)k_pcg_sr<SR_HALO, false>;
+    default: return (const void*)k_pcg_sr<SR_HALO, true>;
   }
 }
 
 int pcg_sr_max_grid(int device, size_t smem, int mode) {
   // (the multi-scene form; the single-scene forms use no more registers or shared memory, so the
   // same one CTA per SM is co-resident, and the launch sets its own kernel's attribute)
-  const void* k = sr_kernel(mode, false);
+  const void* k = sr_kernel(mode, false);  // (SR_HALO: the one form)
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -1095,7 +1135,7 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
   const bool halo = L.sr_mode == SR_HALO;
   if (L.n_scenes <= 0 || L.n_scenes > PCG_MAX_SCENES || L.n_tiles <= 0 || L.grid > XCH_MAX_CTAS || !L.flags ||
       L.sr_mode < SR_RES || L.sr_mode > SR_HALO || (L.sr_mode == SR_RES || halo) != (L.smem_blocks > 0) ||
-      (halo && (L.n_scenes > HALO_MAX_SCENES || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
+      (halo && (L.n_scenes != 1 || L.n_tiles > NTP || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
                 (L.n_tiles + L.grid - 1) / L.grid * PCG_TILE > SR_HALO_MAX_ROWS)))
     return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(L.bar, 0, sizeof(GridBar), st);
