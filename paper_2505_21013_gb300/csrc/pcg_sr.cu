@@ -409,15 +409,25 @@ __device__ __forceinline__ bool sr_solve(
       ld_word4(tw, a, b);
       if (it == 0) ld_word4(tw + 1, fa, fb);
     }
-#pragma unroll 1
-    for (int h = tid; h < nh; h += NTP) {
-      const int row = L.href[h] & ((1 << HALO_ROW_BITS) - 1);
-      const float4* p = reinterpret_cast<const float4*>(S.zrec) + (size_t)par * S.nv + row;
-      unsigned long long wa, wb;
-      ld_word4(p, wa, wb);
-      wait4(p, s, wa, wb, 3, row);
+    // (two halo rows' words in flight; more rows than that are rare)
+    const float4* zp = reinterpret_cast<const float4*>(S.zrec) + (size_t)par * S.nv;
+    auto halo_put = [&](int h, unsigned long long wa, unsigned long long wb) {
       L.lu4[n_items + h] = make_float4(__uint_as_float((unsigned)wa), __uint_as_float((unsigned)(wa >> 32)),
                                        __uint_as_float((unsigned)wb), 0.0f);
+    };
+#pragma unroll 1
+    for (int h = tid; h < nh; h += 2 * NTP) {
+      const bool two = h + NTP < nh;
+      const int r0 = L.href[h] & ((1 << HALO_ROW_BITS) - 1), r1 = two ? L.href[h + NTP] & ((1 << HALO_ROW_BITS) - 1) : r0;
+      unsigned long long wa, wb, xa, xb;
+      ld_word4(zp + r0, wa, wb);
+      ld_word4(zp + r1, xa, xb);
+      wait4(zp + r0, s, wa, wb, 3, r0);
+      halo_put(h, wa, wb);
+      if (two) {
+        wait4(zp + r1, s, xa, xb, 3, r1);
+        halo_put(h + NTP, xa, xb);
+      }
     }
     if (tid < n) {
       wait4(tw, s, a, b, 2, tid);
@@ -638,7 +648,12 @@ __device__ __forceinline__ bool sr_solve(
       }
       // the row's terms: gamma = r.u and rho = r.r in its first lane, delta = w.u in its second
       float x = 0.f, rr = 0.f;
-      if (item < n_items && i >= 0 && !st[slot].done) {
+      if constexpr (HALO) {
+        // (no branch: the second lanes' r is zero, as are rows past the last one)
+        const float4 uv = item < n_items ? L.lu4[item] : make_float4(0.f, 0.f, 0.f, 0.f);
+        x = dot3(lane ? ax : orr[0], lane ? ay : orr[1], lane ? az : orr[2], uv.x, uv.y, uv.z);
+        rr = dot3(orr[0], orr[1], orr[2], orr[0], orr[1], orr[2]);
+      } else if (item < n_items && i >= 0 && !st[slot].done) {
         if (lane == 0) {
           float r[3], u[3];
           if constexpr (GV) {
@@ -646,13 +661,6 @@ __device__ __forceinline__ bool sr_solve(
             const float4 uv = ld_f4_cg(u_ptr(sl[slot].zrec, i));
             r[0] = rv.x, r[1] = rv.y, r[2] = rv.z;
             u[0] = uv.x, u[1] = uv.y, u[2] = uv.z;
-          } else if constexpr (HALO) {
-            st_word4(reinterpret_cast<float4*>(sl[slot].zrec) + (size_t)par * sl[slot].nv + i, ax, ay, az, s);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              u[c] = ou[c];
-              r[c] = orr[c];
-            }
           } else {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -666,9 +674,6 @@ __device__ __forceinline__ bool sr_solve(
           float u[3];
           if constexpr (GV) {
             const float4 uv = ld_f4_cg(u_ptr(sl[slot].zrec, i));
-            u[0] = uv.x, u[1] = uv.y, u[2] = uv.z;
-          } else if constexpr (HALO) {
-            const float4 uv = L.lu4[item];
             u[0] = uv.x, u[1] = uv.y, u[2] = uv.z;
           } else {
 #pragma unroll
@@ -690,6 +695,10 @@ __device__ __forceinline__ bool sr_solve(
       if (lane32 == 0) {
         og[0] = x;
         og[2] = rr;
+      }
+      if constexpr (HALO) {  // (w out after the sums, which the whole grid waits for)
+        if (lane == 0 && i >= 0)
+          st_word4(reinterpret_cast<float4*>(sl[0].zrec) + (size_t)par * sl[0].nv + i, ax, ay, az, s);
       }
       __syncwarp();  // (delta's sum, stored by lane 16, before lane 0's count)
       if (lane32 == 0) {
