@@ -443,9 +443,18 @@ __device__ __forceinline__ bool sr_solve(
     if (s_to) return false;
     if (warp == 0) {
       float acc[3] = {0.0f, 0.0f, 0.0f};
-      for (int t = lane32; t < n; t += 32)
+      // (all of a lane's loads issued before its sums: at most NTP / 32 tiles per lane)
+      for (int t0 = 0; t0 < n; t0 += 32 * 8) {
+        float v[8][3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) acc[q] += L.ltw[q * n + t];
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int q = 0; q < 3; ++q) v[k][q] = t0 + 32 * k + lane32 < n ? L.ltw[q * n + t0 + 32 * k + lane32] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int q = 0; q < 3; ++q) acc[q] += v[k][q];
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
