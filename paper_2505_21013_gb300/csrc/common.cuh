@@ -20,6 +20,7 @@ constexpr int PCG_TILE = 128;  // BSR rows per PCG reduction tile
 constexpr int HE_STRIDE = 96;  // values per element Hessian record (10 blocks x 9, padded)
 constexpr int GE_STRIDE = 12;  // values per element gradient record
 constexpr int TETC_STRIDE = 12;  // Dm^-1 (9), V, mu, lam_s
+constexpr int SELL_STEP = 320;   // words of a block step: 32 x 4 (values 0..3), 32 x 4 (4..7), 32 (8), 32 columns
 
 template <typename T> struct Vec4;
 template <> struct Vec4<float> { using type = float4; };
@@ -116,6 +117,9 @@ struct SceneDev {
   double* tpart;           // tet tiles
   double* ppart;           // PCG tiles
   unsigned long long* pword;  // PCG tile partials as stamped words, [4][n_ptiles][<= 2]
+  const int* gstep;           // FP32 path: ceil(nv / 16) + 1 first block steps of the 16-row groups (streamed PCG layouts)
+  T* steps;                   // FP32 path: room for the blocks by step (SELL_STEP words each), or null; the memory of
+                              // dH, which nothing reads between a solve's start and the next projection
   T* zrec;                    // FP32 path: [2][nv] 32-byte records {z, 0, d_prev, 0} of the resident PCG
   double* psi_out;         // optional per-element energies (probes)
   Ctl* ctl;

@@ -425,6 +425,10 @@ struct Driver {
           }
         PPN_CU(cudaEventRecord(G.tune_ev[0], G.st));
       }
+      // blocks by step (PPN_PCG_NO_STEPS=1: row by row; tests)
+      L.sell = std::getenv("PPN_PCG_NO_STEPS") ? 0 : 1;
+      for (int k : sl)
+        if (!G.h_desc[k].steps) L.sell = 0;
       for (int k : sl) G.S[k]->last_pcg_layout = G.pcg_sr ? L.sr_mode : L.smem_bytes ? 4 : 5;
       L.launch_seq = ++G.pcg_launch_seq;
       L.flags = G.d_flags;

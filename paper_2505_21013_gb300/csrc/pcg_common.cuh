@@ -207,6 +207,8 @@ struct SceneLite {
   double* ppart;
   unsigned long long* pword;
   T* zrec;
+  const int* gstep;
+  T* steps;
   Ctl* ctl;
   double tol2;
   int nv, nnzb, n_ptiles, max_iter;
@@ -229,6 +231,8 @@ __device__ __forceinline__ void load_lite(SceneLite<T>& L, const SceneDev<T>& S)
   L.ppart = S.ppart;
   L.pword = S.pword;
   L.zrec = S.zrec;
+  L.gstep = S.gstep;
+  L.steps = S.steps;
   L.ctl = S.ctl;
   L.tol2 = S.pcg_tol2;
   L.nv = S.nv;

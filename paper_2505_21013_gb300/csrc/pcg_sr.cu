@@ -174,6 +174,19 @@ __device__ __forceinline__ float ld_stream(const float* a, unsigned long long po
   asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
   return v;
 }
+// block steps, which the CTA itself wrote in the set-up (so not the non-coherent path), once per SpMV
+__device__ __forceinline__ float4 ld_step4(const float* a, unsigned long long pol) {
+  float4 v;
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(a), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ float ld_step1(const float* a, unsigned long long pol) {
+  float v;
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
+  return v;
+}
 __device__ __forceinline__ int ld_stream(const int* a, unsigned long long pol) {
   int v;
   asm("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol));
@@ -189,12 +202,13 @@ size_t pcg_sr_smem_bytes(int ni, int nb, int nh, int n_tiles, int mode) {
 // The solve by CTA `cta` of the `grid` CTAs that share the tile table.  TEAM: the table is every
 // tile of the one scene scene_ids[0], whose CTAs are the members of a team (k_pcg_team).  False
 // when a wait ran out (the timeout is recorded).
-template <int MODE, bool ONE, bool TEAM>
+template <int MODE, bool ONE, bool TEAM, bool SELL>
 __device__ __forceinline__ bool sr_solve(
     int cta, int grid, const SceneDev<float>* scenes, const TileRef* tiles, int n_tiles, const int* scene_ids,
     int n_scenes_arg, GridBar* bar, int b_from_g, int nb_cap, unsigned long long* flags, const int* halo_off,
     const int* halo_col, const int* halo_ref, int nh_cap, int l2_keep) {
   static_assert(!TEAM || (ONE && MODE == SR_HALO), "a team solves one scene in the halo layout");
+  static_assert(!SELL || MODE == SR_STREAM || MODE == SR_GLOBAL, "only streamed blocks go by steps");
   using W = Words<float>;
   // ONE: a launch of a single scene, whose slot is 0 and which never finishes while another
   // scene runs on (no progress-flag wait); the same operations in the same order
@@ -367,6 +381,26 @@ __device__ __forceinline__ bool sr_solve(
     if constexpr (!HALO) {
       atomicMin(&s_lo, lo);
       atomicMax(&s_hi, hi);
+    }
+  }
+  // SELL: this CTA's rows' blocks by step, a warp per 16-row group, lanes as in the SpMV
+  if constexpr (SELL) {
+    const int h = spmv_lane(tid);
+    for (int item = 16 * warp + (lane32 & 15); item < n_items; item += 16 * NW) {
+      int slot;
+      const int i = row_of(item, slot);
+      if (i < 0) continue;
+      const SceneLite<float>& S = sl[slot];
+      const int kb = S.row_ptr[i], len = S.row_ptr[i + 1] - kb;
+      const size_t nb = (size_t)S.nnzb;
+      float* p = S.steps + (size_t)S.gstep[i >> 4] * SELL_STEP;
+      for (int k = h; k < len; k += 2, p += SELL_STEP) {
+        const float* v = S.val + kb + k;
+        *reinterpret_cast<float4*>(p + 4 * lane32) = make_float4(v[0], v[nb], v[2 * nb], v[3 * nb]);
+        *reinterpret_cast<float4*>(p + 128 + 4 * lane32) = make_float4(v[4 * nb], v[5 * nb], v[6 * nb], v[7 * nb]);
+        p[256 + lane32] = v[8 * nb];
+        p[288 + lane32] = __int_as_float(S.col[kb + k]);
+      }
     }
   }
   __syncthreads();
@@ -614,6 +648,36 @@ __device__ __forceinline__ bool sr_solve(
                 blk_mv(a, vj[u].x, vj[u].y, vj[u].z, ax, ay, az);
               }
             }
+          }
+        } else if constexpr (SELL) {
+          // blocks by step from global memory: whole lines per load (the loads below touch 28 half-used
+          // sectors each, and the L1's tag lookups, not HBM, set the pace)
+          const int len = S.row_ptr[i + 1] - S.row_ptr[i], g = i >> 4;
+          const int j0 = __ldg(S.gstep + g), nj = __ldg(S.gstep + g + 1) - j0;
+          const float* sb = S.steps + (size_t)j0 * SELL_STEP;
+          constexpr int US = 4;  // steps in flight per lane
+          for (int jb = 0; jb < nj; jb += US) {
+            int cl[US];
+            float4 a0[US], a1[US], vj[US];
+            float a2[US];
+#pragma unroll
+            for (int u = 0; u < US; ++u)
+              if (GP * (jb + u) + lane < len) {
+                const float* p = sb + (size_t)(jb + u) * SELL_STEP;
+                cl[u] = __float_as_int(ld_step1(p + 288 + lane32, pol));
+                a0[u] = ld_step4(p + 4 * lane32, pol);
+                a1[u] = ld_step4(p + 128 + 4 * lane32, pol);
+                a2[u] = ld_step1(p + 256 + lane32, pol);
+              }
+#pragma unroll
+            for (int u = 0; u < US; ++u)
+              if (GP * (jb + u) + lane < len) vj[u] = ld_f4_cg(vb + (size_t)8 * cl[u]);
+#pragma unroll
+            for (int u = 0; u < US; ++u)
+              if (GP * (jb + u) + lane < len) {
+                const float a[9] = {a0[u].x, a0[u].y, a0[u].z, a0[u].w, a1[u].x, a1[u].y, a1[u].z, a1[u].w, a2[u]};
+                blk_mv(a, vj[u].x, vj[u].y, vj[u].z, ax, ay, az);
+              }
           }
         } else {
           // blocks from global memory (component-major values), read-only path, evict-first in L2
@@ -1013,12 +1077,12 @@ __device__ __forceinline__ bool sr_solve(
   return true;
 }
 
-template <int MODE, bool ONE>
+template <int MODE, bool ONE, bool SELL = false>
 __global__ void __launch_bounds__(NTP, 1)
     k_pcg_sr(const SceneDev<float>* scenes, const TileRef* tiles, int n_tiles, const int* scene_ids,
              int n_scenes, GridBar* bar, int b_from_g, int nb_cap, unsigned long long* flags,
              const int* halo_off, const int* halo_col, const int* halo_ref, int nh_cap, int l2_keep) {
-  sr_solve<MODE, ONE, false>((int)blockIdx.x, (int)gridDim.x, scenes, tiles, n_tiles, scene_ids, n_scenes, bar,
+  sr_solve<MODE, ONE, false, SELL>((int)blockIdx.x, (int)gridDim.x, scenes, tiles, n_tiles, scene_ids, n_scenes, bar,
                              b_from_g, nb_cap, flags, halo_off, halo_col, halo_ref, nh_cap, l2_keep);
 }
 
@@ -1043,7 +1107,7 @@ __global__ void __launch_bounds__(NTP, 1)
     for (int j = threadIdx.x; j < n_jobs; j += NTP)
       if (jobs[j].ticket <= t && t < jobs[j].ticket + jobs[j].size) job = jobs[j];
     __syncthreads();
-    if (!sr_solve<SR_HALO, true, true>(t - job.ticket, job.size, scenes, nullptr, job.n_tiles, &job.scene, 1, bar,
+    if (!sr_solve<SR_HALO, true, true, false>(t - job.ticket, job.size, scenes, nullptr, job.n_tiles, &job.scene, 1, bar,
                                        b_from_g, job.slots, nullptr, job.halo_off, job.halo_col, job.halo_ref,
                                        job.halo_cap, 0))
       return;
@@ -1079,11 +1143,17 @@ cudaError_t launch_wait_probe(const unsigned long long* w, int n, unsigned long 
 // (press, global layout, same-box A/B: 50.1 -> 45.5 us per CG iteration, the same bits).
 // The halo layout keeps one form: its single-scene form measured 4.48 -> 4.66 us on the
 // beam, where the compiler schedules the register-resident rows differently.
-static const void* sr_kernel(int mode, bool one) {
+// `sell`: every scene has room for its blocks by step (the streamed layouts).
+template <int MODE>
+static const void* sr_streamed(bool one, bool sell) {
+  return one ? (sell ? (const void*)k_pcg_sr<MODE, true, true> : (const void*)k_pcg_sr<MODE, true, false>)
+             : (sell ? (const void*)k_pcg_sr<MODE, false, true> : (const void*)k_pcg_sr<MODE, false, false>);
+}
+static const void* sr_kernel(int mode, bool one, bool sell) {
   switch (mode) {
     case SR_RES: return one ? (const void*)k_pcg_sr<SR_RES, true> : (const void*)k_pcg_sr<SR_RES, false>;
-    case SR_STREAM: return one ? (const void*)k_pcg_sr<SR_STREAM, true> : (const void*)k_pcg_sr<SR_STREAM, false>;
-    case SR_GLOBAL: return one ? (const void*)k_pcg_sr<SR_GLOBAL, true> : (const void*)k_pcg_sr<SR_GLOBAL, false>;
+    case SR_STREAM: return sr_streamed<SR_STREAM>(one, sell);
+    case SR_GLOBAL: return sr_streamed<SR_GLOBAL>(one, sell);
     default: return (const void*)k_pcg_sr<SR_HALO, true>;
   }
 }
@@ -1091,7 +1161,7 @@ static const void* sr_kernel(int mode, bool one) {
 int pcg_sr_max_grid(int device, size_t smem, int mode) {
   // (the multi-scene form; the single-scene forms use no more registers or shared memory, so the
   // same one CTA per SM is co-resident, and the launch sets its own kernel's attribute)
-  const void* k = sr_kernel(mode, false);  // (SR_HALO: the one form)
+  const void* k = sr_kernel(mode, false, false);  // (SR_HALO: the one form)
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -1186,7 +1256,7 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
   void* args[] = {(void*)&scenes, (void*)&tiles, (void*)&n_tiles, (void*)&ids,   (void*)&n_scenes,
                   (void*)&bar,    (void*)&bg,    (void*)&nb_cap,  (void*)&flags, (void*)&h_off,
                   (void*)&h_col,  (void*)&h_ref, (void*)&nh_cap, (void*)&l2_keep};
-  const void* k = sr_kernel(L.sr_mode, L.n_scenes == 1);
+  const void* k = sr_kernel(L.sr_mode, L.n_scenes == 1, L.sell != 0);
   e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(NTP), args, L.smem_bytes, st);

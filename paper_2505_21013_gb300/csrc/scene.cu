@@ -397,6 +397,22 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
   s.ppart = alloc<double>((size_t)4 * n_ptiles);
   s.pword = alloc<unsigned long long>((size_t)8 * n_ptiles * pword_stride(n_ptiles));
   s.zrec = sizeof(T) == 4 ? alloc<T>((size_t)16 * nv) : nullptr;
+  // the streamed PCG layouts' block steps: their room is dH's when that is large enough (a mesh of few shared
+  // vertices or a group with one very long row may need more; such a scene streams its blocks row by row)
+  std::vector<int> gstep;
+  if (sizeof(T) == 4) {
+    gstep.assign((nv + 15) / 16 + 1, 0);
+    int64_t steps = 0;
+    for (int g = 0; 16 * g < nv; ++g) {
+      int64_t m = 0;
+      for (int r = 16 * g; r < std::min(nv, 16 * g + 16); ++r) m = std::max(m, h_row_ptr[r + 1] - h_row_ptr[r]);
+      steps += (m + 1) / 2;
+      gstep[g + 1] = (int)std::min<int64_t>(steps, INT32_MAX);
+    }
+    d_gstep = alloc<int>(gstep.size());
+    if (steps * SELL_STEP <= (int64_t)nt * HE_STRIDE) s.steps = s.dH;
+  }
+  s.gstep = d_gstep;
   s.ctl = alloc<Ctl>(1);
   d_desc = alloc<SceneDev<T>>(1);
   d_ids = alloc<int>(1);
@@ -418,7 +434,7 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
       !d_col || !d_blk_row || !d_blk_ptr || !d_blk_src || !d_blk_lane || !d_diag || !d_tet_blk || !s.blk_mark || !s.touched || !s.u || !s.u_n || !s.vel ||
       !s.uhat || !s.u_probe || !s.ge || !s.He || !s.dH || !s.g || !s.gmax || !s.val ||
       !s.proj_stamp || !s.round_stamp || !s.cproj_stamp || !d_obs || !s.cround_stamp || !s.dHc || !s.Hc || !s.sel_list || !s.dx || !s.r || !s.z || !s.q || !s.d0 ||
-      !s.d1 || !s.Pinv || !s.vpart || !s.tpart || !s.ppart || !s.pword || (sizeof(T) == 4 && !s.zrec) || !s.ctl || !d_desc || !d_ids ||
+      !s.d1 || !s.Pinv || !s.vpart || !s.tpart || !s.ppart || !s.pword || (sizeof(T) == 4 && (!s.zrec || !d_gstep)) || !s.ctl || !d_desc || !d_ids ||
       !d_bar || !d_fixed_list || !d_targets || !d_xyz || !d_ttiles || !d_vtiles || !d_btiles ||
       !d_ptiles || !d_etiles || !d_projtiles) {
     set_error("cudaMalloc failed (scene needs more device memory than is free)");
@@ -454,6 +470,7 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
     PPN_CU(up(d_blk_lane, lane.data(), lane.size()));
   }
   PPN_CU(up(d_diag, diag_idx.data(), sizeof(int) * nv));
+  if (d_gstep) PPN_CU(up(d_gstep, gstep.data(), sizeof(int) * gstep.size()));
   PPN_CU(up(d_tet_blk, blk_of.data(), sizeof(int) * blk_of.size()));
   PPN_CU(cudaMemset(s.blk_mark, 0xff, sizeof(int) * nnzb));
   if (nfixed) {

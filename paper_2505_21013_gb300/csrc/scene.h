@@ -109,6 +109,7 @@ struct SceneImpl {
           *d_etiles = nullptr, *d_projtiles = nullptr;
   int* d_ids = nullptr;
   GridBar* d_bar = nullptr;
+  int* d_gstep = nullptr;
   int* d_fixed_list = nullptr;
   double* d_targets = nullptr;
   const double* ext_targets = nullptr;  // device targets given by the caller for the next step
