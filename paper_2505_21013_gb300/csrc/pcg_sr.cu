@@ -215,7 +215,7 @@ __device__ __forceinline__ bool sr_solve(
   const int n_scenes = ONE ? 1 : n_scenes_arg;
   constexpr bool HALO = MODE == SR_HALO, RES = MODE == SR_RES || HALO, GV = MODE == SR_GLOBAL;
   static_assert(ONE || !HALO, "the halo layout solves one scene");
-  constexpr int MS = HALO ? 1 : PCG_MAX_SCENES;  // scenes of one launch
+  constexpr int MS = ONE ? 1 : PCG_MAX_SCENES;  // scenes of one launch
   constexpr int GP = SP_GP;             // lanes per BSR row in the SpMV
   constexpr int RPP = NTP / GP;         // rows per SpMV pass
   // blocks per lane per gather round: from shared memory four (more in flight lengthen the
@@ -253,7 +253,7 @@ __device__ __forceinline__ bool sr_solve(
     s_hi = -1;
     s_seen = 0;
     s_wslot = s_widx = -1;
-    if (HALO) s_sum[0][3] = 0.0f;  // (set by a tile with failed blocks)
+    if (ONE) s_sum[0][3] = 0.0f;  // (set by a tile with failed blocks)
   }
   for (int si = tid; si < n_scenes; si += NTP) {
     load_lite(sl[si], scenes[scene_ids[si]]);
@@ -411,9 +411,11 @@ __device__ __forceinline__ bool sr_solve(
   // SR_HALO: w of the halo rows hb, hb + dh, ... (stamp s, buffer par) into their u slots,
   // which the SpMV has finished reading; one row at a time (two rows' loads in flight
   // measured slower in this register-bound kernel)
-  // SR_HALO: a tile's words in buffer par: gamma, delta, rho; failed blocks (set-up).  A line per tile.
+  // ONE: a tile's 16-byte words in buffer par: gamma, delta, rho; failed blocks (set-up).  A line per
+  // tile, or half of one past 512 tiles (the array's size: pword_stride).
+  const int tw_step = ONE && sl[0].n_ptiles > 512 ? 4 : 8;
   auto tile_word = [&](int par, int tile) {
-    return reinterpret_cast<float4*>(sl[0].pword) + ((size_t)par * sl[0].n_ptiles + tile) * 8;
+    return reinterpret_cast<float4*>(sl[0].pword) + ((size_t)par * sl[0].n_ptiles + tile) * tw_step;
   };
   // bounded wait for a 16-byte word of stamp s (the values in a and b); site, index: the timeout record
   auto wait4 = [&](const float4* p, unsigned s, unsigned long long& a, unsigned long long& b, int site, int index) {
@@ -496,6 +498,55 @@ __device__ __forceinline__ bool sr_solve(
       if (lane32 == 0)
         sr_step_fast(st[0], acc[0], acc[1], acc[2], it == 0 ? s_sum[0][3] : 0.0f, it, s_tol2[0], sl[0].max_iter);
     }
+    __syncthreads();
+    return true;
+  };
+  // ONE without the halo: the reduction, in chunks of a tile per thread.  Thread t polls tile c + t's word
+  // (the next chunk's load in flight); warps 0..2 sum a quantity each, in tile order (lane-strided, then
+  // the tree); thread 0 does the scalar step.  Three warps that polled three words per tile, eight at a
+  // time, took 13 k cycles for 2000 tiles.
+  __shared__ float s_ch[ONE && !HALO ? 2 * 3 * NTP : 1];
+  auto reduce_one = [&](unsigned s, int it) -> bool {
+    const int n = sl[0].n_ptiles, par = it & 1;
+    float acc = 0.0f;
+    unsigned long long a = 0, b = 0;
+    if (tid < n) ld_word4(tile_word(par, tid), a, b);
+    for (int c0 = 0; c0 < n; c0 += NTP) {
+      const int t = c0 + tid;
+      float* ch = s_ch + ((c0 / NTP) & 1) * 3 * NTP;
+      unsigned long long na = 0, nb = 0;
+      if (t + NTP < n) ld_word4(tile_word(par, t + NTP), na, nb);
+      if (t < n) {
+        wait4(tile_word(par, t), s, a, b, 2, t);
+        ch[tid] = __uint_as_float((unsigned)a);
+        ch[NTP + tid] = __uint_as_float((unsigned)(a >> 32));
+        ch[2 * NTP + tid] = __uint_as_float((unsigned)b);
+        if (it == 0) {
+          unsigned long long fa, fb;
+          ld_word4(tile_word(par, t) + 1, fa, fb);
+          wait4(tile_word(par, t) + 1, s, fa, fb, 2, t);
+          if (__uint_as_float((unsigned)fa) > 0.0f) s_sum[0][3] = 1.0f;
+        }
+      }
+      a = na, b = nb;
+      __syncthreads();
+      if (warp < 3) {
+        float v[NTP / 32];
+#pragma unroll
+        for (int k = 0; k < NTP / 32; ++k) v[k] = c0 + 32 * k + lane32 < n ? ch[warp * NTP + 32 * k + lane32] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < NTP / 32; ++k) acc += v[k];
+      }
+    }
+    if (warp < 3) {
+      acc = warp_sum(acc);
+      if (lane32 == 0) s_sum[0][warp] = acc;
+    }
+    __syncthreads();
+    if (s_to) return false;
+    if (tid == 0)
+      sr_step_fast(st[0], s_sum[0][0], s_sum[0][1], s_sum[0][2], it == 0 ? s_sum[0][3] : 0.0f, it, s_tol2[0],
+                   sl[0].max_iter);
     __syncthreads();
     return true;
   };
@@ -593,7 +644,7 @@ __device__ __forceinline__ bool sr_solve(
     const SceneLite<float>& S = sl[sc];
     if (st[sc].done) return;
     const float* w = L.lws + NQ * 8 * lt;
-    if constexpr (HALO) {
+    if constexpr (ONE) {
       float v[NQ];
       for (int q = 0; q < nq; ++q)
         v[q] = ((w[q] + w[NQ + q]) + (w[2 * NQ + q] + w[3 * NQ + q])) +
@@ -942,16 +993,34 @@ __device__ __forceinline__ bool sr_solve(
       if (!reduce_halo(s, it)) return fail_out(it);
       if (st[0].done) break;
     } else {
-      if (!reduce(it == 0 ? NQ : 3, s, it & 1)) return fail_out(it);
-      // one thread per scene (n_scenes <= MS < NTP); the barrier also finds whether all are done
-      int done = 1;
-      if (tid < n_scenes) {
-        if (!st[tid].done)
-          sr_step(st[tid], s_sum[tid][0], s_sum[tid][1], s_sum[tid][2], it == 0 ? s_sum[tid][3] : 0.0f, it,
-                  s_tol2[tid], sl[tid].max_iter);
-        done = st[tid].done;
+      if constexpr (SELL && ONE) {
+        // a matrix larger than L2 (evict-first): the start of the next SpMV's steps to L2 while the grid
+        // reduces and updates (press 34.5 -> 33.3 us per CG iteration; 64 and 256 KB: 33.7, 33.6)
+        if (!l2_keep) {
+          const int ng = (sl[0].nv + 15) / 16, j0 = sl[0].gstep[min(8 * t0, ng)];
+          const int n = min(sl[0].gstep[min(8 * t1, ng)] - j0, (128 << 10) / (4 * SELL_STEP));
+          const float* p = sl[0].steps + (size_t)j0 * SELL_STEP;
+          for (int j = tid; j < n; j += NTP)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + (size_t)j * SELL_STEP),
+                         "r"(4 * SELL_STEP)
+                         : "memory");
+        }
       }
-      if (__syncthreads_and(done)) break;
+      if constexpr (ONE) {
+        if (!reduce_one(s, it)) return fail_out(it);
+        if (st[0].done) break;
+      } else {
+        if (!reduce(it == 0 ? NQ : 3, s, it & 1)) return fail_out(it);
+        // one thread per scene (n_scenes <= MS < NTP); the barrier also finds whether all are done
+        int done = 1;
+        if (tid < n_scenes) {
+          if (!st[tid].done)
+            sr_step(st[tid], s_sum[tid][0], s_sum[tid][1], s_sum[tid][2], it == 0 ? s_sum[tid][3] : 0.0f, it,
+                    s_tol2[tid], sl[tid].max_iter);
+          done = st[tid].done;
+        }
+        if (__syncthreads_and(done)) break;
+      }
     }
     // ---- p = u + beta p, s = w + beta s; x += alpha p, r -= alpha s, u = M r (published)
     if constexpr (HALO) {
