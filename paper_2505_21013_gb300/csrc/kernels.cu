@@ -18,6 +18,7 @@
 //   k_energy    per tet and per vertex: incremental potential at u + gamma dx
 //               and g^T dx, FP64 sums (line search, Sec. 5.1)
 //   small vector kernels: predictor, position update, velocity, fallback direction
+#include <algorithm>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -54,17 +55,27 @@ __device__ __forceinline__ void load_u(const double4* U, int v, double* out) {
 }
 
 // ---------------------------------------------------------------- K1 element
+// A warp's tets depend on no other warp's, so a CTA is a warp: EL_CTAS CTAs share a tile.
+// The kernel is bound by its FP64 instructions (a warp's occupies its sub-partition for 64
+// cycles), and the 8-warp CTAs of a small scene kept them on a few SMs.  FP64 scenes that
+// leave sub-partitions idle even so share a tet's ten Hessian blocks out to gridDim.y CTAs
+// (units 2..11 of 12, units 0 and 1 standing for the store of g^e), each repeating the state
+// and g^e: a branch around g^e would save a few microseconds there, but changes the
+// compiler's choice of fused operations, and with it the FP64 bits of every scene.
+// One launch, 256-thread CTAs -> this: 384 tets FP64 57 -> 18.5 us; mixed, 4,350 tets 29 ->
+// 18.7 us, 171,114 tets 87 -> 75 us (the waves end more evenly).
+constexpr int EL_CTAS = TILE / 32;
 template <typename T>
-__global__ void __launch_bounds__(TILE) k_element(const SceneDev<T>* scenes, const TileRef* tiles,
-                                                  int use_probe) {
+__global__ void __launch_bounds__(32) k_element(const SceneDev<T>* scenes, const TileRef* tiles,
+                                                int use_probe) {
   // each 3x3 block goes through shared memory so that a warp writes its 32 tets'
   // blocks as 36-byte runs (one warp store covers ~4 tets, not 32 records)
-  __shared__ T s_blk[TILE / 32][32][9];
-  const TileRef tr = tiles[blockIdx.x];
+  __shared__ T s_blk[32][9];
+  const TileRef tr = tiles[blockIdx.x / EL_CTAS];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int e0 = tr.tile * TILE + wid * 32;  // the warp's first tet
+  const int lane = threadIdx.x, part = blockIdx.y, parts = gridDim.y;
+  const int e0 = tr.tile * TILE + (int)(blockIdx.x % EL_CTAS) * 32;  // the warp's first tet
   if (e0 >= S.nt) return;                    // warp-uniform
   const int e = e0 + lane;
   const bool valid = e < S.nt;
@@ -98,7 +109,8 @@ __global__ void __launch_bounds__(TILE) k_element(const SceneDev<T>* scenes, con
       double pa[3];
       matvec3(Pd, dNd[a], pa);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) ge[3 * a + k] = (double)V * pa[k];
+      for (int k = 0; k < 3; ++k)
+        if (part == 0) ge[3 * a + k] = (double)V * pa[k];
     }
     // Hessian blocks in the storage type
     if constexpr (sizeof(T) == sizeof(double)) {
@@ -122,17 +134,18 @@ __global__ void __launch_bounds__(TILE) k_element(const SceneDev<T>* scenes, con
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = a; b < 4; ++b) {
+      if ((2 + tri4(a, b)) * parts / 12 != part) continue;
       if (valid) {
         T blk[9];
         hess_block(st, V, mu, lam, dN[a], dN[b], cN[a], cN[b], blk);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) s_blk[wid][lane][k] = blk[k];
+        for (int k = 0; k < 9; ++k) s_blk[lane][k] = blk[k];
       }
       __syncwarp();
       const size_t off = (size_t)9 * tri4(a, b);
       for (int j = lane; j < 9 * n_here; j += 32) {
         const int t = j / 9, k = j - 9 * t;
-        S.He[(size_t)(e0 + t) * HE_STRIDE + off + k] = s_blk[wid][t][k];
+        S.He[(size_t)(e0 + t) * HE_STRIDE + off + k] = s_blk[t][k];
       }
       __syncwarp();
     }
@@ -254,6 +267,10 @@ __device__ __forceinline__ void add_elem_block(const T* rec, int a, int b, T* ac
   }
 }
 
+// NT: 32 (no warp needs another's blocks, so that the warps of a small matrix reach more
+// SMs) while the SMs hold all of them at once, 32 CTAs an SM; beyond that TILE, whose CTAs
+// let an SM hold 48 warps: 3.7M blocks take 430 us
+// in it, 443 us in one-warp CTAs; 13,000 blocks 17 us in one-warp CTAs, 18.5 us in it.
 // A warp assembles 32 consecutive blocks from their contribution list (the
 // blocks' (tet, a, b) sources, contiguous in blk_src), 32 contributions at a time:
 // lane l loads contribution c0 + l and its block's place among the warp's 32 (a
@@ -263,15 +280,15 @@ __device__ __forceinline__ void add_elem_block(const T* rec, int a, int b, T* ac
 // order).  Work per warp follows the number of contributions, not the longest
 // block (a diagonal block has ~24, an off-diagonal one ~4-6).  Then lane l writes
 // block k0 + l, with the inertia (and contact) terms on the diagonal.
-template <typename T>
-__global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 6 : 4) k_assemble(const SceneDev<T>* scenes, const TileRef* tiles, int use_probe) {
-  constexpr int NWA = TILE / 32;
-  __shared__ T s_acc[NWA][32][9];
-  const TileRef tr = tiles[blockIdx.x];
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, NT == 32 ? 32 : sizeof(T) == 4 ? 6 : 4)
+    k_assemble(const SceneDev<T>* scenes, const TileRef* tiles, int use_probe) {
+  __shared__ T s_acc[NT / 32][32][9];
+  const TileRef tr = tiles[blockIdx.x / (TILE / NT)];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int k0 = tr.tile * TILE + warp * 32;
+  const int k0 = tr.tile * TILE + (int)(blockIdx.x % (TILE / NT)) * NT + warp * 32;
   if (k0 >= S.nnzb) return;  // warp-uniform
   const int nk = min(32, S.nnzb - k0);
   const int it = S.it_id;
@@ -358,35 +375,67 @@ __global__ void __launch_bounds__(TILE, sizeof(T) == 4 ? 6 : 4) k_assemble(const
   for (int q = 0; q < 9; ++q) S.val[(size_t)q * S.nnzb + k] = acc[q];
 }
 
+// Sums contributions [c0, c1) of a block to acc in order, each formed (He, plus dH if
+// projected) before it is added.  A contribution is loaded while the one before it is
+// added, its source two ahead: at a few warps per SM the loop waits on its loads, at many
+// on its FP64 additions (nine a contribution: He is taken as it is, not added to zeros,
+// which could only turn a -0 into +0, and acc is never -0).
+// VERT: src = 4 tet + corner (a = b), else 16 tet + 4 a + b.
+template <bool VERT = false, typename T>
+__device__ __forceinline__ void sum_contributions(const SceneDev<T>& S, const int* list, int c0, int c1, T* acc) {
+  if (c0 >= c1) return;
+  const int it = S.it_id;
+  auto tet = [](int src) { return src >> (VERT ? 2 : 4); };
+  auto load = [&](const T* recs, int src, T* v) {
+    const int a = VERT ? src & 3 : (src >> 2) & 3, b = src & 3;
+    const T* p = recs + (size_t)tet(src) * HE_STRIDE + 9 * (a <= b ? tri4(a, b) : tri4(b, a));
+    const bool tr = a > b;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v[3 * i + k] = p[tr ? 3 * k + i : 3 * i + k];
+  };
+  int src = list[c0], src_n = c0 + 1 < c1 ? list[c0 + 1] : src;
+  T v[9];
+  load(S.He, src, v);
+  int stamp = S.proj_stamp[tet(src)];
+  for (int c = c0; c < c1; ++c) {
+    const int src_nn = c + 2 < c1 ? list[c + 2] : src_n;
+    T w[9];
+    load(S.He, src_n, w);  // (the last step loads its own block again)
+    const int stamp_n = S.proj_stamp[tet(src_n)];
+    if (stamp == it) {
+      T d[9];
+      load(S.dH, src, d);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) v[q] += d[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      acc[q] += v[q];
+      v[q] = w[q];
+    }
+    src = src_n;
+    src_n = src_nn;
+    stamp = stamp_n;
+  }
+}
+
 // Off-diagonal blocks: a thread per block sums its contributions (the block's (tet, a,
 // b) sources, a != b, in element order) one after another, the next source loaded one
 // step ahead; a contribution is formed (He, plus dH if projected) before it is added.
 // The sums run in the order of the plain per-element scatter.
 template <typename T>
-__device__ __forceinline__ void assemble_offdiag(const SceneDev<T>& S, int tile) {
-  const int k = tile * TILE + (int)threadIdx.x;
+__device__ __forceinline__ void assemble_offdiag(const SceneDev<T>& S, int k) {
   if (k >= S.nnzb) return;
   const int i = S.blk_row[k], j = S.col[k];
   if (i == j) return;  // (the diagonal blocks: assemble_diag)
-  const int it = S.it_id;
   T acc[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) acc[q] = (T)0;
   if (!S.fixed[i] && !S.fixed[j]) {
     const int c0 = S.blk_ptr[k], c1 = S.blk_ptr[k + 1];
-    int src_n = c0 < c1 ? S.blk_src[c0] : 0;
-    for (int c = c0; c < c1; ++c) {
-      const int src = src_n;
-      if (c + 1 < c1) src_n = S.blk_src[c + 1];
-      const int e = src >> 4, a = (src >> 2) & 3, b = src & 3;
-      T v[9];
-#pragma unroll
-      for (int q = 0; q < 9; ++q) v[q] = (T)0;
-      add_elem_block(S.He + (size_t)e * HE_STRIDE, a, b, v);
-      if (S.proj_stamp[e] == it) add_elem_block(S.dH + (size_t)e * HE_STRIDE, a, b, v);
-#pragma unroll
-      for (int q = 0; q < 9; ++q) acc[q] += v[q];
-    }
+    sum_contributions(S, S.blk_src, c0, c1, acc);
   }
 #pragma unroll
   for (int q = 0; q < 9; ++q) S.val[(size_t)q * S.nnzb + k] = acc[q];
@@ -397,8 +446,7 @@ __device__ __forceinline__ void assemble_offdiag(const SceneDev<T>& S, int tile)
 // ahead), then adds the inertia (and contact) terms.  Each contribution is formed as in
 // the off-diagonal form (He, plus dH if projected) before it is added.
 template <typename T>
-__device__ __forceinline__ void assemble_diag(const SceneDev<T>& S, int tile) {
-  const int i = tile * TILE + (int)threadIdx.x;
+__device__ __forceinline__ void assemble_diag(const SceneDev<T>& S, int i) {
   if (i >= S.nv) return;
   const int it = S.it_id;
   const int k = S.diag_idx[i];
@@ -409,19 +457,7 @@ __device__ __forceinline__ void assemble_diag(const SceneDev<T>& S, int tile) {
     acc[0] = acc[4] = acc[8] = (T)1;
   } else {
     const int c0 = S.vt_ptr[i], c1 = S.vt_ptr[i + 1];
-    int src_n = c0 < c1 ? S.vt_src[c0] : 0;  // the next incidence, loaded one step ahead
-    for (int c = c0; c < c1; ++c) {
-      const int src = src_n;
-      if (c + 1 < c1) src_n = S.vt_src[c + 1];
-      const int e = src >> 2, a = src & 3;
-      T v[9];
-#pragma unroll
-      for (int q = 0; q < 9; ++q) v[q] = (T)0;
-      add_elem_block(S.He + (size_t)e * HE_STRIDE, a, a, v);
-      if (S.proj_stamp[e] == it) add_elem_block(S.dH + (size_t)e * HE_STRIDE, a, a, v);
-#pragma unroll
-      for (int q = 0; q < 9; ++q) acc[q] += v[q];
-    }
+    sum_contributions<true>(S, S.vt_src, c0, c1, acc);
     // inertia, and the Dirichlet penalty k m / dt^2 of a constrained vertex
     const T m = (T)(S.mass[i] * S.inv_dt2 * (S.pen_k > 0.0 && S.con[i] ? 1.0 + S.pen_k : 1.0));
     acc[0] += m;
@@ -445,16 +481,19 @@ __device__ __forceinline__ void assemble_diag(const SceneDev<T>& S, int tile) {
 // order, the order of a plain per-element scatter, so that the FP64 matrix follows that
 // reference's rounding; the warp form above is the faster FP32 path.
 template <typename T>
-__global__ void __launch_bounds__(TILE)
-    k_assemble_seq(const SceneDev<T>* scenes, const TileRef* btiles, int n_btiles, const TileRef* vtiles) {
-  const bool off = (int)blockIdx.x < n_btiles;
-  const TileRef tr = off ? btiles[blockIdx.x] : vtiles[blockIdx.x - n_btiles];
+__global__ void __launch_bounds__(32)
+    k_assemble_seq(const SceneDev<T>* scenes, const TileRef* btiles, int n_btiles, const TileRef* vtiles, int n_vtiles) {
+  // (the vertex tiles' warps first: theirs are the long sums)
+  const int b = blockIdx.x / EL_CTAS;
+  const bool off = b >= n_vtiles;
+  const TileRef tr = off ? btiles[b - n_vtiles] : vtiles[b];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
+  const int i = tr.tile * TILE + (int)(blockIdx.x % EL_CTAS) * 32 + (int)threadIdx.x;
   if (off)
-    assemble_offdiag(S, tr.tile);
+    assemble_offdiag(S, i);
   else
-    assemble_diag(S, tr.tile);
+    assemble_diag(S, i);
 }
 
 // ----------------------------------------------------- K6 incremental update
@@ -1130,7 +1169,11 @@ void launch_obst_gap(const SceneDev<T>* s, const TileRef* t, int n, int k0, cuda
 }
 template <typename T>
 void launch_element(const SceneDev<T>* s, const TileRef* t, int n, int probe, cudaStream_t st) {
-  if (n) k_element<T><<<n, TILE, 0, st>>>(s, t, probe);
+  if (!n) return;
+  // FP64: parts while the 4 sub-partitions of each of 152 SMs outnumber the warps
+  const int warps = n * EL_CTAS, fit = sizeof(T) == 8 ? 4 * 152 / warps : 1;
+  const int parts = fit >= 12 ? 12 : fit >= 6 ? 6 : fit >= 1 ? std::min(fit, 4) : 1;
+  k_element<T><<<dim3(warps, parts), 32, 0, st>>>(s, t, probe);
 }
 template <typename T>
 void launch_gradient(const SceneDev<T>* s, const TileRef* t, int n, int probe, cudaStream_t st) {
@@ -1140,9 +1183,12 @@ template <typename T>
 void launch_assemble(const SceneDev<T>* s, const TileRef* bt, int nb, const TileRef* vt, int nv, cudaStream_t st,
                      int use_probe) {
   if constexpr (sizeof(T) == 8) {
-    if (nb + nv) k_assemble_seq<T><<<nb + nv, TILE, 0, st>>>(s, bt, nb, vt);
+    if (nb + nv) k_assemble_seq<T><<<(nb + nv) * EL_CTAS, 32, 0, st>>>(s, bt, nb, vt, nv);
   } else {
-    if (nb) k_assemble<T><<<nb, TILE, 0, st>>>(s, bt, use_probe);
+    if (nb && nb * EL_CTAS <= 32 * 152)
+      k_assemble<T, 32><<<nb * EL_CTAS, 32, 0, st>>>(s, bt, use_probe);
+    else if (nb)
+      k_assemble<T, TILE><<<nb, TILE, 0, st>>>(s, bt, use_probe);
   }
 }
 template <typename T>
