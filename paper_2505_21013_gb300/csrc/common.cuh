@@ -176,68 +176,127 @@ __device__ __forceinline__ void st_d4(double4* p, double4 v) {
   q[1] = make_double2(v.z, v.w);
 }
 
-// fixed-order block reduction of one double per thread (blockDim.x == TILE);
-// result valid in thread 0
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* sm) {
+// FP32 to FP64 by moving bits: a conversion instruction costs an FP64 issue slot (64 cycles
+// of a warp's sub-partition), twelve integer ones about a third of that.  Zeros are handled,
+// denormals, infinities and NaN (any of the N) take the instruction.
+template <int N>
+__device__ __forceinline__ void widen(const float* x, double* d) {
+  bool odd = false;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sm[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (threadIdx.x < NT / 32) ? sm[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  for (int k = 0; k < N; ++k) {
+    const unsigned m = __float_as_uint(x[k]) & 0x7fffffffu;
+    odd |= m != 0u && m - 0x00800000u >= 0x7f000000u;
   }
-  return s;
+  if (odd) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) d[k] = (double)x[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const unsigned b = __float_as_uint(x[k]), m = b & 0x7fffffffu;
+      d[k] = __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
+    }
+  }
 }
-template <int NT>
-__device__ __forceinline__ double block_max(double v, double* sm) {
+template <int N>
+__device__ __forceinline__ void widen(const double* x, double* d) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sm[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (threadIdx.x < NT / 32) ? sm[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_down_sync(0xffffffffu, s, o));
-  }
-  return s;
+  for (int k = 0; k < N; ++k) d[k] = x[k];
 }
 
-// Last-tile finish of a per-scene reduction: every tile has written K partials
-// to part[tile * 4 + k]; the CTA that completes the count sums them in tile
-// order (sum for k < n_sum, max for the rest) and writes out[0..K).
-template <int NT, int K>
-__device__ __forceinline__ void finish_reduction(double* part, unsigned* counter, int n_tiles,
-                                                 int n_sum, double* out, double* sm) {
-  __shared__ int is_last;
+// Fixed-order reductions of K values per thread over a CTA of TILE threads (N_SUM sums, then
+// maxima, which are of values >= 0: negative ones and NaN count as 0).  An FP64 instruction
+// costs a warp 64 cycles however few of its lanes matter, so the sums of a warp share the
+// lanes after their first steps (5 additions for two sums, 6 for four, instead of 5 each),
+// the second stage takes all K values at once, and maxima compare bits as integers.  The
+// sums' tree is that of a shuffle-down per value: offsets 16, 8, 4, 2, 1, twice.
+// Result k in lane 8 k of warp 0; sm: 8 K doubles.
+__device__ __forceinline__ double max_bits(double a, double b) {  // of two results of max_clamp
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return x > y ? a : b;
+}
+__device__ __forceinline__ double max_clamp(double a) {
+  const long long x = __double_as_longlong(a);
+  return x < 0 || x > 0x7ff0000000000000ll ? 0.0 : a;
+}
+template <int K, int N_SUM>
+__device__ __forceinline__ double block_reduce(const double* v, double* sm) {
+  static_assert(TILE == 256 && K <= 4 && N_SUM <= K, "eight warps, four groups of eight lanes");
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  auto xadd = [](double x, int o) { return x + __shfl_xor_sync(0xffffffffu, x, o); };
+  // two sums into one register: lanes with bit o clear go on with a, the others with b
+  auto fold = [&](double a, double b, int o) {
+    return (l & o ? b : a) + __shfl_xor_sync(0xffffffffu, l & o ? a : b, o);
+  };
+  if constexpr (N_SUM > 0) {
+    double x;
+    if constexpr (N_SUM == 1) {
+      x = xadd(xadd(v[0], 16), 8);
+    } else if constexpr (N_SUM == 2) {
+      x = xadd(fold(v[0], v[1], 16), 8);
+    } else {
+      double d = 0.0;
+      if constexpr (N_SUM > 3) d = v[3];
+      x = fold(fold(v[0], v[1], 16), fold(v[2], d, 16), 8);
+    }
+    x = xadd(xadd(xadd(x, 4), 2), 1);
+    const int k = N_SUM == 1 ? l : N_SUM == 2 ? (l >> 4) + (l & 15) * 4 : (l >> 4) + ((l >> 2) & 2) + (l & 7) * 4;
+    if (k < N_SUM) sm[8 * k + w] = x;
+  }
+#pragma unroll
+  for (int k = N_SUM; k < K; ++k) {
+    double x = max_clamp(v[k]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = max_bits(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if (l == 0) sm[8 * k + w] = x;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  double r = 0.0;
+  if (w == 0) {
+    double x = l < 8 * K ? sm[l] : 0.0, m = x;
+    if constexpr (N_SUM > 0) x = xadd(xadd(xadd(x + 0.0, 4), 2), 1);
+    if constexpr (N_SUM < K)
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+    r = l < 8 * N_SUM ? x : m;
+  }
+  return r;
+}
+
+// A per-scene reduction: the CTA writes its tile's K results to part[tile * 4 + k]; the CTA
+// that completes the count reduces them in tile order and writes out[0..K).
+template <int K, int N_SUM>
+__device__ __forceinline__ void scene_reduce(const double* v, double* part, int tile, unsigned* counter, int n_tiles,
+                                             double* out) {
+  __shared__ double sm[8 * K];
+  __shared__ int is_last;
+  const int l = threadIdx.x & 31;
+  const double r = block_reduce<K, N_SUM>(v, sm);
+  if (threadIdx.x < 32) {
+    if (l < 8 * K && (l & 7) == 0) part[4 * tile + (l >> 3)] = r;
     __threadfence();
-    const unsigned done = atomicAdd(counter, 1u);
-    is_last = (done == (unsigned)(n_tiles - 1));
+    __syncwarp();
+    if (l == 0) is_last = atomicAdd(counter, 1u) == (unsigned)(n_tiles - 1);
   }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
+  double acc[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    // thread t sums tiles t, t + NT, ... in order; then a fixed tree
-    double acc = 0.0;
-    for (int t = threadIdx.x; t < n_tiles; t += NT) {
-      const double v = __ldcg(part + 4 * t + k);
-      acc = (k < n_sum) ? acc + v : fmax(acc, v);
+  for (int k = 0; k < K; ++k) acc[k] = 0.0;
+  // thread t takes tiles t, t + TILE, ... in order; then a fixed tree
+  for (int t = threadIdx.x; t < n_tiles; t += TILE) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const double x = __ldcg(part + 4 * t + k);
+      if (k < N_SUM)
+        acc[k] = t < TILE ? x : acc[k] + x;
+      else
+        acc[k] = max_bits(acc[k], x);
     }
-    const double tot = (k < n_sum) ? block_sum<NT>(acc, sm) : block_max<NT>(acc, sm);
-    if (threadIdx.x == 0) out[k] = tot;
   }
+  const double tot = block_reduce<K, N_SUM>(acc, sm);
+  if (threadIdx.x < 32 && l < 8 * K && (l & 7) == 0) out[l >> 3] = tot;
   if (threadIdx.x == 0) *counter = 0u;
 }
 

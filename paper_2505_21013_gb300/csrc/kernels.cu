@@ -89,18 +89,18 @@ __global__ void __launch_bounds__(32) k_element(const SceneDev<T>* scenes, const
     load_u(U, t.y, u[1]);
     load_u(U, t.z, u[2]);
     load_u(U, t.w, u[3]);
-    T W[9];
+    T W[12];
     load_tetc(S.tetc, e, W, V, mu, lam);
+    W[9] = V, W[10] = mu, W[11] = lam;
     // g^e in FP64 in both precisions: the assembled residual drives convergence and
     // selection, and near equilibrium it is a small sum of large element forces
-    double Wd[9], Hd[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Wd[k] = (double)W[k];
+    double Wd[12], Hd[9];
+    widen<12>(W, Wd);
     disp_grad(u[0], u[1], u[2], u[3], Wd, Hd);
     TetState<double> sd;
-    tet_state(Hd, (double)mu, (double)lam, sd);
+    tet_state(Hd, Wd[10], Wd[11], sd);
     double Pd[9];
-    snh_pk1_disp(sd, (double)mu, (double)lam, Pd);
+    snh_pk1_disp(sd, Wd[10], Wd[11], Pd);
     double dNd[4][3];
     shape_grads(Wd, dNd);
     double* ge = S.ge + (size_t)e * GE_STRIDE;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(32) k_element(const SceneDev<T>* scenes, const
       matvec3(Pd, dNd[a], pa);
 #pragma unroll
       for (int k = 0; k < 3; ++k)
-        if (part == 0) ge[3 * a + k] = (double)V * pa[k];
+        if (part == 0) ge[3 * a + k] = Wd[9] * pa[k];
     }
     // Hessian blocks in the storage type
     if constexpr (sizeof(T) == sizeof(double)) {
@@ -155,7 +155,6 @@ __global__ void __launch_bounds__(32) k_element(const SceneDev<T>* scenes, const
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_gradient(const SceneDev<T>* scenes, const TileRef* tiles,
                                                    int use_probe) {
-  __shared__ double sm[32];
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
@@ -172,15 +171,27 @@ __global__ void __launch_bounds__(TILE) k_gradient(const SceneDev<T>* scenes, co
       g[2] = w * (uv.z - uh.z);
       // s: the same terms in magnitude (the rounding scale of g)
       double a[3] = {fabs(g[0]), fabs(g[1]), fabs(g[2])};
-      for (int c = S.vt_ptr[v]; c < S.vt_ptr[v + 1]; ++c) {
-        const int src = S.vt_src[c];
-        const double* ge = S.ge + (size_t)(src >> 2) * GE_STRIDE + 3 * (src & 3);
-        g[0] += ge[0];
-        g[1] += ge[1];
-        g[2] += ge[2];
-        a[0] += fabs(ge[0]);
-        a[1] += fabs(ge[1]);
-        a[2] += fabs(ge[2]);
+      // in order; a corner's force is loaded while the one before it is added, its source
+      // two ahead
+      const int c0 = S.vt_ptr[v], c1 = S.vt_ptr[v + 1];
+      auto force = [&](int src) { return S.ge + (size_t)(src >> 2) * GE_STRIDE + 3 * (src & 3); };
+      int src_n = c0 < c1 ? S.vt_src[c0] : 0;
+      double f[3] = {0.0, 0.0, 0.0};
+      if (c0 < c1) {
+        const double* p = force(src_n);
+        for (int k = 0; k < 3; ++k) f[k] = p[k];
+        if (c0 + 1 < c1) src_n = S.vt_src[c0 + 1];
+      }
+      for (int c = c0; c < c1; ++c) {
+        const double* p = force(src_n);  // (the last step loads its own again)
+        const double n[3] = {p[0], p[1], p[2]};
+        if (c + 2 < c1) src_n = S.vt_src[c + 2];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          g[k] += f[k];
+          a[k] += fabs(f[k]);
+          f[k] = n[k];
+        }
       }
       if (S.pen_k > 0.0 && S.con[v]) {  // Dirichlet penalty potential: k m / dt^2 (u - t)
         const double4 t = ld_d4(S.tgt + v);
@@ -213,17 +224,8 @@ __global__ void __launch_bounds__(TILE) k_gradient(const SceneDev<T>* scenes, co
     n2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
     ninf = m;
   }
-  const double s = block_sum<TILE>(n2, sm);
-  const double ss = block_sum<TILE>(s2, sm);
-  const double cs = block_sum<TILE>(nc, sm);
-  const double mx = block_max<TILE>(ninf, sm);
-  if (threadIdx.x == 0) {
-    S.vpart[4 * tr.tile + 0] = s;
-    S.vpart[4 * tr.tile + 1] = ss;
-    S.vpart[4 * tr.tile + 2] = cs;
-    S.vpart[4 * tr.tile + 3] = mx;
-  }
-  finish_reduction<TILE, 4>(S.vpart, &S.ctl->tiles_done[0], S.n_vtiles, 3, S.ctl->grad, sm);
+  const double red[4] = {n2, s2, nc, ninf};
+  scene_reduce<4, 3>(red, S.vpart, tr.tile, &S.ctl->tiles_done[0], S.n_vtiles, S.ctl->grad);
 }
 
 // ------------------------------------------------------------- K3 assembly
@@ -890,7 +892,6 @@ __global__ void __launch_bounds__(TILE) k_update_contact(const SceneDev<T>* scen
 // filtering of the line search: gamma_ccd = 1 / ctl->ccd)
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_ccd(const SceneDev<T>* scenes, const TileRef* tiles) {
-  __shared__ double sm[32];
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
@@ -903,16 +904,13 @@ __global__ void __launch_bounds__(TILE) k_ccd(const SceneDev<T>* scenes, const T
     const double dx[3] = {(double)d.x, (double)d.y, (double)d.z};
     for (int k = 0; k < S.obs->n; ++k) inv = fmax(inv, 1.0 / obst_ccd(S.obs->o[k], x, dx));
   }
-  const double mx = block_max<TILE>(inv, sm);
-  if (threadIdx.x == 0) S.vpart[4 * tr.tile] = mx;
-  finish_reduction<TILE, 1>(S.vpart, &S.ctl->tiles_done[2], S.n_vtiles, 0, &S.ctl->ccd, sm);
+  scene_reduce<1, 0>(&inv, S.vpart, tr.tile, &S.ctl->tiles_done[2], S.n_vtiles, &S.ctl->ccd);
 }
 
 // smallest distance of a free vertex to obstacles k0..k0+3, reduced as
 // ctl->gap[j] = max 1 / d (+inf when some vertex is not strictly feasible)
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_obst_gap(const SceneDev<T>* scenes, const TileRef* tiles, int k0) {
-  __shared__ double sm[32];
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
@@ -927,13 +925,7 @@ __global__ void __launch_bounds__(TILE) k_obst_gap(const SceneDev<T>* scenes, co
       inv[j] = ok && d > 0.0 ? 1.0 / d : std::numeric_limits<double>::infinity();
     }
   }
-  double mx[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) mx[j] = block_max<TILE>(inv[j], sm);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) S.vpart[4 * tr.tile + j] = mx[j];
-  finish_reduction<TILE, 4>(S.vpart, &S.ctl->tiles_done[3], S.n_vtiles, 0, S.ctl->gap, sm);
+  scene_reduce<4, 0>(inv, S.vpart, tr.tile, &S.ctl->tiles_done[3], S.n_vtiles, S.ctl->gap);
 }
 
 // ---------------------------------------------------------- K10 energy
@@ -943,7 +935,6 @@ __global__ void __launch_bounds__(TILE) k_obst_gap(const SceneDev<T>* scenes, co
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_energy(const SceneDev<T>* scenes, const TileRef* tiles,
                                                  int use_probe) {
-  __shared__ double sm[32];
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
@@ -961,19 +952,21 @@ __global__ void __launch_bounds__(TILE) k_energy(const SceneDev<T>* scenes, cons
         load_u(U, vs[a], u[a]);
         if (gam != 0.0) {
           const vec4_t<T> d = S.dx[vs[a]];
-          u[a][0] += gam * (double)d.x;
-          u[a][1] += gam * (double)d.y;
-          u[a][2] += gam * (double)d.z;
+          const T dt[3] = {d.x, d.y, d.z};
+          double dd3[3];
+          widen<3>(dt, dd3);
+          u[a][0] += gam * dd3[0];
+          u[a][1] += gam * dd3[1];
+          u[a][2] += gam * dd3[2];
         }
       }
-      T Wt[9], Vt, mut, lamt;
-      load_tetc(S.tetc, e, Wt, Vt, mut, lamt);
-      double W[9];
-#pragma unroll
-      for (int k = 0; k < 9; ++k) W[k] = (double)Wt[k];
+      T Wt[12];
+      load_tetc(S.tetc, e, Wt, Wt[9], Wt[10], Wt[11]);
+      double W[12];
+      widen<12>(Wt, W);
       double H[9];
       disp_grad(u[0], u[1], u[2], u[3], W, H);
-      en = (double)Vt * snh_psi_disp(H, (double)mut, (double)lamt);
+      en = W[9] * snh_psi_disp(H, W[10], W[11]);
       if (S.psi_out) S.psi_out[e] = en;
     }
   } else {
@@ -1010,16 +1003,8 @@ __global__ void __launch_bounds__(TILE) k_energy(const SceneDev<T>* scenes, cons
       }
     }
   }
-  const double s0 = block_sum<TILE>(en, sm);
-  const double s1 = block_sum<TILE>(dd, sm);
-  const double s2 = block_max<TILE>(dmax, sm);
-  if (threadIdx.x == 0) {
-    S.tpart[4 * tr.tile + 0] = s0;
-    S.tpart[4 * tr.tile + 1] = s1;
-    S.tpart[4 * tr.tile + 2] = s2;
-  }
-  finish_reduction<TILE, 3>(S.tpart, &S.ctl->tiles_done[1], S.n_ttiles + S.n_vtiles, 2,
-                            S.ctl->energy, sm);
+  const double red[3] = {en, dd, dmax};
+  scene_reduce<3, 2>(red, S.tpart, tr.tile, &S.ctl->tiles_done[1], S.n_ttiles + S.n_vtiles, S.ctl->energy);
 }
 
 // g^T dx and max |dx| over the free vertices into ctl->energy[1], [2] (the line search's
@@ -1027,7 +1012,6 @@ __global__ void __launch_bounds__(TILE) k_energy(const SceneDev<T>* scenes, cons
 // iteration's accepted trial energy, computed at the same displacement bits)
 template <typename T>
 __global__ void __launch_bounds__(TILE) k_dirderiv(const SceneDev<T>* scenes, const TileRef* tiles) {
-  __shared__ double sm[32];
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
@@ -1039,13 +1023,8 @@ __global__ void __launch_bounds__(TILE) k_dirderiv(const SceneDev<T>* scenes, co
     dd = g.x * (double)d.x + g.y * (double)d.y + g.z * (double)d.z;
     dmax = fmax(fabs((double)d.x), fmax(fabs((double)d.y), fabs((double)d.z)));
   }
-  const double s0 = block_sum<TILE>(dd, sm);
-  const double s1 = block_max<TILE>(dmax, sm);
-  if (threadIdx.x == 0) {
-    S.vpart[4 * tr.tile + 0] = s0;
-    S.vpart[4 * tr.tile + 1] = s1;
-  }
-  finish_reduction<TILE, 2>(S.vpart, &S.ctl->tiles_done[4], S.n_vtiles, 1, S.ctl->energy + 1, sm);
+  const double red[2] = {dd, dmax};
+  scene_reduce<2, 1>(red, S.vpart, tr.tile, &S.ctl->tiles_done[4], S.n_vtiles, S.ctl->energy + 1);
 }
 
 // per-vertex |g_v|_inf of a given assembled gradient (selection probe)

@@ -43,3 +43,26 @@ def test_assembly_forms(nz, frac):
     v, vo = sc.probe_assemble(x, proj), o.assemble(x, proj)
     sc.close()
     assert np.abs(v - vo).max() <= 4 * 2e-5 * np.abs(vo).max()  # the mixed stages' tolerance, with projection
+
+
+# vertex and tet counts at the reductions' edges: one warp, tiles of 256 and one more, and
+# more than 256 tiles (several per thread of the finishing CTA)
+@pytest.mark.parametrize("dims", [(2, 2, 3), (4, 8, 8), (5, 4, 13), (41, 40, 41)])
+@pytest.mark.parametrize("prec", [P.PREC_FP64, P.PREC_MIXED])
+def test_gradient_and_energy_reductions(dims, prec):
+    spec = twisting_beam_scene(*dims, h=0.02, E=1e5, nu=0.45, omega=5.0, dt=1 / 30, seed=1)
+    x = deformed(spec, 3)
+    sc = P.Scene.from_spec(spec, precision=prec)
+    g, norms, en = sc.probe_gradient(x, x)  # no inertia: the energy is the tets' alone
+    psi = sc.probe_elements(x)[0]
+    # sums of 64-bit terms by trees of depth < 32 here and in numpy: 64 roundings at most
+    s2 = (g * g).sum()
+    assert abs(norms[0] ** 2 - s2) <= 80 * 1.2e-16 * s2
+    assert norms[1] == np.abs(g).max()
+    assert abs(en - psi.sum()) <= 80 * 1.2e-16 * np.abs(psi).sum()
+    # a vertex that is not a number spoils the sums, and the maximum is of the others
+    y = x.copy()
+    y[np.setdiff1d(np.arange(spec.n_verts), spec.fixed)[0]] = np.nan
+    g, norms, en = sc.probe_gradient(y, x)
+    sc.close()
+    assert np.isnan(norms[0]) and np.isnan(en) and norms[1] == np.nanmax(np.abs(g), initial=0.0)
