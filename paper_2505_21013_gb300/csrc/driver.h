@@ -1494,34 +1494,67 @@ struct Driver {
 
 // ------------------------------------------------------------------ group cache
 
+// Up to two arrays as per-vertex triples (the first plus X when given), into device or
+// pinned host memory.
+template <typename T>
+__global__ void __launch_bounds__(128) k_state_out(const double4* X, const double4* a, double* oa, const double4* b,
+                                                   double* ob, int n) {
+  __shared__ double t[384];
+  const int v0 = blockIdx.x * 128, m = 3 * min(128, n - v0), i = threadIdx.x;
+  const double4* src[2] = {a, b};
+  double* dst[2] = {oa, ob};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (!dst[k]) continue;
+    __syncthreads();
+    if (3 * i < m) {
+      double4 w = ld_d4(src[k] + v0 + i);
+      if (k == 0 && X) {
+        const double4 r = ld_d4(X + v0 + i);
+        w = make_double4(r.x + w.x, r.y + w.y, r.z + w.z, 0.0);
+      }
+      t[3 * i] = w.x;
+      t[3 * i + 1] = w.y;
+      t[3 * i + 2] = w.z;
+    }
+    __syncthreads();
+    for (int j = i; j < m; j += 128) dst[k][3 * (size_t)v0 + j] = t[j];
+  }
+}
+
+// Arrays a (plus X when given) and b into host buffers, either of them null.  A scene of at
+// most IO_VERTS vertices: one kernel writes pinned memory, one wait, and a copy to the
+// caller's pages.  A larger one: through d_xyz and the copy engine, array by array.
+template <typename T>
+inline ppn_status state_out(SceneImpl<T>& s, const double4* X, const double4* a, double* oa, const double4* b,
+                            double* ob) {
+  if (!oa && !ob) return PPN_OK;
+  const int n = s.nv, grid = (n + 127) / 128;
+  const size_t bytes = sizeof(double) * 3 * n;
+  if (n <= s.io_verts) {
+    double *ha = s.h_io, *hb = s.h_io + 3 * (size_t)n;
+    k_state_out<T><<<grid, 128, 0, s.stream>>>(X, a, oa ? ha : nullptr, b, ob ? hb : nullptr, n);
+    PPN_CU(cudaGetLastError());
+    PPN_CU(cudaStreamSynchronize(s.stream));
+    if (oa) std::memcpy(oa, ha, bytes);
+    if (ob) std::memcpy(ob, hb, bytes);
+    return PPN_OK;
+  }
+  for (int k = 0; k < 2; ++k) {
+    double* out = k ? ob : oa;
+    if (!out) continue;
+    k_state_out<T><<<grid, 128, 0, s.stream>>>(k ? nullptr : X, k ? b : a, s.d_xyz, nullptr, nullptr, n);
+    PPN_CU(cudaGetLastError());
+    PPN_CU(cudaMemcpyAsync(out, s.d_xyz, bytes, cudaMemcpyDeviceToHost, s.stream));
+    PPN_CU(cudaStreamSynchronize(s.stream));
+  }
+  return PPN_OK;
+}
+
 // positions x = X + u into a host buffer
 template <typename T>
-__global__ void k_positions(const double4* X, const double4* u, double* xyz, int nv) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= nv) return;
-  const double4 a = ld_d4(X + v), b = ld_d4(u + v);
-  xyz[3 * v] = a.x + b.x;
-  xyz[3 * v + 1] = a.y + b.y;
-  xyz[3 * v + 2] = a.z + b.z;
-}
-
-template <typename T>
-__global__ void k_vel_out(const double4* w, double* xyz, int nv) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= nv) return;
-  const double4 a = ld_d4(w + v);
-  xyz[3 * v] = a.x;
-  xyz[3 * v + 1] = a.y;
-  xyz[3 * v + 2] = a.z;
-}
-
-template <typename T>
 inline ppn_status read_positions(SceneImpl<T>& s, double* out) {
-  k_positions<T><<<(s.nv + 255) / 256, 256, 0, s.stream>>>(s.d.X, s.d.u, s.d_xyz, s.nv);
-  PPN_CU(cudaGetLastError());
-  PPN_CU(cudaMemcpyAsync(out, s.d_xyz, sizeof(double) * 3 * s.nv, cudaMemcpyDeviceToHost, s.stream));
-  PPN_CU(cudaStreamSynchronize(s.stream));
-  return PPN_OK;
+  return state_out(s, s.d.X, s.d.u, out, s.d.vel, nullptr);
 }
 
 }  // namespace ppn

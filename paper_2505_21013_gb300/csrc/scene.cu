@@ -133,7 +133,7 @@ SceneImpl<T>::~SceneImpl() {
   if (stream) cudaStreamSynchronize(stream);
   for (void* p : allocs) dev_free(dalloc, p);
   for (TeamTables& t : team) dev_free(dalloc, t.d_tab);
-  if (h_ctl) cudaFreeHost(h_ctl);
+  if (h_io) cudaFreeHost(h_io);
   if (ev_a) cudaEventDestroy(ev_a);
   if (ev_b) cudaEventDestroy(ev_b);
   if (own_stream && stream) cudaStreamDestroy(stream);
@@ -533,7 +533,8 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
   s.active = 1;
   d = s;
   PPN_CU(up(d_desc, &s, sizeof(SceneDev<T>)));  // for single-scene launches outside a step
-  PPN_CU(cudaMallocHost(&h_ctl, sizeof(Ctl)));
+  io_verts = std::min(nv, IO_VERTS);
+  PPN_CU(cudaMallocHost(&h_io, sizeof(double) * 6 * io_verts));
   int dev = 0;
   PPN_CU(cudaGetDevice(&dev));
   pcg_group = 4;
@@ -619,15 +620,54 @@ static ppn_status step_scenes(const std::vector<SceneImpl<T>*>& members, const i
   return PPN_OK;
 }
 
+// Per-vertex triples from pinned host memory into up to two device arrays.
+__global__ void __launch_bounds__(128) k_state_in(const double* a, double4* da, const double* b, double4* db, int n) {
+  __shared__ double t[384];
+  const int v0 = blockIdx.x * 128, m = 3 * min(128, n - v0), i = threadIdx.x;
+  const double* src[2] = {a, b};
+  double4* dst[2] = {da, db};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (!dst[k]) continue;
+    __syncthreads();
+    for (int j = i; j < m; j += 128) t[j] = src[k][3 * (size_t)v0 + j];
+    __syncthreads();
+    if (3 * i < m) st_d4(dst[k] + v0 + i, make_double4(t[3 * i], t[3 * i + 1], t[3 * i + 2], 0.0));
+  }
+}
+__global__ void k_copy_in(const double* a, double* d, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) d[i] = a[i];
+}
+
+// Host triples a (minus a0 when given) into da and b into db, either of them null: a kernel
+// that reads the pinned copy, and one wait, per io_verts vertices.  (64 scenes of 350 to 10,000
+// vertices, a call for each, both arrays: 2370 us with a pageable copy per array and the waits
+// around it, 1630 us so.)
+template <typename T>
+static ppn_status state_in(SceneImpl<T>& s, const double* a, const double* a0, double4* da, const double* b,
+                           double4* db) {
+  if (!a && !b) return PPN_OK;
+  for (int v0 = 0; v0 < s.nv; v0 += s.io_verts) {
+    const int n = std::min(s.io_verts, s.nv - v0);
+    double *ha = s.h_io, *hb = s.h_io + 3 * (size_t)n;
+    const size_t o = 3 * (size_t)v0;
+    if (a && a0)
+      for (int k = 0; k < 3 * n; ++k) ha[k] = a[o + k] - a0[o + k];
+    else if (a)
+      std::memcpy(ha, a + o, sizeof(double) * 3 * n);
+    if (b) std::memcpy(hb, b + o, sizeof(double) * 3 * n);
+    k_state_in<<<(n + 127) / 128, 128, 0, s.stream>>>(ha, a ? da + v0 : nullptr, hb, b ? db + v0 : nullptr, n);
+    PPN_CU(cudaGetLastError());
+    PPN_CU(cudaStreamSynchronize(s.stream));
+  }
+  return PPN_OK;
+}
+
 // upload host positions as a displacement into `dst` (u = x - X)
 template <typename T>
 static ppn_status upload_positions(SceneImpl<T>& s, const double* x, double4* dst) {
-  std::vector<double4> u(s.nv);
-  for (int v = 0; v < s.nv; ++v)
-    u[v] = make_double4(x[3 * v] - s.rest[3 * v], x[3 * v + 1] - s.rest[3 * v + 1], x[3 * v + 2] - s.rest[3 * v + 2], 0.0);
-  PPN_CU(cudaMemcpyAsync(dst, u.data(), sizeof(double4) * s.nv, cudaMemcpyHostToDevice, s.stream));
-  PPN_CU(cudaStreamSynchronize(s.stream));
-  return PPN_OK;
+  return state_in(s, x, s.rest.data(), dst, nullptr, nullptr);
 }
 
 // ------------------------------------------------------------------ probes
@@ -1049,7 +1089,13 @@ ppn_status ppn_set_kinematic_targets(ppn_scene* s, const double* xyz) {
       set_error("null targets");
       return PPN_ERR_INVALID_ARG;
     }
-    PPN_CU(cudaMemcpyAsync(x.d_targets, xyz, sizeof(double) * 3 * x.nfixed, cudaMemcpyHostToDevice, x.stream));
+    const int n = 3 * x.nfixed;
+    if (n <= 6 * x.io_verts) {
+      std::memcpy(x.h_io, xyz, sizeof(double) * n);
+      k_copy_in<<<(n + 255) / 256, 256, 0, x.stream>>>(x.h_io, x.d_targets, n);
+    } else {
+      PPN_CU(cudaMemcpyAsync(x.d_targets, xyz, sizeof(double) * n, cudaMemcpyHostToDevice, x.stream));
+    }
     // a penalty's targets take effect at once (positions are set at the next step)
     if (x.params.dirichlet_penalty > 0.0)
       launch_apply_targets(x.d_desc, 0, x.d_fixed_list, x.d_targets, x.nfixed, 2, x.stream);
@@ -1261,70 +1307,19 @@ ppn_status ppn_get_attempt_selection(const ppn_scene* s, int idx, int32_t* buf, 
 }
 
 ppn_status ppn_get_state(const ppn_scene* s, double* xo, double* vo) {
-  return dispatch_c(s, [&](auto& x) {
-    if (xo) {
-      ppn_status rc = read_positions(x, xo);
-      if (rc) return rc;
-    }
-    if (vo) {
-      using SI = std::remove_reference_t<decltype(x)>;
-      using TT = typename std::conditional<std::is_same<SI, SceneImpl<float>>::value, float, double>::type;
-      k_vel_out<TT><<<(x.nv + 255) / 256, 256, 0, x.stream>>>(x.d.vel, x.d_xyz, x.nv);
-      PPN_CU(cudaGetLastError());
-      PPN_CU(cudaMemcpyAsync(vo, x.d_xyz, sizeof(double) * 3 * x.nv, cudaMemcpyDeviceToHost, x.stream));
-      PPN_CU(cudaStreamSynchronize(x.stream));
-    }
-    return PPN_OK;
-  });
+  return dispatch_c(s, [&](auto& x) { return state_out(x, x.d.X, x.d.u, xo, x.d.vel, vo); });
 }
 
 ppn_status ppn_set_state(ppn_scene* s, const double* xi, const double* vi) {
-  return dispatch(s, [&](auto& x) {
-    if (xi) {
-      ppn_status rc = upload_positions(x, xi, x.d.u);
-      if (rc) return rc;
-    }
-    if (vi) {
-      std::vector<double4> w(x.nv);
-      for (int v = 0; v < x.nv; ++v) w[v] = make_double4(vi[3 * v], vi[3 * v + 1], vi[3 * v + 2], 0.0);
-      PPN_CU(cudaMemcpy(x.d.vel, w.data(), sizeof(double4) * x.nv, cudaMemcpyHostToDevice));
-    }
-    return PPN_OK;
-  });
+  return dispatch(s, [&](auto& x) { return state_in(x, xi, x.rest.data(), x.d.u, vi, x.d.vel); });
 }
 
 ppn_status ppn_get_displacement(const ppn_scene* s, double* uo, double* vo) {
-  return dispatch_c(s, [&](auto& x) {
-    std::vector<double4> h(x.nv);
-    double* outs[2] = {uo, vo};
-    double4* src[2] = {x.d.u, x.d.vel};
-    PPN_CU(cudaStreamSynchronize(x.stream));
-    for (int k = 0; k < 2; ++k) {
-      if (!outs[k]) continue;
-      PPN_CU(cudaMemcpy(h.data(), src[k], sizeof(double4) * x.nv, cudaMemcpyDeviceToHost));
-      for (int v = 0; v < x.nv; ++v) {
-        outs[k][3 * v] = h[v].x;
-        outs[k][3 * v + 1] = h[v].y;
-        outs[k][3 * v + 2] = h[v].z;
-      }
-    }
-    return PPN_OK;
-  });
+  return dispatch_c(s, [&](auto& x) { return state_out(x, nullptr, x.d.u, uo, x.d.vel, vo); });
 }
 
 ppn_status ppn_set_displacement(ppn_scene* s, const double* ui, const double* vi) {
-  return dispatch(s, [&](auto& x) {
-    std::vector<double4> h(x.nv);
-    const double* ins[2] = {ui, vi};
-    double4* dst[2] = {x.d.u, x.d.vel};
-    PPN_CU(cudaStreamSynchronize(x.stream));
-    for (int k = 0; k < 2; ++k) {
-      if (!ins[k]) continue;
-      for (int v = 0; v < x.nv; ++v) h[v] = make_double4(ins[k][3 * v], ins[k][3 * v + 1], ins[k][3 * v + 2], 0.0);
-      PPN_CU(cudaMemcpy(dst[k], h.data(), sizeof(double4) * x.nv, cudaMemcpyHostToDevice));
-    }
-    return PPN_OK;
-  });
+  return dispatch(s, [&](auto& x) { return state_in(x, ui, nullptr, x.d.u, vi, x.d.vel); });
 }
 
 ppn_status ppn_set_profiling(ppn_scene* s, int on) {

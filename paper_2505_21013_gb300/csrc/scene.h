@@ -88,6 +88,9 @@ enum KernelFamily {
 };
 extern const char* kFamilyNames[FAM_COUNT];
 
+// vertices whose state goes through a scene's pinned buffer at once (at most 768 KB of it)
+constexpr int IO_VERTS = 16384;
+
 template <typename T>
 struct SceneImpl {
   // sizes and parameters
@@ -117,7 +120,9 @@ struct SceneImpl {
   ObstSet* d_obs = nullptr;             // the scene's obstacles as applied (device)
   int n_obst = 0;                       // host copy of their count
   ObstSet obs_app{}, obs_req{};         // applied and requested poses (host)
-  Ctl* h_ctl = nullptr;                 // pinned
+  // pinned, read and written by kernels (state_in/state_out): io_verts x 6 doubles, free between calls
+  double* h_io = nullptr;
+  int io_verts = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   Staging staging;

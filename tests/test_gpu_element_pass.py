@@ -66,3 +66,42 @@ def test_gradient_and_energy_reductions(dims, prec):
     g, norms, en = sc.probe_gradient(y, x)
     sc.close()
     assert np.isnan(norms[0]) and np.isnan(en) and norms[1] == np.nanmax(np.abs(g), initial=0.0)
+
+
+# state in and out: around one CTA's 128 vertices, the pinned buffer's 16384 (a second piece on
+# the way in, the copy engine on the way out), and targets that do not fit the buffer (34848)
+@pytest.mark.parametrize("dims", [(2, 2, 2), (4, 4, 8), (3, 43, 1 + 2), (32, 32, 16), (5, 29, 113), (33, 33, 33)])
+@pytest.mark.parametrize("prec", [P.PREC_FP64, P.PREC_MIXED])
+def test_state_in_and_out(dims, prec):
+    import dataclasses
+    spec = twisting_beam_scene(*dims, h=0.02, E=1e5, nu=0.45, omega=5.0, dt=1 / 30, seed=2)
+    n = spec.n_verts
+    fixed = np.arange(n - dims[0] * dims[1], dtype=np.int32)  # all but the last layer
+    spec = dataclasses.replace(spec, fixed=fixed, targets=None)
+    rng = np.random.default_rng(n)
+    u, v, w = (rng.standard_normal((n, 3)) for _ in range(3))
+    sc = P.Scene.from_spec(spec, precision=prec)
+    sc.set_displacement(u, v)
+    a, b = sc.get_displacement()
+    assert np.array_equal(a, u) and np.array_equal(b, v)
+    X = spec.rest
+    a, b = sc.get_state()
+    assert np.array_equal(a, X + u) and np.array_equal(b, v)
+    sc.set_state(X + w, u)
+    a, b = sc.get_displacement()
+    assert np.array_equal(a, (X + w) - X) and np.array_equal(b, u)
+    # one of the two alone leaves the other as it is
+    L, d = P.ppn.lib(), P.ppn._d
+    assert L.ppn_set_displacement(sc._h, d(w), None) == 0 and L.ppn_set_state(sc._h, None, d(w)) == 0
+    a = np.full((n, 3), 7.0)
+    b = np.full((n, 3), 7.0)
+    assert L.ppn_get_displacement(sc._h, d(a), None) == 0 and L.ppn_get_state(sc._h, None, d(b)) == 0
+    assert np.array_equal(a, w) and np.array_equal(b, w)
+    # targets take effect at the step's start: the fixed vertices end on them
+    sc.set_displacement(np.zeros((n, 3)), np.zeros((n, 3)))
+    t = X[fixed] + 1e-5 * rng.standard_normal((len(fixed), 3))
+    sc.set_targets(t)
+    sc.step(P.MODE_PPN, 1e-2)
+    a = sc.get_displacement()[0]
+    sc.close()
+    assert np.array_equal(a[fixed], t - X[fixed])
