@@ -73,17 +73,19 @@ PPN_HD JRot<T> jrot_params(const T* A) {
   const T apq = r.skip ? (T)1 : r.apq;
   const T tau = (r.aqq - r.app) / ((T)2 * apq);
   const T at = tau < (T)0 ? -tau : tau;
-  T t = at > JacobiCfg<T>::big_tau ? (T)0.5 / at : (T)1 / (at + sqrt((T)1 + at * at));
+  const bool big = at > JacobiCfg<T>::big_tau;
+  T t = (big ? (T)0.5 : (T)1) / (big ? at : at + sqrt((T)1 + at * at));
   if (tau < (T)0) t = -t;
-  r.t = t;
-  r.c = rsqrt_t<T>((T)1 + t * t);
-  r.s = t * r.c;
+  const T c = rsqrt_t<T>((T)1 + t * t);
+  // (a pair that is zero already: the identity, with no branch around its 64 operations)
+  r.t = r.skip ? (T)0 : t;
+  r.c = r.skip ? (T)1 : c;
+  r.s = r.skip ? (T)0 : t * c;
   return r;
 }
 // A <- J^T A J and V <- V J for the rotation of (P, Q); V accumulates the eigenvectors (columns)
 template <typename T, int P, int Q>
 PPN_HD void jrot_apply(T* A, T* V, const JRot<T>& r) {
-  if (r.skip) return;
   const T t = r.t, c = r.c, s = r.s;
   A[s9(P, P)] = r.app - t * r.apq;
   A[s9(Q, Q)] = r.aqq + t * r.apq;

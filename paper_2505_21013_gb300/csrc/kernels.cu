@@ -620,33 +620,52 @@ __global__ void __launch_bounds__(TILE) k_select(const SceneDev<T>* scenes, cons
 }
 
 // ------------------------------------------------------- K5 eigen + clamp
+// A thread per tet; 254 registers, so two warps per scheduler, which wait on arithmetic most
+// of the time.  The ten blocks go out through shared memory, a warp's 32 as 36-byte runs:
+// stored by the threads themselves, words 384 bytes apart, they cost a fifth of the time in
+// waits for the load/store unit.  171,114 tets: 398 us; without the branch around a rotation
+// 344; with one division for the tangent 298 (331 if the threads store).
 template <typename T>
 __global__ void __launch_bounds__(PROJ_CTA) k_project(const SceneDev<T>* scenes, const TileRef* tiles,
                                                       int use_probe) {
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
   if (!S.active) return;
-  const int idx = tr.tile * PROJ_CTA + threadIdx.x;
-  if (idx >= S.ctl->n_new) return;
-  const int e = S.sel_list[idx];
-  const int4 t = S.tets[e];
-  const double4* U = use_probe ? S.u_probe : S.u;
-  double u[4][3];
-  load_u(U, t.x, u[0]);
-  load_u(U, t.y, u[1]);
-  load_u(U, t.z, u[2]);
-  load_u(U, t.w, u[3]);
-  T W[9], V, mu, lam;
-  load_tetc(S.tetc, e, W, V, mu, lam);
-  T H[9];
-  disp_grad(u[0], u[1], u[2], u[3], W, H);
-  TetState<T> st;
-  tet_state(H, mu, lam, st);
+  __shared__ T s_blk[PROJ_CTA / 32][32][9];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int i0 = tr.tile * PROJ_CTA + wid * 32, n = S.ctl->n_new;
+  if (i0 >= n) return;  // warp-uniform
+  const int e = i0 + lane < n ? S.sel_list[i0 + lane] : -1;
   T out[90];
-  clamp_tet(st, W, V, mu, lam, (T)S.eig_eps, S.proj_kind == 1, out);
-  T* dst = S.dH + (size_t)e * HE_STRIDE;
+  if (e >= 0) {
+    const int4 t = S.tets[e];
+    const double4* U = use_probe ? S.u_probe : S.u;
+    double u[4][3];
+    load_u(U, t.x, u[0]);
+    load_u(U, t.y, u[1]);
+    load_u(U, t.z, u[2]);
+    load_u(U, t.w, u[3]);
+    T W[9], V, mu, lam;
+    load_tetc(S.tetc, e, W, V, mu, lam);
+    T H[9];
+    disp_grad(u[0], u[1], u[2], u[3], W, H);
+    TetState<T> st;
+    tet_state(H, mu, lam, st);
+    clamp_tet(st, W, V, mu, lam, (T)S.eig_eps, S.proj_kind == 1, out);
+  }
 #pragma unroll
-  for (int k = 0; k < 90; ++k) dst[k] = out[k];
+  for (int b = 0; b < 10; ++b) {
+    if (e >= 0)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) s_blk[wid][lane][k] = out[9 * b + k];
+    __syncwarp();
+    for (int j = lane; j < 9 * 32; j += 32) {  // (nine rounds, every lane in each)
+      const int t = j / 9, k = j - 9 * t;
+      const int et = __shfl_sync(0xffffffffu, e, t);
+      if (et >= 0) S.dH[(size_t)et * HE_STRIDE + 9 * b + k] = s_blk[wid][t][k];
+    }
+    __syncwarp();
+  }
 }
 
 // K5, warp form, for the few hundred to few thousand tets of a PPN selection round,
@@ -684,7 +703,8 @@ __device__ __forceinline__ void wround(T* a, T* v, int i, int base, bool done) {
   const T apq = skip ? (T)1 : dim;
   const T tau = (dmm - dii) / ((T)2 * apq);
   const T at = tau < (T)0 ? -tau : tau;
-  T t = at > JacobiCfg<T>::big_tau ? (T)0.5 / at : (T)1 / (at + sqrt((T)1 + at * at));
+  const bool big = at > JacobiCfg<T>::big_tau;
+  T t = (big ? (T)0.5 : (T)1) / (big ? at : at + sqrt((T)1 + at * at));
   if (tau < (T)0) t = -t;
   if (skip) t = (T)0;
   const T cs = rsqrt_t<T>((T)1 + t * t);

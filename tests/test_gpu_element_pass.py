@@ -105,3 +105,25 @@ def test_state_in_and_out(dims, prec):
     a = sc.get_displacement()[0]
     sc.close()
     assert np.array_equal(a[fixed], t - X[fixed])
+
+
+# the one-thread-per-tet projection (forced for the short lists too) at the ends of a warp and
+# a CTA, on rest, inverted and clamped tets: the oracle's eigenvalue clamping
+@pytest.mark.parametrize("n_sel", [1, 31, 33, 127, 129, 750])
+@pytest.mark.parametrize("prec", [P.PREC_FP64, P.PREC_MIXED])
+def test_projection_forms(n_sel, prec, monkeypatch):
+    spec = cube_scene(6, seed=3)
+    x = deformed(spec, 4, amp=0.8)
+    x[: spec.n_verts // 3] = spec.rest[: spec.n_verts // 3]  # tets at rest: many zero pairs in the rotations
+    sel = np.sort(np.random.default_rng(n_sel).permutation(spec.n_tets)[:n_sel]).astype(np.int32)
+    mask = np.zeros(spec.n_tets, np.uint8)
+    mask[sel] = 1
+    monkeypatch.setenv("PPN_PROJECT_THREAD", "1")
+    sc, o = P.Scene.from_spec(spec, precision=prec), O.Scene.from_spec(spec, O.default_params())
+    He, dH = sc.probe_elements(x)[2], sc.probe_project(x, sel)
+    v, vo = sc.probe_assemble(x, mask), o.assemble(x, mask)
+    sc.close()
+    tol = 1e-9 if prec == P.PREC_FP64 else 8e-5
+    w = np.linalg.eigvalsh(He[sel] + dH)
+    assert w.min() >= -tol * np.abs(He).max()  # clamped: no negative eigenvalue is left
+    assert np.abs(v - vo).max() <= tol * np.abs(vo).max()
