@@ -247,6 +247,7 @@ struct Group {
     std::memset(c0.data(), 0, sizeof(Ctl) * n);
     for (auto& c : c0) c.pcg_done = 1;
     PPN_CU(cudaMemcpy(d_ctl, c0.data(), sizeof(Ctl) * n, cudaMemcpyHostToDevice));
+    PPN_CU(legacy_done());
     for (int i = 0; i < n; ++i) {
       h_desc[i] = S[i]->d;
       h_desc[i].ctl = d_ctl + i;

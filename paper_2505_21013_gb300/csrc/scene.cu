@@ -544,6 +544,7 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
     set_error("PCG kernel cannot be made co-resident on this device");
     return PPN_ERR_CUDA;
   }
+  PPN_CU(legacy_done());
   return PPN_OK;
 }
 
@@ -776,9 +777,9 @@ static ppn_status read_bsr(SceneImpl<T>& s, double* vals) {
 template <typename T>
 static ppn_status probe_clamp_list(SceneImpl<T>& s, Probe<T>& p, const std::vector<int>& sel) {
   if (sel.empty()) return PPN_OK;
-  PPN_CU(cudaMemcpy(s.d.sel_list, sel.data(), sizeof(int) * sel.size(), cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(s.d.sel_list, sel.data(), sizeof(int) * sel.size(), s.stream));
   const int n = (int)sel.size();
-  PPN_CU(cudaMemcpy(&p.G->d_ctl[0].n_new, &n, sizeof(int), cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(&p.G->d_ctl[0].n_new, &n, sizeof(int), s.stream));
   const bool warp = project_warp_form(true);  // as a PPN selection round
   const int per = warp ? PROJW_TETS : PROJ_CTA;
   std::vector<TileRef> jt;
@@ -824,12 +825,12 @@ static ppn_status probe_select(SceneImpl<T>& s, const double* g, double delta, c
   if (rc) return rc;
   std::vector<double4> g4(s.nv);
   for (int v = 0; v < s.nv; ++v) g4[v] = make_double4(g[3 * v], g[3 * v + 1], g[3 * v + 2], 0.0);
-  PPN_CU(cudaMemcpy(s.d.g, g4.data(), sizeof(double4) * s.nv, cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(s.d.g, g4.data(), sizeof(double4) * s.nv, s.stream));
   std::vector<int> stamp(s.nt, -1);
   if (already)
     for (int e = 0; e < s.nt; ++e)
       if (already[e]) stamp[e] = p.G->h_desc[0].it_id;
-  PPN_CU(cudaMemcpy(s.d.proj_stamp, stamp.data(), sizeof(int) * s.nt, cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(s.d.proj_stamp, stamp.data(), sizeof(int) * s.nt, s.stream));
   p.G->h_desc[0].delta = delta;
   if ((rc = p.G->upload_desc())) return rc;
   PPN_CU(cudaMemsetAsync(&p.G->d_ctl[0].n_new, 0, 3 * sizeof(int), s.stream));  // n_new, n_new_c, n_ties
@@ -892,7 +893,7 @@ static ppn_status probe_pcg(SceneImpl<T>& s, const double* vals, const double* b
   std::vector<T> h((size_t)9 * s.nnzb);
   for (int k = 0; k < s.nnzb; ++k)
     for (int c = 0; c < 9; ++c) h[(size_t)c * s.nnzb + k] = (T)vals[(size_t)9 * k + c];
-  PPN_CU(cudaMemcpy(s.d.val, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(s.d.val, h.data(), sizeof(T) * h.size(), s.stream));
   std::vector<V4> r(s.nv);
   for (int v = 0; v < s.nv; ++v) {
     r[v].x = (T)b[3 * v];
@@ -900,7 +901,7 @@ static ppn_status probe_pcg(SceneImpl<T>& s, const double* vals, const double* b
     r[v].z = (T)b[3 * v + 2];
     r[v].w = (T)0;
   }
-  PPN_CU(cudaMemcpy(s.d.r, r.data(), sizeof(V4) * s.nv, cudaMemcpyHostToDevice));
+  PPN_CU(copy_in(s.d.r, r.data(), sizeof(V4) * s.nv, s.stream));
   p.G->h_desc[0].pcg_tol2 = rel_tol * rel_tol;
   p.G->h_desc[0].pcg_max_iter = max_iter > 0 ? max_iter : s.d.pcg_max_iter;
   Driver<T> D(*p.G);
@@ -1142,8 +1143,7 @@ ppn_status ppn_set_obstacles(ppn_scene* s, const ppn_obstacle* obs, int n) {
     if (!same) x.obs_app = h;
     for (int k = 0; k < n; ++k)
       if (h.o[k].type != PPN_OBST_PLANE) x.obs_app.o[k] = h.o[k];
-    PPN_CU(cudaStreamSynchronize(x.stream));
-    PPN_CU(cudaMemcpy(x.d_obs, &x.obs_app, sizeof(ObstSet), cudaMemcpyHostToDevice));
+    PPN_CU(copy_in(x.d_obs, &x.obs_app, sizeof(ObstSet), x.stream));
     x.n_obst = n;
     return PPN_OK;
   });

@@ -91,6 +91,15 @@ extern const char* kFamilyNames[FAM_COUNT];
 // vertices whose state goes through a scene's pinned buffer at once (at most 768 KB of it)
 constexpr int IO_VERTS = 16384;
 
+// A scene's stream does not wait for the default stream, a memset there returns before it is done,
+// and so may a copy from pageable memory.  What is set up there (a new scene, a group's tables) is
+// waited for before the stream's first kernel; later copies go on the stream itself.
+inline cudaError_t legacy_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+inline cudaError_t copy_in(void* dst, const void* src, size_t n, cudaStream_t st) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+}
+
 template <typename T>
 struct SceneImpl {
   // sizes and parameters
