@@ -1149,7 +1149,20 @@ __global__ void k_fallback_dir(const SceneDev<T>* scenes, const TileRef* tiles, 
   S.dx[v] = d;
 }
 
+// before a selection: the counts of the scenes that take part (one launch, not a memset per scene)
+template <typename T>
+__global__ void k_clear_counts(const SceneDev<T>* scenes, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n || !scenes[i].active) return;
+  Ctl* c = scenes[i].ctl;
+  c->n_new = c->n_new_c = c->n_ties = c->n_touched = 0;
+}
+
 // ---------------------------------------------------------------- launchers
+template <typename T>
+void launch_clear_counts(const SceneDev<T>* s, int n, cudaStream_t st) {
+  k_clear_counts<T><<<(n + 127) / 128, 128, 0, st>>>(s, n);
+}
 template <typename T>
 void launch_select_contact(const SceneDev<T>* s, const TileRef* t, int n, cudaStream_t st) {
   if (n) k_select_contact<T><<<n, TILE, 0, st>>>(s, t);
@@ -1257,6 +1270,7 @@ void launch_fallback(const SceneDev<T>* s, const TileRef* t, int n, int kind, cu
   template void launch_update_touched<T>(const SceneDev<T>*, const TileRef*, int, cudaStream_t); \
   template void launch_select<T>(const SceneDev<T>*, const TileRef*, int, cudaStream_t);       \
   template void launch_project<T>(const SceneDev<T>*, const TileRef*, int, int, cudaStream_t, int); \
+  template void launch_clear_counts<T>(const SceneDev<T>*, int, cudaStream_t);               \
   template void launch_energy<T>(const SceneDev<T>*, const TileRef*, int, int, cudaStream_t);  \
   template void launch_predict<T>(const SceneDev<T>*, const TileRef*, int, cudaStream_t); \
   template void launch_dirderiv<T>(const SceneDev<T>*, const TileRef*, int, cudaStream_t); \

@@ -28,6 +28,7 @@ template <typename T> void launch_project(const SceneDev<T>*, const TileRef*, in
 // the projection form for a selection round (true) or a pass over every element (false),
 // unless PPN_PROJECT_THREAD=1 or PPN_PROJECT_WARP=1 fixes it
 bool project_warp_form(bool selection_round);
+template <typename T> void launch_clear_counts(const SceneDev<T>*, int n_scenes, cudaStream_t);
 template <typename T> void launch_energy(const SceneDev<T>*, const TileRef*, int, int, cudaStream_t);
 template <typename T> void launch_predict(const SceneDev<T>*, const TileRef*, int, cudaStream_t);
 // g^T dx and max |dx| over the free vertices (vertex tiles) into ctl->energy[1], [2]

@@ -1288,6 +1288,19 @@ cudaError_t launch_pcg_team(const SceneDev<float>* scenes, const TeamLaunch& L, 
   return cudaLaunchCooperativeKernel((const void*)k_pcg_team, dim3(L.grid), dim3(NTP), args, L.smem_bytes, st);
 }
 
+// before any other launch: ranges of 8-byte words to zero (blocks (*, k): range k).  One launch
+// for the three or four memsets there were: 17 solves of 32,000 rows 16.60 -> 16.43 ms.
+struct ClearList {
+  int n;
+  void* p[PCG_MAX_SCENES + 3];
+  size_t words[PCG_MAX_SCENES + 3];
+};
+__global__ void k_sr_clear(ClearList c) {
+  unsigned long long* p = reinterpret_cast<unsigned long long*>(c.p[blockIdx.y]);
+  const size_t n = c.words[blockIdx.y];
+  for (size_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) p[k] = 0;
+}
+
 cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cudaStream_t st) {
   const bool halo = L.sr_mode == SR_HALO;
   if (L.n_scenes <= 0 || L.n_scenes > PCG_MAX_SCENES || L.n_tiles <= 0 || L.grid > XCH_MAX_CTAS || !L.flags ||
@@ -1295,20 +1308,20 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
       (halo && (L.n_scenes != 1 || L.n_tiles > NTP || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
                 (L.n_tiles + L.grid - 1) / L.grid * PCG_TILE > SR_HALO_MAX_ROWS)))
     return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(L.bar, 0, sizeof(GridBar), st);
+  // the barrier; flags, exchange words and w records carry stamps of this launch only
+  ClearList c{};
+  auto clear = [&](void* p, size_t bytes) {
+    c.p[c.n] = p;
+    c.words[c.n++] = bytes / 8;
+  };
+  clear(L.bar, sizeof(GridBar));
+  clear(L.flags, sizeof(unsigned long long) * L.grid);
+  for (int k = 0; k < L.n_pword; ++k) clear(L.pword[k], L.pword_bytes[k]);
+  if (halo && !L.zrec[0]) return cudaErrorInvalidValue;
+  if (halo) clear(L.zrec[0], L.zrec_bytes[0]);
+  k_sr_clear<<<dim3(halo ? 64 : 8, c.n), 256, 0, st>>>(c);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // flags and exchange words carry stamps of this launch only
-  e = cudaMemsetAsync(L.flags, 0, sizeof(unsigned long long) * L.grid, st);
-  if (e != cudaSuccess) return e;
-  for (int k = 0; k < L.n_pword; ++k) {
-    e = cudaMemsetAsync(L.pword[k], 0, L.pword_bytes[k], st);
-    if (e != cudaSuccess) return e;
-  }
-  for (int k = 0; halo && k < L.n_scenes; ++k) {
-    if (!L.zrec[k]) return cudaErrorInvalidValue;
-    e = cudaMemsetAsync(L.zrec[k], 0, L.zrec_bytes[k], st);
-    if (e != cudaSuccess) return e;
-  }
   const TileRef* tiles = L.tiles;
   int n_tiles = L.n_tiles;
   const int* ids = L.scene_ids;
