@@ -419,10 +419,8 @@ struct Driver {
       L.halo_col = G.halo_col;
       L.halo_ref = G.halo_ref;
       L.halo_cap = G.halo_cap;
-      for (size_t k = 0; k < sl.size() && k < (size_t)HALO_MAX_SCENES; ++k) {
-        L.zrec[k] = G.h_desc[sl[k]].zrec;
-        L.zrec_bytes[k] = sizeof(T) * 16 * (size_t)G.S[sl[k]]->nv;
-      }
+      L.zrec = G.h_desc[sl[0]].zrec;
+      L.zrec_bytes = 2 * sizeof(float4) * (size_t)G.S[sl[0]]->nv;  // two parity buffers
       const bool tune = G.pcg_sr && G.pcg_tune && ids.size() <= (size_t)PCG_MAX_SCENES;
       L.l2_keep = std::getenv("PPN_PCG_L2_KEEP") ? 1 : 0;
       if (tune) {
@@ -622,11 +620,13 @@ struct Driver {
   }
 
   // Choose the PCG kernel for the launch's tile table.  FP32 (unless
-  // PPN_PCG_STD is set): the single-reduction kernel, with the rows' BSR blocks
-  // and vectors resident in shared memory and the halo replicated when they fit
-  // (unless PPN_PCG_NO_HALO is set), else without the halo, else the vectors
-  // alone, else neither.  Otherwise the standard resident kernel when its
-  // layout fits, else the global-memory kernel.
+  // PPN_PCG_STD is set): a scene alone of at most a row tile per SM takes the
+  // unit kernel of pcg_su.cu; the rest the single-reduction kernel, with the
+  // rows' BSR blocks and vectors resident in shared memory, and one scene's halo
+  // replicated, when they fit (unless PPN_PCG_NO_HALO is set), else without the
+  // halo, else the vectors alone, else neither.  FP64: a scene alone takes the
+  // unit kernel of pcg_rd.cu when it fits.  Otherwise the standard resident
+  // kernel when its layout fits, else the global-memory kernel.
   void plan_smem(const std::vector<int>& sl, const std::vector<TileRef>& tt) {
     G.pcg_smem_bytes = 0;
     G.rd_smem_bytes = 0;

@@ -60,7 +60,7 @@ struct GridBar {
 
 constexpr int PCG_MAX_SCENES = 64;      // scenes per PCG launch (per-CTA scalar state in shared memory)
 constexpr int XCH_MAX_CTAS_HOST = 1024;  // CTAs of one resident PCG launch
-constexpr int HALO_MAX_SCENES = 8;       // scenes per launch of the halo layout (SR_HALO)
+constexpr int HALO_MAX_SCENES = 8;       // scenes of one set of halo tables (SR_HALO launches take one)
 constexpr int HALO_ROW_BITS = 26;        // halo reference: slot << HALO_ROW_BITS | row
 
 struct PcgLaunch {
@@ -86,8 +86,8 @@ struct PcgLaunch {
   const int* halo_col;
   const int* halo_ref;
   int halo_cap;          // most halo rows of one CTA
-  void* zrec[HALO_MAX_SCENES];  // SR_HALO: exchange records of the slots (zeroed before the launch)
-  size_t zrec_bytes[HALO_MAX_SCENES];
+  void* zrec;            // SR_HALO: the scene's w words (zeroed before the launch)
+  size_t zrec_bytes;
   unsigned launch_seq;
   unsigned long long* flags;  // single-reduction kernel: per-CTA publication and progress flags (grid words)
   int n_pword;           // stamped partial arrays to clear before the launch

@@ -31,23 +31,26 @@
 //
 // Synchronisation.  The reduction's tile partials go out as stamped words
 // after the SpMV, into one of two parity buffers, and every CTA sums them in
-// tile order.  Each CTA raises a progress flag with the iteration's stamp as
-// it starts an iteration.  Once a scene of the launch has finished, so that a
-// CTA may have no live tile left to post, the reduction also waits for every
-// CTA's flag.  Either way a buffer is overwritten two iterations later, after
-// every CTA has finished reading it.
+// tile order.  A launch of one scene posts a tile's three sums as one 16-byte
+// word with its stamp, and every CTA posts in every iteration.  A launch of
+// several scenes posts 8-byte words, a value each; once one of its scenes has
+// finished, a CTA may have no live tile left to post, and the reduction then
+// also waits for every CTA's progress flag, raised with the iteration's stamp
+// as the CTA starts it.  Either way a buffer is overwritten two iterations
+// later, after every CTA has finished reading it.
 //   SR_RES, SR_STREAM, SR_GLOBAL: the progress flag also publishes the CTA's
 // u (released by a fence); before its SpMV a CTA waits only for the flags of
 // the CTAs that own the columns of its rows (a contiguous CTA range found at
 // set-up).  One u array suffices: a CTA overwrites it only after it has seen
 // every CTA's partials of the previous iteration, which each CTA posts after
 // finishing the SpMV that read the old values.
-//   SR_HALO: the SpMV stores w of each row as three stamped 64-bit words (the
-// partials' format) in one of two parity buffers; while some warps wait for
-// the reduction's words, the others read the halo rows' w words, each valid
-// once it carries the iteration's stamp.  A buffer is overwritten two
-// iterations later, after every CTA has raised the progress flag that follows
-// its reads.  This leaves one synchronisation per iteration, the reduction.
+//   SR_HALO (launches of one scene, and the teams of k_pcg_team): the SpMV
+// stores w of each row as one 16-byte word of three values and a stamp, in one
+// of two parity buffers; every thread reads the words of its halo rows, each
+// valid once it carries the iteration's stamp, before the tile words that it
+// waits for.  A buffer is overwritten two iterations later: its writer then has
+// the sums of the iteration between, which every CTA posted after its reads.
+// This leaves one synchronisation per iteration, the reduction.
 //
 // All waits are bounded.  Every layout evaluates the same expressions in the
 // same order, through the explicit fused multiply-adds of the helpers below:
@@ -408,9 +411,6 @@ __device__ __forceinline__ bool sr_solve(
   // ---------------- exchange helpers
   // tile words: quantity k of a tile in parity buffer par is
   // pword[((par * NQ + k) * n_ptiles + tile) * pword_stride(n_ptiles)]
-  // SR_HALO: w of the halo rows hb, hb + dh, ... (stamp s, buffer par) into their u slots,
-  // which the SpMV has finished reading; one row at a time (two rows' loads in flight
-  // measured slower in this register-bound kernel)
   // ONE: a tile's 16-byte words in buffer par: gamma, delta, rho; failed blocks (set-up).  A line per
   // tile, or half of one past 512 tiles (the array's size: pword_stride).
   const int tw_step = ONE && sl[0].n_ptiles > 512 ? 4 : 8;
@@ -932,22 +932,15 @@ __device__ __forceinline__ bool sr_solve(
         st_f4(reinterpret_cast<float*>(S.d1 + i), 0.f, 0.f, 0.f);
       } else {
         const int k = 3 * item;
-        if constexpr (HALO) {
-          L.lu4[item] = make_float4(u[0], u[1], u[2], 0.0f);
-        } else {
-          st_f4(u_ptr(S.zrec, i), u[0], u[1], u[2]);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) L.lu[k + c] = u[c];
-        }
+        st_f4(u_ptr(S.zrec, i), u[0], u[1], u[2]);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
+          L.lu[k + c] = u[c];
           L.lr[k + c] = r[c];
           L.lx[k + c] = L.lp[k + c] = L.ls[k + c] = 0.0f;
         }
       }
       fail = ok ? 0.0f : 1.0f;
-    } else if (HALO && item < n_items) {
-      L.lu4[item] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     fail = warp_sum(fail);  // the warp's 32 rows: its first 16-row group takes the count
     if (lane32 == 0) {
@@ -960,7 +953,7 @@ __device__ __forceinline__ bool sr_solve(
     for (int h = tid; h < nh; h += NTP) {
       const int ref = halo_ref[h0 + h];
       L.href[h] = ref;
-      const SceneLite<float>& S = sl[ONE ? 0 : ref >> HALO_ROW_BITS];
+      const SceneLite<float>& S = sl[0];
       const int i = ref & ((1 << HALO_ROW_BITS) - 1);
       float D[9], Pm[9], r[3], u[3];
 #pragma unroll
@@ -1065,17 +1058,9 @@ __device__ __forceinline__ bool sr_solve(
         q[3] = __ldcg(P + 4), q[4] = __ldcg(P + 5), q[5] = __ldcg(P + 8);
       } else {
         const int k = 3 * item;
-        float uo[3];
-        if constexpr (HALO) {
-          const float4 uv = L.lu4[item];
-          uo[0] = uv.x, uo[1] = uv.y, uo[2] = uv.z;
-        } else {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) uo[c] = L.lu[k + c];
-        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          upd_px(a, b, uo[c], L.lp[k + c], L.lx[k + c]);
+          upd_px(a, b, L.lu[k + c], L.lp[k + c], L.lx[k + c]);
           r[c] = L.lr[k + c];
           upd_sr(a, b, L.lw[k + c], L.ls[k + c], r[c]);
           L.lr[k + c] = r[c];
@@ -1084,15 +1069,11 @@ __device__ __forceinline__ bool sr_solve(
         for (int c = 0; c < 6; ++c) q[c] = L.lP[6 * item + c];
       }
       prec6(q, r, u);
-      if constexpr (HALO) {
-        L.lu4[item] = make_float4(u[0], u[1], u[2], 0.0f);
-      } else {
-        if constexpr (!GV) {
+      if constexpr (!GV) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) L.lu[3 * item + c] = u[c];
-        }
-        st_f4(u_ptr(S.zrec, i), u[0], u[1], u[2]);
+        for (int c = 0; c < 3; ++c) L.lu[3 * item + c] = u[c];
       }
+      st_f4(u_ptr(S.zrec, i), u[0], u[1], u[2]);
     }
     // SR_HALO: the halo rows repeat their owners' s, r and u updates with the owners' w
     if constexpr (HALO) {
@@ -1100,9 +1081,7 @@ __device__ __forceinline__ bool sr_solve(
       // is kept rolled (unrolled it measured 1 % slower in this register-bound kernel)
 #pragma unroll 1
       for (int h = tid; h < nh; h += NTP) {
-        const int slot = ONE ? 0 : L.href[h] >> HALO_ROW_BITS;
-        if (st[slot].done) continue;
-        const float a = st[slot].alpha, b = st[slot].beta;
+        const float a = st[0].alpha, b = st[0].beta;
         const float4 wv = L.lu4[n_items + h];
         float r[3], sv[3], q[6], u[3];
 #pragma unroll
@@ -1210,8 +1189,7 @@ cudaError_t launch_wait_probe(const unsigned long long* w, int n, unsigned long 
 // The kernel of a layout; `one`: a launch of a single scene.  The single-scene forms of
 // the layouts without the halo drop the per-scene indexing of their SpMV and update
 // (press, global layout, same-box A/B: 50.1 -> 45.5 us per CG iteration, the same bits).
-// The halo layout keeps one form: its single-scene form measured 4.48 -> 4.66 us on the
-// beam, where the compiler schedules the register-resident rows differently.
+// The halo layout has only this form.
 // `sell`: every scene has room for its blocks by step (the streamed layouts).
 template <int MODE>
 static const void* sr_streamed(bool one, bool sell) {
@@ -1269,7 +1247,7 @@ __global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* j
   const int n_thr = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
   ulonglong2* w = reinterpret_cast<ulonglong2*>(S.pword);
   ulonglong2* z = reinterpret_cast<ulonglong2*>(S.zrec);
-  const int nw = 4 * S.n_ptiles * pword_stride(S.n_ptiles), nz = 4 * S.nv;  // 16-byte pieces
+  const int nw = 4 * S.n_ptiles * pword_stride(S.n_ptiles), nz = 2 * S.nv;  // 16-byte pieces
   for (int k = t0; k < nw; k += n_thr) w[k] = make_ulonglong2(0, 0);
   for (int k = t0; k < nz; k += n_thr) z[k] = make_ulonglong2(0, 0);
 }
@@ -1305,7 +1283,7 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
   const bool halo = L.sr_mode == SR_HALO;
   if (L.n_scenes <= 0 || L.n_scenes > PCG_MAX_SCENES || L.n_tiles <= 0 || L.grid > XCH_MAX_CTAS || !L.flags ||
       L.sr_mode < SR_RES || L.sr_mode > SR_HALO || (L.sr_mode == SR_RES || halo) != (L.smem_blocks > 0) ||
-      (halo && (L.n_scenes != 1 || L.n_tiles > NTP || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
+      (halo && (L.n_scenes != 1 || !L.zrec || L.n_tiles > NTP || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
                 (L.n_tiles + L.grid - 1) / L.grid * PCG_TILE > SR_HALO_MAX_ROWS)))
     return cudaErrorInvalidValue;
   // the barrier; flags, exchange words and w records carry stamps of this launch only
@@ -1317,8 +1295,7 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
   clear(L.bar, sizeof(GridBar));
   clear(L.flags, sizeof(unsigned long long) * L.grid);
   for (int k = 0; k < L.n_pword; ++k) clear(L.pword[k], L.pword_bytes[k]);
-  if (halo && !L.zrec[0]) return cudaErrorInvalidValue;
-  if (halo) clear(L.zrec[0], L.zrec_bytes[0]);
+  if (halo) clear(L.zrec, L.zrec_bytes);
   k_sr_clear<<<dim3(halo ? 64 : 8, c.n), 256, 0, st>>>(c);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
