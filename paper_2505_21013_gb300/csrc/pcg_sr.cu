@@ -103,7 +103,7 @@ struct SrLayout {
   float* lP;     // SR_RES, SR_STREAM: [ni * 6] inverse (00 01 02 11 12 22 of the symmetric block)
   float *lx, *lr, *lu, *lw, *lp, *ls;  // SR_RES, SR_STREAM: [ni * 3] each (SR_HALO: in registers)
   float4* lu4;   // SR_HALO: [ni + nh] u of the own rows, then of the halo rows (w while it arrives)
-  float *hr, *hs, *hP;  // SR_HALO: [nh * 3], [nh * 3], [nh * 6] r, s and inverse of the halo rows
+  float4* hst;   // SR_HALO: [nh * 3] state of the halo rows: r0 r1 r2 s0, s1 s2 and the inverse's first two, its last four
   int* href;     // SR_HALO: [nh] halo rows (slot << HALO_ROW_BITS | row)
   float* ltw;    // SR_HALO: [3][tiles of the scene] sums of the iteration's tile words
 };
@@ -136,9 +136,7 @@ __host__ __device__ inline size_t carve_sr(char* base, int ni, int nb, int nh, i
   }
   if (mode == SR_HALO) {
     l.lu4 = (float4*)take(sizeof(float4) * (ni + nh));
-    l.hr = (float*)take(sizeof(float) * 3 * nh);
-    l.hs = (float*)take(sizeof(float) * 3 * nh);
-    l.hP = (float*)take(sizeof(float) * 6 * nh);
+    l.hst = (float4*)take(sizeof(float4) * 3 * nh);
     l.href = (int*)take(sizeof(int) * nh);
     l.ltw = (float*)take(sizeof(float) * 3 * nt);
   }
@@ -435,7 +433,14 @@ __device__ __forceinline__ bool sr_solve(
   // SR_HALO: the reduction, and meanwhile the halo rows' w.  A tile's three sums come as one 16-byte
   // word: thread t polls tile t's (at most two tiles per CTA: fewer than threads), then every thread its
   // halo rows' words, which are posted earlier; warp 0 sums in tile order (lane-strided, then the tree)
-  // and does the scalar step.
+  // and does the scalar step.  The other warps hold the halo rows, HR a thread, and meanwhile load those
+  // rows' state, so that the update waits for no load (beam 3.75 -> 3.70 us per CG iteration, a
+  // batch of 64 scenes 7.75 -> 7.38 ms per step; loading it in the update, after the step).  Rows past
+  // HR a thread (rare) keep w in their u slot.
+  constexpr int HR = 2, HT = NTP - 32;
+  const int hme = tid - 32;  // the thread's first halo row (none in warp 0)
+  float4 hst[HALO ? HR : 1][3];
+  float hw[HALO ? HR : 1][3];
   auto reduce_halo = [&](unsigned s, int it) -> bool {
     const SceneLite<float>& S = sl[0];
     const int n = S.n_ptiles, par = it & 1;
@@ -451,19 +456,28 @@ __device__ __forceinline__ bool sr_solve(
       L.lu4[n_items + h] = make_float4(__uint_as_float((unsigned)wa), __uint_as_float((unsigned)(wa >> 32)),
                                        __uint_as_float((unsigned)wb), 0.0f);
     };
-#pragma unroll 1
-    for (int h = tid; h < nh; h += 2 * NTP) {
-      const bool two = h + NTP < nh;
-      const int r0 = L.href[h] & ((1 << HALO_ROW_BITS) - 1), r1 = two ? L.href[h + NTP] & ((1 << HALO_ROW_BITS) - 1) : r0;
+    if (hme >= 0 && hme < nh) {
+      const bool two = hme + HT < nh;
+      const int r0 = L.href[hme] & ((1 << HALO_ROW_BITS) - 1), r1 = two ? L.href[hme + HT] & ((1 << HALO_ROW_BITS) - 1) : r0;
       unsigned long long wa, wb, xa, xb;
       ld_word4(zp + r0, wa, wb);
       ld_word4(zp + r1, xa, xb);
       wait4(zp + r0, s, wa, wb, 3, r0);
+      hw[0][0] = __uint_as_float((unsigned)wa);
+      hw[0][1] = __uint_as_float((unsigned)(wa >> 32));
+      hw[0][2] = __uint_as_float((unsigned)wb);
+      if (two) wait4(zp + r1, s, xa, xb, 3, r1);
+      hw[1][0] = __uint_as_float((unsigned)xa);
+      hw[1][1] = __uint_as_float((unsigned)(xa >> 32));
+      hw[1][2] = __uint_as_float((unsigned)xb);
+    }
+#pragma unroll 1
+    for (int h = HR * HT + tid; h < nh; h += NTP) {
+      const int r = L.href[h] & ((1 << HALO_ROW_BITS) - 1);
+      unsigned long long wa, wb;
+      ld_word4(zp + r, wa, wb);
+      wait4(zp + r, s, wa, wb, 3, r);
       halo_put(h, wa, wb);
-      if (two) {
-        wait4(zp + r1, s, xa, xb, 3, r1);
-        halo_put(h + NTP, xa, xb);
-      }
     }
     if (tid < n) {
       wait4(tw, s, a, b, 2, tid);
@@ -477,7 +491,13 @@ __device__ __forceinline__ bool sr_solve(
     }
     __syncthreads();
     if (s_to) return false;
-    if (warp == 0) {
+    if (warp != 0) {
+#pragma unroll
+      for (int k = 0; k < HR; ++k)
+        if (hme + k * HT < nh)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) hst[k][c] = L.hst[3 * (hme + k * HT) + c];
+    } else {
       float acc[3] = {0.0f, 0.0f, 0.0f};
       // (all of a lane's loads issued before its sums: at most NTP / 32 tiles per lane)
       for (int t0 = 0; t0 < n; t0 += 32 * 8) {
@@ -955,20 +975,17 @@ __device__ __forceinline__ bool sr_solve(
       L.href[h] = ref;
       const SceneLite<float>& S = sl[0];
       const int i = ref & ((1 << HALO_ROW_BITS) - 1);
-      float D[9], Pm[9], r[3], u[3];
+      float D[9], Pm[9], q[6], r[3], u[3];
 #pragma unroll
       for (int c = 0; c < 9; ++c) D[c] = S.val[(size_t)c * S.nnzb + S.diag_idx[i]];
       spd_inv3(D, Pm);
-      float* q = L.hP + 6 * h;
       sym6(Pm, q);
       rhs(S, i, r);
       prec6(q, r, u);
       L.lu4[n_items + h] = make_float4(u[0], u[1], u[2], 0.0f);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        L.hr[3 * h + c] = r[c];
-        L.hs[3 * h + c] = 0.0f;
-      }
+      L.hst[3 * h] = make_float4(r[0], r[1], r[2], 0.0f);
+      L.hst[3 * h + 1] = make_float4(0.0f, 0.0f, q[0], q[1]);
+      L.hst[3 * h + 2] = make_float4(q[2], q[3], q[4], q[5]);
     }
   }
 
@@ -1077,30 +1094,26 @@ __device__ __forceinline__ bool sr_solve(
     }
     // SR_HALO: the halo rows repeat their owners' s, r and u updates with the owners' w
     if constexpr (HALO) {
-      // every load of a row issued before its arithmetic (the arrays do not alias); the loop
-      // is kept rolled (unrolled it measured 1 % slower in this register-bound kernel)
-#pragma unroll 1
-      for (int h = tid; h < nh; h += NTP) {
-        const float a = st[0].alpha, b = st[0].beta;
-        const float4 wv = L.lu4[n_items + h];
-        float r[3], sv[3], q[6], u[3];
+      const float a = st[0].alpha, b = st[0].beta;
+      auto halo_update = [&](int h, const float* w, float4 A, float4 B, float4 C) {
+        float r[3] = {A.x, A.y, A.z}, sv[3] = {A.w, B.x, B.y}, u[3];
+        const float q[6] = {B.z, B.w, C.x, C.y, C.z, C.w};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          r[c] = L.hr[3 * h + c];
-          sv[c] = L.hs[3 * h + c];
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) q[c] = L.hP[6 * h + c];
-        upd_sr(a, b, wv.x, sv[0], r[0]);
-        upd_sr(a, b, wv.y, sv[1], r[1]);
-        upd_sr(a, b, wv.z, sv[2], r[2]);
+        for (int c = 0; c < 3; ++c) upd_sr(a, b, w[c], sv[c], r[c]);
         prec6(q, r, u);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          L.hr[3 * h + c] = r[c];
-          L.hs[3 * h + c] = sv[c];
-        }
         L.lu4[n_items + h] = make_float4(u[0], u[1], u[2], 0.0f);
+        L.hst[3 * h] = make_float4(r[0], r[1], r[2], sv[0]);
+        *reinterpret_cast<float2*>(L.hst + 3 * h + 1) = make_float2(sv[1], sv[2]);
+      };
+      if (hme >= 0)
+#pragma unroll
+        for (int k = 0; k < HR; ++k)
+          if (hme + k * HT < nh) halo_update(hme + k * HT, hw[k], hst[k][0], hst[k][1], hst[k][2]);
+#pragma unroll 1
+      for (int h = HR * HT + tid; h < nh; h += NTP) {
+        const float4 wv = L.lu4[n_items + h];
+        const float w[3] = {wv.x, wv.y, wv.z};
+        halo_update(h, w, L.hst[3 * h], L.hst[3 * h + 1], L.hst[3 * h + 2]);
       }
     }
     for (int si = tid; si < n_scenes; si += NTP)

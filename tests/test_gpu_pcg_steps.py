@@ -89,3 +89,21 @@ def test_scenes_in_lockstep_with_retries(form, monkeypatch):
             sc.close()
     assert out[0][0] == out[1][0] and sum(t[2] for step in out[0][0] for t in step) > 0
     assert all(np.array_equal(a, b) for a, b in zip(out[0][1], out[1][1]))
+
+
+# the halo layout's rows of other CTAs: fewer than threads, one and two a thread, and more than that.
+# Vertices numbered at random give a CTA of 128 rows most of a small mesh (896 rows of 1024) or some
+# 1700 rows of a larger one as its halo.
+@pytest.mark.parametrize("dims,shuffled", [((8, 8, 16), False), ((8, 8, 16), True), ((16, 16, 19), True)])
+def test_halo_rows_per_thread(dims, shuffled, monkeypatch):
+    spec = beam(*dims)
+    if shuffled:
+        perm = np.random.default_rng(1).permutation(spec.n_verts)  # new number of each vertex
+        rest = np.empty_like(spec.rest)
+        rest[perm] = spec.rest
+        spec = dataclasses.replace(spec, rest=rest, tets=perm[spec.tets].astype(np.int32),
+                                   fixed=np.sort(perm[spec.fixed]).astype(np.int32), targets=None)
+    monkeypatch.setenv("PPN_PCG_NO_UNITS", "1")
+    a, b = solve(spec, monkeypatch), solve(spec, monkeypatch, "PPN_PCG_NO_HALO")
+    assert (a[2], b[2]) == ("halo", "resident") and a[1] == b[1] and a[1]["iters"] > 20
+    assert np.array_equal(a[0], b[0])
