@@ -620,13 +620,14 @@ __global__ void __launch_bounds__(TILE) k_select(const SceneDev<T>* scenes, cons
 }
 
 // ------------------------------------------------------- K5 eigen + clamp
-// A thread per tet; 254 registers, so two warps per scheduler, which wait on arithmetic most
-// of the time.  The ten blocks go out through shared memory, a warp's 32 as 36-byte runs:
-// stored by the threads themselves, words 384 bytes apart, they cost a fifth of the time in
-// waits for the load/store unit.  171,114 tets: 398 us; without the branch around a rotation
-// 344; with one division for the tangent 298 (331 if the threads store).
+// A thread per tet.  Its warps wait on arithmetic most of the time, so warps in flight are
+// what counts: held to 168 registers (FP32; a few spill), three CTAs an SM instead of two.
+// The ten blocks go out through shared memory, a warp's 32 as 36-byte runs: stored by the
+// threads themselves, words 384 bytes apart, they cost a fifth of the time in waits for the
+// load/store unit.  171,114 tets: 398 us; without the branch around a rotation 344; with one
+// division for the tangent 298 (331 if the threads store); with three CTAs an SM 256.
 template <typename T>
-__global__ void __launch_bounds__(PROJ_CTA) k_project(const SceneDev<T>* scenes, const TileRef* tiles,
+__global__ void __launch_bounds__(PROJ_CTA, sizeof(T) == 4 ? 3 : 1) k_project(const SceneDev<T>* scenes, const TileRef* tiles,
                                                       int use_probe) {
   const TileRef tr = tiles[blockIdx.x];
   const SceneDev<T>& S = scenes[tr.scene];
