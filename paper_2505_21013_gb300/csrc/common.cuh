@@ -274,9 +274,11 @@ __device__ __forceinline__ void scene_reduce(const double* v, double* part, int 
   const double r = block_reduce<K, N_SUM>(v, sm);
   if (threadIdx.x < 32) {
     if (l < 8 * K && (l & 7) == 0) part[4 * tile + (l >> 3)] = r;
-    __threadfence();
     __syncwarp();
-    if (l == 0) is_last = atomicAdd(counter, 1u) == (unsigned)(n_tiles - 1);
+    if (l == 0) {  // the counting lane's fence, after the barrier, covers the other lanes' stores
+      __threadfence();
+      is_last = atomicAdd(counter, 1u) == (unsigned)(n_tiles - 1);
+    }
   }
   __syncthreads();
   if (!is_last) return;

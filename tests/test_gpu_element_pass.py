@@ -68,6 +68,19 @@ def test_gradient_and_energy_reductions(dims, prec):
     assert np.isnan(norms[0]) and np.isnan(en) and norms[1] == np.nanmax(np.abs(g), initial=0.0)
 
 
+# every CTA's partials, stored by several lanes, are there when the last CTA to count sums them:
+# the same bits each time, whichever CTA is the last (794 and 125 tiles)
+def test_reductions_repeat():
+    spec = twisting_beam_scene(20, 20, 80, h=0.02, E=1e5, nu=0.45, omega=5.0, dt=1 / 30, seed=1)
+    x, y = deformed(spec, 3), deformed(spec, 4)
+    sc = P.Scene.from_spec(spec, precision=P.PREC_MIXED)
+    first = {k: sc.probe_gradient(p, spec.rest) for k, p in enumerate((x, y))}
+    for i in range(40):  # in turn, so that a partial left from the call before would show
+        g, norms, en = sc.probe_gradient((x, y)[i % 2], spec.rest)
+        assert np.array_equal(norms, first[i % 2][1]) and en == first[i % 2][2]
+    sc.close()
+
+
 # state in and out: around one CTA's 128 vertices, the pinned buffer's 16384 (a second piece on
 # the way in, the copy engine on the way out), and targets that do not fit the buffer (34848)
 @pytest.mark.parametrize("dims", [(2, 2, 2), (4, 4, 8), (3, 43, 1 + 2), (32, 32, 16), (5, 29, 113), (33, 33, 33)])
