@@ -3,6 +3,8 @@
 // loads, fixed-order reductions and the per-scene CG state.
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -312,6 +314,23 @@ __device__ __forceinline__ void after_rz(SState<R>& s, R rz, R r2, double tol2, 
     s.beta = rz / s.rz;
     s.rz = rz;
   }
+}
+
+// Host: lets kernel k be launched with smem bytes of dynamic shared memory.  The limit is the kernel's, not
+// the launch's or the thread's: it is raised to all that its static shared memory leaves and never
+// lowered, so that a thread that solves a small scene cannot take it from under another's large launch.
+inline cudaError_t allow_shared(const void* k, size_t smem) {
+  cudaFuncAttributes a;
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&a, k);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const int room = most - (int)a.sharedSizeBytes;
+  if (smem > (size_t)std::max(room, 0)) return cudaErrorInvalidValue;
+  return a.maxDynamicSharedSizeBytes == room
+             ? cudaSuccess
+             : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
 }
 
 constexpr int XCH_MAX_CTAS = 1024;  // CTAs of one resident PCG launch (XCH_MAX_CTAS_HOST in kernels.h)

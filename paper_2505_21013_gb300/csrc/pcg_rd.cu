@@ -792,7 +792,7 @@ template <typename T>
 int pcg_rd_max_grid(int device, size_t smem, bool resident) {
   const void* k = rd_kernel<T>(resident);
   int n_sm = 0, per_sm = 0;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_shared(k, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, RD_NT, smem) != cudaSuccess) {
     cudaGetLastError();
@@ -815,7 +815,7 @@ cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const void* k = rd_kernel<T>(L.resident);
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+  e = allow_shared(k, L.smem_bytes);
   if (e != cudaSuccess) return e;
   RdLaunch<T> a = L;
   void* args[] = {(void*)&a};

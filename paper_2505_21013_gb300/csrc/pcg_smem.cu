@@ -546,7 +546,7 @@ static const void* smem_kernel(int) {
 
 int pcg_smem_max_grid(int group, int device, size_t smem, int fsize) {
   const void* k = fsize == 4 ? smem_kernel<float>(group) : smem_kernel<double>(group);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (allow_shared(k, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -581,7 +581,7 @@ cudaError_t launch_pcg_smem(const SceneDev<T>* scenes, const PcgLaunch& L, cudaS
   void* args[] = {(void*)&scenes, (void*)&tiles, (void*)&n_tiles, (void*)&ids, (void*)&n_scenes,
                   (void*)&bar, (void*)&bg, (void*)&nb_cap};
   const void* k = smem_kernel<T>(L.group);
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+  e = allow_shared(k, L.smem_bytes);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(NTS), args, L.smem_bytes, st);
 }

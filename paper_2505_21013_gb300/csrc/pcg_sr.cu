@@ -1220,9 +1220,9 @@ static const void* sr_kernel(int mode, bool one, bool sell) {
 
 int pcg_sr_max_grid(int device, size_t smem, int mode) {
   // (the multi-scene form; the single-scene forms use no more registers or shared memory, so the
-  // same one CTA per SM is co-resident, and the launch sets its own kernel's attribute)
+  // same one CTA per SM is co-resident, and the launch raises its own kernel's limit)
   const void* k = sr_kernel(mode, false, false);  // (SR_HALO: the one form)
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (allow_shared(k, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1237,8 +1237,7 @@ int pcg_sr_max_grid(int device, size_t smem, int mode) {
 }
 
 int pcg_team_max_grid(int device, size_t smem) {
-  if (cudaFuncSetAttribute((const void*)k_pcg_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess) {
+  if (allow_shared((const void*)k_pcg_team, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1270,7 +1269,7 @@ cudaError_t launch_pcg_team(const SceneDev<float>* scenes, const TeamLaunch& L, 
   k_pcg_team_clear<<<dim3(CLEAR_BLOCKS, L.n_jobs), 256, 0, st>>>(scenes, L.jobs, L.bar);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)k_pcg_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+  e = allow_shared((const void*)k_pcg_team, L.smem_bytes);
   if (e != cudaSuccess) return e;
   const TeamJob* jobs = L.jobs;
   int n_jobs = L.n_jobs, bg = L.use_b_from_g;
@@ -1329,7 +1328,7 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
                   (void*)&bar,    (void*)&bg,    (void*)&nb_cap,  (void*)&flags, (void*)&h_off,
                   (void*)&h_col,  (void*)&h_ref, (void*)&nh_cap, (void*)&l2_keep};
   const void* k = sr_kernel(L.sr_mode, L.n_scenes == 1, L.sell != 0);
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+  e = allow_shared(k, L.smem_bytes);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(NTP), args, L.smem_bytes, st);
 }

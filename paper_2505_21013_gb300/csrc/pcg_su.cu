@@ -403,7 +403,7 @@ int pcg_su_hpt(const RdPlan& p, int nh) {
 int pcg_su_max_grid(int device, size_t smem, int rows, int hpt) {
   const void* k = su_kernel(rows, hpt);
   int n_sm = 0, per_sm = 0;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_shared(k, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, SU_NT, smem) != cudaSuccess) {
     cudaGetLastError();
@@ -423,7 +423,7 @@ cudaError_t launch_pcg_su(const SuLaunch& L, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const void* k = su_kernel(p.post_rows, hpt);
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+  e = allow_shared(k, L.smem_bytes);
   if (e != cudaSuccess) return e;
   SuLaunch a = L;
   void* args[] = {(void*)&a};
