@@ -138,7 +138,8 @@ struct Group {
   size_t cap_halo = 0;
   const int *halo_off = nullptr, *halo_col = nullptr, *halo_ref = nullptr;
   int halo_cap = 0;
-  TeamJob* d_jobs = nullptr;  // job table of the team launches
+  TeamJob* d_jobs = nullptr;  // job table of the team launches, and a seat count per job
+  unsigned* d_seats = nullptr;
   size_t cap_jobs = 0;
   GridBar* d_bar = nullptr;   // [2]: of the lockstep and single-scene launches, of the team launches
   cudaStream_t st = nullptr;
@@ -591,13 +592,14 @@ struct Driver {
       s.last_pcg_layout = SR_HALO;
     }
     if (!G.d_jobs || jobs.size() > G.cap_jobs) {
-      G.d_jobs = G.template alloc<TeamJob>(G.cap_n);
+      G.d_jobs = reinterpret_cast<TeamJob*>(G.template alloc<unsigned char>((sizeof(TeamJob) + sizeof(unsigned)) * G.cap_n));
       G.cap_jobs = G.d_jobs ? G.cap_n : 0;
       if (!G.d_jobs) return PPN_OK;  // (the lockstep forms)
+      G.d_seats = reinterpret_cast<unsigned*>(G.d_jobs + G.cap_n);
     }
     ppn_status rc = G.upload(G.d_jobs, jobs.data(), sizeof(TeamJob) * jobs.size());
     if (rc) return rc;
-    TeamLaunch L{G.d_jobs, (int)jobs.size(), G.d_bar + 1, std::min(max_grid, ticket), b_from_g, smem};
+    TeamLaunch L{G.d_jobs, (int)jobs.size(), G.d_seats, G.d_bar + 1, std::min(max_grid, ticket), b_from_g, smem};
     cudaError_t err = cudaSuccess;
     timed(FAM_PCG, 0.0, [&] { err = launch_pcg_team(reinterpret_cast<const SceneDev<float>*>(G.d_desc), L, G.st); });
     if (err != cudaSuccess) {

@@ -51,12 +51,16 @@ struct GridBar {
   unsigned count;      // arrivals, monotonic within a launch
   int timeout;
   unsigned to_iter;    // first timeout: the CG iteration and the wait that ran out
-  int to_site;         // (1 neighbour flags, 2 reduction words, 3 halo w words, 4 progress flags; 0 not recorded)
-  unsigned to_seen;    // the stamp the wait last saw, on the word it waited for
+  int to_site;         // (1 neighbour flags, 2 reduction words, 3 halo w words, 4 progress flags, 6 seats of a team;
+                       // 0 not recorded)
+  unsigned to_seen;    // the stamp the wait last saw, on the word it waited for (site 6: the seats taken)
   int to_slot;         // that word's scene slot and tile (site 2) or row (site 3)
   int to_index;
   int to_cta;
+  unsigned beat;       // team launches: counts on while any team iterates
+  int unused;
 };
+static_assert(sizeof(GridBar) % 8 == 0, "cleared in 8-byte words");
 
 constexpr int PCG_MAX_SCENES = 64;      // scenes per PCG launch (per-CTA scalar state in shared memory)
 constexpr int XCH_MAX_CTAS_HOST = 1024;  // CTAs of one resident PCG launch
@@ -108,6 +112,7 @@ struct TeamJob {
 struct TeamLaunch {
   const TeamJob* jobs;   // device
   int n_jobs;
+  unsigned* seats;       // device, one per job: its members that have set up
   GridBar* bar;
   int grid;              // co-resident CTAs
   int use_b_from_g;

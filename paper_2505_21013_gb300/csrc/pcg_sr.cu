@@ -207,7 +207,7 @@ template <int MODE, bool ONE, bool TEAM, bool SELL>
 __device__ __forceinline__ bool sr_solve(
     int cta, int grid, const SceneDev<float>* scenes, const TileRef* tiles, int n_tiles, const int* scene_ids,
     int n_scenes_arg, GridBar* bar, int b_from_g, int nb_cap, unsigned long long* flags, const int* halo_off,
-    const int* halo_col, const int* halo_ref, int nh_cap, int l2_keep) {
+    const int* halo_col, const int* halo_ref, int nh_cap, int l2_keep, unsigned* seats) {
   static_assert(!TEAM || (ONE && MODE == SR_HALO), "a team solves one scene in the halo layout");
   static_assert(!SELL || MODE == SR_STREAM || MODE == SR_GLOBAL, "only streamed blocks go by steps");
   using W = Words<float>;
@@ -989,8 +989,35 @@ __device__ __forceinline__ bool sr_solve(
     }
   }
 
+  // TEAM: the whole team seated before any wait on another member, whose ticket may only be taken when an
+  // earlier job ends.  That can take as many iterations as the job has (a cap of 100,000 and more), so the
+  // limit of this wait starts anew whenever the launch's beat, which every team's first CTA counts on,
+  // has moved: it runs out only when no team iterates any more.
+  if constexpr (TEAM) {
+    if (tid == 0) {
+      atomicAdd(seats, 1u);
+      unsigned seen = ld_relaxed(&bar->beat), here = ld_relaxed(seats);
+      for (unsigned spins = 0; here < (unsigned)grid; ++spins) {
+        const unsigned beat = ld_relaxed(&bar->beat);
+        if (beat != seen) spins = 0;
+        seen = beat;
+        if (spins > kWaitSpins || *(volatile int*)&bar->timeout) {
+          s_to = 6;
+          s_seen = here;
+          break;
+        }
+        __nanosleep(200);
+        here = ld_relaxed(seats);
+      }
+    }
+    __syncthreads();
+    if (s_to) return fail_out(0);
+  }
+
   for (int it = 0;; ++it) {
     const unsigned s = W::stamp((unsigned)it + 1);
+    if constexpr (TEAM)
+      if (cta == 0 && tid == NTP - 1 && (it & 63) == 0) atomicAdd(&bar->beat, 1u);
     if constexpr (HALO) {
       __syncthreads();  // set-up, or the previous update, before the SpMV
     } else {
@@ -1144,7 +1171,7 @@ __global__ void __launch_bounds__(NTP, 1)
              int n_scenes, GridBar* bar, int b_from_g, int nb_cap, unsigned long long* flags,
              const int* halo_off, const int* halo_col, const int* halo_ref, int nh_cap, int l2_keep) {
   sr_solve<MODE, ONE, false, SELL>((int)blockIdx.x, (int)gridDim.x, scenes, tiles, n_tiles, scene_ids, n_scenes, bar,
-                             b_from_g, nb_cap, flags, halo_off, halo_col, halo_ref, nh_cap, l2_keep);
+                             b_from_g, nb_cap, flags, halo_off, halo_col, halo_ref, nh_cap, l2_keep, nullptr);
 }
 
 // Many scenes, each solved by a team of CTAs of its own, in the halo layout and without any
@@ -1155,22 +1182,27 @@ __global__ void __launch_bounds__(NTP, 1)
 // Tickets: the jobs' members are numbered one job after the other; a free CTA takes the next
 // number (its block index first).  Members of earlier jobs are then always running or done, so a
 // member that waits for its team waits for jobs that finish; all CTAs are co-resident
-// (cooperative launch).  After a timeout no further ticket is taken.
+// (cooperative launch).  That wait (sr_solve's for the seats) is the only one that spans other scenes'
+// solves.  After a timeout no further ticket is taken.
 // Bound, as the halo layout, by an iteration's latency; 64 scenes of 1k to 50k tets (150k rows,
 // 60 to 400 iterations each): 11.9 -> 2.8 ms per solve, 36.6 -> 18.1 ms per time step.
 __global__ void __launch_bounds__(NTP, 1)
-    k_pcg_team(const SceneDev<float>* scenes, const TeamJob* jobs, int n_jobs, GridBar* bar, int b_from_g) {
+    k_pcg_team(const SceneDev<float>* scenes, const TeamJob* jobs, int n_jobs, unsigned* seats, GridBar* bar,
+               int b_from_g) {
   __shared__ TeamJob job;
-  __shared__ int s_ticket;
+  __shared__ int s_ticket, s_job;
   const int n_tickets = jobs[n_jobs - 1].ticket + jobs[n_jobs - 1].size;
   for (int t = (int)blockIdx.x;;) {
     if (t >= n_tickets) return;
     for (int j = threadIdx.x; j < n_jobs; j += NTP)
-      if (jobs[j].ticket <= t && t < jobs[j].ticket + jobs[j].size) job = jobs[j];
+      if (jobs[j].ticket <= t && t < jobs[j].ticket + jobs[j].size) {
+        job = jobs[j];
+        s_job = j;
+      }
     __syncthreads();
     if (!sr_solve<SR_HALO, true, true, false>(t - job.ticket, job.size, scenes, nullptr, job.n_tiles, &job.scene, 1, bar,
                                        b_from_g, job.slots, nullptr, job.halo_off, job.halo_col, job.halo_ref,
-                                       job.halo_cap, 0))
+                                       job.halo_cap, 0, seats + s_job))
       return;
     if (threadIdx.x == 0)
       s_ticket = *(volatile int*)&bar->timeout ? n_tickets : (int)gridDim.x + (int)atomicAdd(&bar->count, 1u);
@@ -1250,11 +1282,12 @@ int pcg_team_max_grid(int device, size_t smem) {
   return per_sm * n_sm;
 }
 
-// before a team launch: the barrier, and every job's exchange words and w records, which carry
+// before a team launch: the barrier, and every job's seats, exchange words and w records, which carry
 // stamps of one launch only, in one launch (blocks (*, j): job j) instead of two memsets per scene
 constexpr int CLEAR_BLOCKS = 8;
-__global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* jobs, GridBar* bar) {
+__global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* jobs, unsigned* seats, GridBar* bar) {
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *bar = GridBar{};
+  if (blockIdx.x == 0 && threadIdx.x == 0) seats[blockIdx.y] = 0;
   const SceneDev<float>& S = scenes[jobs[blockIdx.y].scene];
   const int n_thr = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
   ulonglong2* w = reinterpret_cast<ulonglong2*>(S.pword);
@@ -1265,16 +1298,17 @@ __global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* j
 }
 
 cudaError_t launch_pcg_team(const SceneDev<float>* scenes, const TeamLaunch& L, cudaStream_t st) {
-  if (!L.jobs || L.n_jobs <= 0 || L.grid <= 0 || !L.bar) return cudaErrorInvalidValue;
-  k_pcg_team_clear<<<dim3(CLEAR_BLOCKS, L.n_jobs), 256, 0, st>>>(scenes, L.jobs, L.bar);
+  if (!L.jobs || L.n_jobs <= 0 || L.grid <= 0 || !L.bar || !L.seats) return cudaErrorInvalidValue;
+  k_pcg_team_clear<<<dim3(CLEAR_BLOCKS, L.n_jobs), 256, 0, st>>>(scenes, L.jobs, L.seats, L.bar);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = allow_shared((const void*)k_pcg_team, L.smem_bytes);
   if (e != cudaSuccess) return e;
   const TeamJob* jobs = L.jobs;
   int n_jobs = L.n_jobs, bg = L.use_b_from_g;
+  unsigned* seats = L.seats;
   GridBar* bar = L.bar;
-  void* args[] = {(void*)&scenes, (void*)&jobs, (void*)&n_jobs, (void*)&bar, (void*)&bg};
+  void* args[] = {(void*)&scenes, (void*)&jobs, (void*)&n_jobs, (void*)&seats, (void*)&bar, (void*)&bg};
   return cudaLaunchCooperativeKernel((const void*)k_pcg_team, dim3(L.grid), dim3(NTP), args, L.smem_bytes, st);
 }
 

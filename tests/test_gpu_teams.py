@@ -42,6 +42,30 @@ def run(specs, mode):
     return out, layouts, [(x["newton_iters"], x["total_cg_iters"], x["total_projections"]) for x in st]
 
 
+def test_a_long_solve_before_a_queued_one():
+    # 149 CTAs iterate for more than half a second (150,000 iterations of an ill-conditioned system);
+    # three members of the second team sit and wait meanwhile for CTAs that only then become free
+    params = P.ppn_default_params()
+    params.pcg_rel_tol, params.pcg_max_iter, params.newton_max_iter = 1e-30, 200000, 1
+    long = twisting_beam_scene(9, 9, 470, h=0.02, E=1e6, nu=0.45, omega=4.0, dt=2.0, seed=3)
+    short = twisting_beam_scene(10, 10, 380, h=0.02, E=1e5, nu=0.45, omega=4.0, dt=1 / 30, seed=4)
+    assert long.n_verts > short.n_verts  # (the order of the jobs)
+    out = []
+    for batch in (True, False):
+        scs = [P.Scene.from_spec(s, params=params, precision=P.PREC_MIXED) for s in (long, short)]
+        for sc, s in zip(scs, (long, short)):
+            sc.set_targets(s.targets_at(0))
+        if batch:
+            rc, st = P.ppn_step_batch(scs, [P.MODE_NEWTON] * 2, 1e-9)
+        else:
+            st = [sc.step(P.MODE_NEWTON, 1e-9)[2] for sc in scs]
+        out.append(([(x["status"], x["total_cg_iters"]) for x in st], [sc.get_displacement()[0] for sc in scs]))
+        for sc in scs:
+            sc.close()
+    assert out[0][0] == out[1][0] and out[0][0][0][1] > 100000
+    assert all(np.array_equal(a, b) for a, b in zip(out[0][1], out[1][1]))
+
+
 @pytest.mark.parametrize("name", list(SETS))
 def test_teams_equal_the_lockstep_forms(name, monkeypatch):
     u, layouts, st = run(SETS[name], P.MODE_PPN)
