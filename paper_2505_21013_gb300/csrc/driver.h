@@ -499,56 +499,6 @@ struct Driver {
     return PPN_OK;
   }
 
-  // The halo tables of scene s alone, one or two tiles per CTA (two = 0, 1), built at the scene's
-  // first team launch of that form and kept with it.  False when its rows do not fit.
-  bool team_tables(SceneImpl<T>& s, int two, int n_sm) {
-    auto& t = s.team[two];
-    if (t.state) return t.state > 0;
-    t.state = -1;
-    const int size = two ? (s.n_ptiles + 1) / 2 : s.n_ptiles;
-    if (size > n_sm || s.nv >= (1 << HALO_ROW_BITS)) return false;
-    int slots = 0;  // most block slots of one CTA (as plan_smem counts them)
-    for (int b = 0; b < size; ++b) {
-      const int t0 = (int)(((long long)b * s.n_ptiles) / size), t1 = (int)(((long long)(b + 1) * s.n_ptiles) / size);
-      const int r1 = std::min(s.nv, t1 * PCG_TILE);
-      int n = 0;
-      for (int g = t0 * PCG_TILE; g < r1; g += 16) {
-        int m = 0;
-        for (int r = g; r < std::min(r1, g + 16); ++r) m = std::max(m, (int)(s.h_row_ptr[r + 1] - s.h_row_ptr[r]));
-        n += 32 * ((m + 1) / 2);
-      }
-      slots = std::max(slots, n);
-    }
-    const int rows = (s.n_ptiles + size - 1) / size * PCG_TILE;
-    if (pcg_sr_smem_bytes(rows, slots, 0, s.n_ptiles, SR_HALO) > (size_t)227 * 1024) return false;
-    std::vector<int> tab;
-    const int nh = build_halo_tables({{s.nv, s.h_row_ptr.data(), s.h_col.data()}}, size, tab);
-    if (nh < 0) return false;
-    const size_t smem = pcg_sr_smem_bytes(rows, slots, nh, s.n_ptiles, SR_HALO);
-    // (leaves room for the kernel's static shared memory)
-    if (smem > (size_t)220 * 1024) return false;
-    t.d_tab = (int*)dev_alloc(s.dalloc, sizeof(int) * tab.size());
-    if (!t.d_tab) {
-      cudaGetLastError();
-      t.state = 0;  // (memory may be free again later)
-      return false;
-    }
-    if (cudaMemcpyAsync(t.d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, G.st) != cudaSuccess ||
-        cudaStreamSynchronize(G.st) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    t.size = size;
-    t.slots = slots;
-    t.halo = nh;
-    t.smem = smem;
-    t.off = t.d_tab;
-    t.col = t.d_tab + 2 * (size + 1);
-    t.ref = t.col + tab[2 * size];
-    t.state = 1;
-    return true;
-  }
-
   // A group of scenes: those whose rows fit a team of CTAs go into one team launch (k_pcg_team) and
   // leave `ids`.  Two tiles per CTA use an SM's time best (4.5 us per iteration of two tiles, 3.1
   // of one); one tile per CTA is taken while all scenes' tiles fit the device at once (9 scenes of
@@ -567,7 +517,7 @@ struct Driver {
     std::vector<int> in, out;
     size_t smem = 0;
     for (int i : ids) {
-      if (team_tables(*G.S[i], two, n_sm)) {
+      if (G.S[i]->team[two].size) {
         in.push_back(i);
         smem = std::max(smem, G.S[i]->team[two].smem);
       } else {

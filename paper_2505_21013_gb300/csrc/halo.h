@@ -42,58 +42,62 @@ inline int build_halo_tables(const std::vector<HaloPattern>& pats, int grid, std
   }
   const int n_tiles = toff[ns];
   if (grid < 1 || grid > n_tiles) return -1;
-  std::vector<int> tslot(n_tiles);
-  for (size_t k = 0; k < ns; ++k)
-    for (int t = toff[k]; t < toff[k + 1]; ++t) tslot[t] = (int)k;
   std::vector<std::vector<int>> mark(ns), hidx(ns);
+  size_t n_blocks = 0;
   for (size_t k = 0; k < ns; ++k) {
     mark[k].assign(pats[k].nv, -1);
-    hidx[k].assign(pats[k].nv, 0);
+    hidx[k].resize(pats[k].nv);
+    n_blocks += (size_t)pats[k].row_ptr[pats[k].nv];
   }
-  std::vector<int> off(2 * (grid + 1), 0), col, ref;
-  std::vector<long long> hs;
+  const size_t col0 = 2 * ((size_t)grid + 1), ref0 = col0 + n_blocks;
+  tab.assign(ref0, 0);
+  size_t nc = 0;
+  std::vector<int> hs;
   int maxh = 0;
-  // every block of launch tiles [t0, t1), in the kernel's order: f(slot, column, column's launch tile)
-  auto blocks = [&](int t0, int t1, auto&& f) {
-    for (int t = t0; t < t1; ++t) {
-      const int k = tslot[t];
-      const HaloPattern& p = pats[k];
-      const int r0 = (t - toff[k]) * PCG_TILE, r1 = std::min(p.nv, r0 + PCG_TILE);
-      for (int r = r0; r < r1; ++r)
-        for (int64_t q = p.row_ptr[r]; q < p.row_ptr[r + 1]; ++q) {
-          const int j = p.col[q];
-          f(k, j, toff[k] + j / PCG_TILE);
-        }
-    }
-  };
   for (int b = 0; b < grid; ++b) {
     const int t0 = (int)(((long long)b * n_tiles) / grid), t1 = (int)(((long long)(b + 1) * n_tiles) / grid);
     const int n_items = (t1 - t0) * PCG_TILE;
-    off[2 * b] = (int)col.size();
-    off[2 * b + 1] = (int)ref.size();
-    hs.clear();
-    blocks(t0, t1, [&](int k, int j, int gt) {
-      if ((gt < t0 || gt >= t1) && mark[k][j] != b) {
-        mark[k][j] = b;
-        hs.push_back(((long long)k << 32) | j);
+    tab[2 * b] = (int)nc;
+    tab[2 * b + 1] = (int)(tab.size() - ref0);
+    int nh = 0;
+    // the CTA's run of rows of each slot in turn: columns within it are its own, the others halo rows
+    for (int t = t0, k = (int)(std::upper_bound(toff.begin(), toff.end(), t0) - toff.begin()) - 1; t < t1; ++k) {
+      const HaloPattern& p = pats[k];
+      const int te = std::min(t1, toff[k + 1]);
+      const int r0 = (t - toff[k]) * PCG_TILE, re = (te - toff[k]) * PCG_TILE, item0 = (t - t0) * PCG_TILE;
+      const int64_t q0 = p.row_ptr[r0], q1 = p.row_ptr[std::min(p.nv, re)];
+      int *mk = mark[k].data(), *hx = hidx[k].data(), lo = p.nv, hi = -1;
+      hs.clear();
+      for (int64_t q = q0; q < q1; ++q) {
+        const int j = p.col[q];
+        if ((j < r0 || j >= re) && mk[j] != b) {
+          mk[j] = b;
+          hs.push_back(j);
+          lo = std::min(lo, j);
+          hi = std::max(hi, j);
+        }
       }
-    });
-    std::sort(hs.begin(), hs.end());
-    for (size_t h = 0; h < hs.size(); ++h) {
-      const int k = (int)(hs[h] >> 32), j = (int)(hs[h] & 0xffffffffll);
-      hidx[k][j] = (int)h;
-      ref.push_back((k << HALO_ROW_BITS) | j);
+      if (hi - lo < 16 * (int)hs.size()) {  // ascending: a scan of their range, unless they are few in a wide one
+        size_t n = 0;
+        for (int j = lo; j <= hi; ++j)
+          if (mk[j] == b) hs[n++] = j;
+      } else {
+        std::sort(hs.begin(), hs.end());
+      }
+      for (int j : hs) {
+        hx[j] = nh++;
+        tab.push_back((k << HALO_ROW_BITS) | j);
+      }
+      for (int64_t q = q0; q < q1; ++q) {
+        const int j = p.col[q];
+        tab[col0 + nc++] = j >= r0 && j < re ? item0 + (j - r0) : n_items + hx[j];
+      }
+      t = te;
     }
-    blocks(t0, t1, [&](int k, int j, int gt) {
-      col.push_back(gt >= t0 && gt < t1 ? (gt - t0) * PCG_TILE + j % PCG_TILE : n_items + hidx[k][j]);
-    });
-    maxh = std::max(maxh, (int)hs.size());
+    maxh = std::max(maxh, nh);
   }
-  off[2 * grid] = (int)col.size();
-  off[2 * grid + 1] = (int)ref.size();
-  tab = off;
-  tab.insert(tab.end(), col.begin(), col.end());
-  tab.insert(tab.end(), ref.begin(), ref.end());
+  tab[2 * grid] = (int)nc;
+  tab[2 * grid + 1] = (int)(tab.size() - ref0);
   return maxh;
 }
 

@@ -132,11 +132,55 @@ template <typename T>
 SceneImpl<T>::~SceneImpl() {
   if (stream) cudaStreamSynchronize(stream);
   for (void* p : allocs) dev_free(dalloc, p);
-  for (TeamTables& t : team) dev_free(dalloc, t.d_tab);
   if (h_io) cudaFreeHost(h_io);
   if (ev_a) cudaEventDestroy(ev_a);
   if (ev_b) cudaEventDestroy(ev_b);
   if (own_stream && stream) cudaStreamDestroy(stream);
+}
+
+// The halo tables (build_halo_tables) of both team forms, one after the other in `tab`, and the forms'
+// sizes.  Built with the scene, so that no batch waits for them: for 64 scenes of 2.2 million blocks
+// they take 10 of 484 ms of creation; built by the first batched step they made it 24.1 ms instead of 11.0.
+template <typename T>
+ppn_status SceneImpl<T>::team_plan(std::vector<int>& tab) {
+  int dev = 0, n_sm = 0;
+  PPN_CU(cudaGetDevice(&dev));
+  PPN_CU(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  if (nv >= (1 << HALO_ROW_BITS)) return PPN_OK;
+  std::vector<int> one;
+  for (int two = 0; two < 2; ++two) {
+    TeamTables& t = team[two];
+    const int size = two ? (n_ptiles + 1) / 2 : n_ptiles;
+    if (two && team[0].size == size) {  // a scene of one tile
+      t = team[0];
+      continue;
+    }
+    if (size > n_sm) continue;
+    int slots = 0;  // most block slots of one CTA (as plan_smem counts them)
+    for (int b = 0; b < size; ++b) {
+      const int t0 = (int)(((long long)b * n_ptiles) / size), t1 = (int)(((long long)(b + 1) * n_ptiles) / size);
+      const int r1 = std::min(nv, t1 * PCG_TILE);
+      int n = 0;
+      for (int g = t0 * PCG_TILE; g < r1; g += 16) {
+        int m = 0;
+        for (int r = g; r < std::min(r1, g + 16); ++r) m = std::max(m, (int)(h_row_ptr[r + 1] - h_row_ptr[r]));
+        n += 32 * ((m + 1) / 2);
+      }
+      slots = std::max(slots, n);
+    }
+    const int rows = (n_ptiles + size - 1) / size * PCG_TILE;
+    if (pcg_sr_smem_bytes(rows, slots, 0, n_ptiles, SR_HALO) > (size_t)220 * 1024) continue;
+    const int nh = build_halo_tables({{nv, h_row_ptr.data(), h_col.data()}}, size, one);
+    if (nh < 0) continue;
+    t.smem = pcg_sr_smem_bytes(rows, slots, nh, n_ptiles, SR_HALO);
+    if (t.smem > (size_t)220 * 1024) continue;  // (leaves room for the kernel's static shared memory)
+    t.size = size;
+    t.slots = slots;
+    t.halo = nh;
+    t.word0 = tab.size();
+    tab.insert(tab.end(), one.begin(), one.end());
+  }
+  return PPN_OK;
 }
 
 static std::vector<TileRef> make_tiles(int scene, int n_items, int tile) {
@@ -413,6 +457,12 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
     if (steps * SELL_STEP <= (int64_t)nt * HE_STRIDE) s.steps = s.dH;
   }
   s.gstep = d_gstep;
+  std::vector<int> team_tab;
+  if (sizeof(T) == 4) {
+    const ppn_status rc = team_plan(team_tab);
+    if (rc) return rc;
+  }
+  int* d_team = team_tab.empty() ? nullptr : alloc<int>(team_tab.size());
   s.ctl = alloc<Ctl>(1);
   d_desc = alloc<SceneDev<T>>(1);
   d_ids = alloc<int>(1);
@@ -434,7 +484,7 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
       !d_col || !d_blk_row || !d_blk_ptr || !d_blk_src || !d_blk_lane || !d_diag || !d_tet_blk || !s.blk_mark || !s.touched || !s.u || !s.u_n || !s.vel ||
       !s.uhat || !s.u_probe || !s.ge || !s.He || !s.dH || !s.g || !s.gmax || !s.val ||
       !s.proj_stamp || !s.round_stamp || !s.cproj_stamp || !d_obs || !s.cround_stamp || !s.dHc || !s.Hc || !s.sel_list || !s.dx || !s.r || !s.z || !s.q || !s.d0 ||
-      !s.d1 || !s.Pinv || !s.vpart || !s.tpart || !s.ppart || !s.pword || (sizeof(T) == 4 && (!s.zrec || !d_gstep)) || !s.ctl || !d_desc || !d_ids ||
+      !s.d1 || !s.Pinv || !s.vpart || !s.tpart || !s.ppart || !s.pword || (sizeof(T) == 4 && (!s.zrec || !d_gstep)) || (!team_tab.empty() && !d_team) || !s.ctl || !d_desc || !d_ids ||
       !d_bar || !d_fixed_list || !d_targets || !d_xyz || !d_ttiles || !d_vtiles || !d_btiles ||
       !d_ptiles || !d_etiles || !d_projtiles) {
     set_error("cudaMalloc failed (scene needs more device memory than is free)");
@@ -471,6 +521,13 @@ ppn_status SceneImpl<T>::init(const double* rest_xyz, int64_t n_verts, const int
   }
   PPN_CU(up(d_diag, diag_idx.data(), sizeof(int) * nv));
   if (d_gstep) PPN_CU(up(d_gstep, gstep.data(), sizeof(int) * gstep.size()));
+  if (d_team) PPN_CU(up(d_team, team_tab.data(), sizeof(int) * team_tab.size()));
+  for (TeamTables& t : team)
+    if (t.size) {
+      t.off = d_team + t.word0;
+      t.col = t.off + 2 * (t.size + 1);
+      t.ref = t.col + nnzb;
+    }
   PPN_CU(up(d_tet_blk, blk_of.data(), sizeof(int) * blk_of.size()));
   PPN_CU(cudaMemset(s.blk_mark, 0xff, sizeof(int) * nnzb));
   if (nfixed) {

@@ -138,14 +138,14 @@ struct SceneImpl {
   KernelTimer timer;
   int pcg_group = 8, pcg_grid = 0;
   int last_pcg_layout = -1;  // ppn_scene_info::pcg_layout
-  // halo tables of the scene alone over 1 or 2 tiles per CTA, for team launches (Driver::team_tables)
+  // FP32: halo tables of the scene alone over 1 or 2 tiles per CTA, for team launches (init)
   struct TeamTables {
-    int state = 0;  // 0 not built, 1 usable, -1 does not fit
-    int size = 0, slots = 0, halo = 0;
-    size_t smem = 0;
-    int* d_tab = nullptr;
+    int size = 0;  // CTAs of the team; 0: the rows do not fit that form
+    int slots = 0, halo = 0;
+    size_t smem = 0, word0 = 0;
     const int *off = nullptr, *col = nullptr, *ref = nullptr;
   } team[2];
+  ppn_status team_plan(std::vector<int>& tab);
   int last_cg = 0;  // CG iterations of the scene's last solve (orders the jobs of a team launch)
   // counters and per-step records
   int it_counter = 0, round_counter = 0;

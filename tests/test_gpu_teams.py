@@ -66,6 +66,31 @@ def test_a_long_solve_before_a_queued_one():
     assert all(np.array_equal(a, b) for a, b in zip(out[0][1], out[1][1]))
 
 
+def test_team_tables_come_with_the_scene():
+    # a scene's device memory is allocated at its creation, and device_bytes counts all of it: a
+    # batch's first step, and its later ones, add only the group's own buffers (one dozen)
+    torch = pytest.importorskip("torch")
+    sizes = []
+
+    def alloc(n):
+        sizes.append(n)
+        return torch.cuda.caching_allocator_alloc(n, device=0)
+
+    P.ppn.set_allocator(alloc, torch.cuda.caching_allocator_delete)
+    try:
+        scs = [P.Scene.from_spec(beam(4, 4, 8 + k % 3, k, 10.0 + k), precision=P.PREC_MIXED) for k in range(24)]
+        assert sum(sizes) == sum(sc.info()["device_bytes"] for sc in scs)
+        created = len(sizes)
+        for _ in range(3):
+            assert P.ppn_step_batch(scs, [P.MODE_PPN] * len(scs), 1e-4)[0] == 0
+        assert len(sizes) - created < len(scs)
+        assert sum(sc.info()["device_bytes"] for sc in scs) == sum(sizes[:created])
+        for sc in scs:
+            sc.close()
+    finally:
+        P.ppn.set_allocator(None, None)
+
+
 @pytest.mark.parametrize("name", list(SETS))
 def test_teams_equal_the_lockstep_forms(name, monkeypatch):
     u, layouts, st = run(SETS[name], P.MODE_PPN)
