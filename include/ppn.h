@@ -153,8 +153,9 @@ typedef struct {
   int64_t device_bytes;  /* device memory owned by the scene */
   int precision;
   /* layout of the scene's last linear solve: -1 none yet; FP32 single-reduction
-   * kernel 0 resident, 1 blocks streamed, 2 global vectors, 3 resident with the
-   * halo replicated; 4 the standard resident kernel; 5 the global-memory kernel */
+   * recurrences 0 resident, 1 blocks streamed, 2 global vectors, 3 resident with the
+   * halo replicated; textbook recurrences 4 resident, 5 in global memory.  Several
+   * kernels share layouts 3 and 4: ppn_probe_solver names the one that ran */
   int pcg_layout;
 } ppn_scene_info;
 
@@ -300,6 +301,13 @@ PPN_API ppn_status ppn_probe_project(ppn_scene* s, const double* x, const int32_
                              double* dH);
 /* block-Jacobi PCG on the scene's pattern with values vals (nnzb*9) and right-hand
  * side b (n_verts*3); info: [iterations, ind, precond_fail, hit_max] */
+/* Kernel of the scene's last linear solve: -1 none yet; single-reduction recurrences
+ * (FP32): 0 k_pcg_sr, 1 k_pcg_team (a team of a batch), 2 k_pcg_su (one scene of at most
+ * a row tile per SM); textbook recurrences: 3 k_pcg_rd (32-row units), 4 the same with
+ * the blocks read every iteration (the allocation-free solve), 5 k_pcg_s, 6 k_pcg.
+ * With s NULL, of the calling thread's last ppn_pcg_solve_static. */
+PPN_API ppn_status ppn_probe_solver(const ppn_scene* s, int* kernel);
+
 /* Bounded-wait check (the grid-wide waits of the PCG kernels, Sec. 4.1 "Linear
  * Solvers" runs the solve as one resident kernel): one warp polls n_words stamped
  * 64-bit words in device memory with the PCG's wait routine, at most spin_limit

@@ -440,7 +440,13 @@ struct Driver {
       L.sell = std::getenv("PPN_PCG_NO_STEPS") ? 0 : 1;
       for (int k : sl)
         if (!G.h_desc[k].steps) L.sell = 0;
-      for (int k : sl) G.S[k]->last_pcg_layout = G.pcg_sr ? L.sr_mode : L.smem_bytes ? 4 : 5;
+      for (int k : sl) {
+        G.S[k]->last_pcg_layout = G.pcg_sr ? L.sr_mode : L.smem_bytes ? 4 : 5;
+        G.S[k]->last_solver = G.rd_smem_bytes ? (sizeof(T) == 4 ? SOLVER_SU : SOLVER_RD)
+                              : G.pcg_sr      ? SOLVER_SR
+                              : L.smem_bytes  ? SOLVER_S
+                                              : SOLVER_GLOBAL;
+      }
       L.launch_seq = ++G.pcg_launch_seq;
       L.flags = G.d_flags;
       L.n_pword = (int)sl.size();
@@ -540,6 +546,7 @@ struct Driver {
       jobs.push_back({i, ticket, t.size, s.n_ptiles, t.slots, t.halo, t.off, t.col, t.ref});
       ticket += t.size;
       s.last_pcg_layout = SR_HALO;
+      s.last_solver = SOLVER_TEAM;
     }
     if (!G.d_jobs || jobs.size() > G.cap_jobs) {
       G.d_jobs = reinterpret_cast<TeamJob*>(G.template alloc<unsigned char>((sizeof(TeamJob) + sizeof(unsigned)) * G.cap_n));

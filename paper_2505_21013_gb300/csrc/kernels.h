@@ -99,6 +99,10 @@ struct PcgLaunch {
   size_t pword_bytes[PCG_MAX_SCENES];
 };
 
+// the kernel of a solve, as ppn_probe_solver reports it
+enum Solver { SOLVER_SR, SOLVER_TEAM, SOLVER_SU, SOLVER_RD, SOLVER_RD_READ, SOLVER_S, SOLVER_GLOBAL };
+int static_solver();  // of the calling thread's last allocation-free solve (-1: none yet)
+
 // Team launch (single-reduction kernel, halo layout): every scene of a batch is a job solved by
 // a team of `size` CTAs of its own; the jobs' members are numbered one job after the other.
 struct TeamJob {

@@ -111,6 +111,7 @@ struct DeviceSetup {
   unsigned long long ctx = 0;     // id of the context the address belongs to (0: unknown)
 };
 std::mutex g_lock;
+thread_local int g_solver = -1;
 DeviceSetup g_dev[kMaxDevices];
 
 // id of the calling thread's current context, through the driver's entry points
@@ -173,6 +174,8 @@ ppn_status fail(ppn_status rc, const std::string& msg) {
 }
 
 }  // namespace
+
+int static_solver() { return g_solver; }
 
 }  // namespace ppn
 
@@ -291,6 +294,7 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   L.grid = std::min(D.grid, n_tiles);
   L.group = 4;
   L.use_b_from_g = 0;
+  g_solver = !units ? SOLVER_GLOBAL : R.resident ? SOLVER_RD : SOLVER_RD_READ;
   if (units) {
     R.scene = A.desc;
     R.plan = plan;

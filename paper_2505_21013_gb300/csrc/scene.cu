@@ -1507,6 +1507,18 @@ ppn_status ppn_probe_bounded_wait(int n_words, int spin_limit, int preset) {
   return PPN_OK;
 }
 
+ppn_status ppn_probe_solver(const ppn_scene* s, int* kernel) {
+  if (!kernel) return PPN_ERR_INVALID_ARG;
+  if (!s) {
+    *kernel = ppn::static_solver();
+    return PPN_OK;
+  }
+  return dispatch_c(s, [&](auto& x) {
+    *kernel = x.last_solver;
+    return PPN_OK;
+  });
+}
+
 ppn_status ppn_probe_pcg(ppn_scene* s, const double* vals, const double* b, double rel_tol,
                          int max_iter, double* x, int* info) {
   if (!vals || !b || !x) return PPN_ERR_INVALID_ARG;

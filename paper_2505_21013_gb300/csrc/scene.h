@@ -138,6 +138,7 @@ struct SceneImpl {
   KernelTimer timer;
   int pcg_group = 8, pcg_grid = 0;
   int last_pcg_layout = -1;  // ppn_scene_info::pcg_layout
+  int last_solver = -1;      // ppn_probe_solver
   // FP32: halo tables of the scene alone over 1 or 2 tiles per CTA, for team launches (init)
   struct TeamTables {
     int size = 0;  // CTAs of the team; 0: the rows do not fit that form

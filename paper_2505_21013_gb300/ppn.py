@@ -109,6 +109,8 @@ class ppn_scene_info(C.Structure):
                 ("precision", C.c_int), ("pcg_layout", C.c_int)]
 
 
+# ppn_probe_solver
+SOLVERS = {-1: "none", 0: "sr", 1: "team", 2: "su", 3: "rd", 4: "rd_read", 5: "standard", 6: "standard_global"}
 PCG_LAYOUTS = {-1: "none", 0: "resident", 1: "streamed", 2: "global", 3: "halo", 4: "standard", 5: "standard_global"}
 
 
@@ -159,6 +161,7 @@ SIGNATURES = {
     "ppn_probe_select": (_st, [_P, _pd, C.c_double, _pu, _pu, _pl, _pl]),
     "ppn_probe_project": (_st, [_P, _pd, _pi, C.c_int64, _pd]),
     "ppn_probe_pcg": (_st, [_P, _pd, _pd, C.c_double, C.c_int, _pd, C.POINTER(C.c_int)]),
+    "ppn_probe_solver": (_st, [_P, C.POINTER(C.c_int)]),
     "ppn_probe_bounded_wait": (_st, [C.c_int, C.c_int, C.c_int]),
     "ppn_probe_halo_tables": (_st, [C.c_int, C.POINTER(_pl), C.POINTER(_pi), _pl, C.c_int, _pi, C.c_int64, _pl,
                                     _pi]),
@@ -445,6 +448,10 @@ class Scene:
                "ppn_probe_project")
         return dH
 
+    def probe_solver(self) -> str:
+        """The kernel of the scene's last linear solve (a value of SOLVERS)."""
+        return _solver(self._h)
+
     def probe_pcg(self, vals, b, rel_tol=1e-4, max_iter=0):
         vals = _arr(vals, np.float64)
         b = _arr(b, np.float64)
@@ -527,6 +534,17 @@ def ppn_step_batch(scenes, modes, tol):
     out = (ppn_step_stats * n)()
     rc = lib().ppn_step_batch(arr, n, m, float(tol), out)
     return rc, [struct_dict(out[i]) for i in range(n)]
+
+
+def _solver(handle) -> str:
+    k = C.c_int()
+    _check(lib().ppn_probe_solver(handle, C.byref(k)), "ppn_probe_solver")
+    return SOLVERS[k.value]
+
+
+def pcg_static_solver() -> str:
+    """The kernel of this thread's last pcg_solve_static (a value of SOLVERS)."""
+    return _solver(None)
 
 
 def pcg_solve_static(row_ptr: int, col: int, val: int, n_rows: int, nnzb: int, b: int, x: int,

@@ -120,3 +120,41 @@ def test_allocation_free_solve(dims, monkeypatch):
                                   d_x.data_ptr(), rel_tol=1e-5)
     assert info == info0
     assert np.array_equal(d_x[:, :3].cpu().numpy().astype(np.float64), x0)
+
+
+# the comparisons above are between kernels only if each of them runs: which one does, at every size
+def test_fp64_scenes_run_the_unit_kernel(monkeypatch):
+    for env, want in ((None, "rd"), ("PPN_PCG_NO_UNITS", "standard")):
+        if env:
+            monkeypatch.setenv(env, "1")
+        assert [solver(dims, P.PREC_FP64) for dims in DIMS] == [want] * len(DIMS)
+
+
+def test_mixed_scenes_run_the_unit_kernel(monkeypatch):
+    dims = DIMS + [(16, 19, 32), (16, 16, 76)]
+    assert [solver(d, P.PREC_MIXED) for d in dims + [(16, 16, 77)]] == ["su"] * len(dims) + ["sr"]
+    monkeypatch.setenv("PPN_PCG_NO_UNITS", "1")
+    assert [solver(d, P.PREC_MIXED) for d in dims] == ["sr"] * len(dims)
+
+
+def solver(dims, precision):
+    sc = P.Scene.from_spec(twisting_beam_scene(*dims, h=0.1, seed=3), precision=precision)
+    assert sc.probe_solver() == "none"
+    _, _, _, K, b = springs(dims, 5)
+    sc.probe_pcg(K, b, max_iter=2)
+    name = sc.probe_solver()
+    sc.close()
+    return name
+
+
+def test_allocation_free_solve_runs_the_unit_kernel():
+    dev = torch.device("cuda", 0)
+    for dims, want in [(d, "rd") for d in DIMS + [(20, 20, 80)]] + [((27, 30, 70), "rd_read"), ((32, 32, 64), "rd_read")]:
+        _, rp, col, K, b = springs(dims, 6)
+        n = len(rp) - 1
+        d_rp, d_col = torch.tensor(rp.astype(np.int32), device=dev), torch.tensor(col, device=dev)
+        d_val = torch.tensor(np.ascontiguousarray(K.reshape(-1, 9).T.astype(np.float32)), device=dev)
+        d_x = torch.tensor(np.pad(b, ((0, 0), (0, 1))).astype(np.float32), device=dev)
+        P.ppn.pcg_solve_static(d_rp.data_ptr(), d_col.data_ptr(), d_val.data_ptr(), n, len(col), d_x.data_ptr(),
+                               d_x.data_ptr(), max_iter=2)
+        assert P.ppn.pcg_static_solver() == want, dims

@@ -100,3 +100,36 @@ def test_teams_equal_the_lockstep_forms(name, monkeypatch):
     assert all(np.array_equal(a, b) for a, b in zip(u, u0))
     assert "halo" not in layouts0
     assert [x for x in layouts if x != "halo"] == ([] if name != "too_large" else [layouts[1]])
+
+
+def test_team_exits():
+    # indefinite systems, the iteration cap and a converged solve beside one another: each scene's
+    # step is the one it takes alone (a diagonal block of an elastic energy never fails)
+    params = [P.ppn_default_params() for _ in range(4)]
+    for p in params:
+        p.newton_max_iter = 2
+    params[2].pcg_max_iter = 5
+    specs = [beam(5, 5, 12, 50), beam(5, 6, 12, 51), beam(6, 6, 12, 52), beam(6, 5, 12, 53)]
+    out = []
+    for batch in (True, False):
+        scs = [P.Scene.from_spec(s, params=p, precision=P.PREC_MIXED) for s, p in zip(specs, params)]
+        for sc, s, amp in zip(scs, specs, (3.0, 0.5, 0.0, 0.0)):
+            u = amp * s.meta["h"] * np.random.default_rng(9).standard_normal(s.rest.shape)
+            u[s.fixed] = 0
+            sc.set_displacement(u, np.zeros_like(u))
+            sc.set_targets(s.targets_at(0))
+        if batch:
+            P.ppn_step_batch(scs, [P.MODE_NEWTON] * 4, 1e-9)
+            assert [sc.probe_solver() for sc in scs] == ["team"] * 4
+        else:
+            for sc in scs:
+                sc.step(P.MODE_NEWTON, 1e-9)
+        out.append(([(sc.iter_stats(), sc.attempts()) for sc in scs], [sc.get_displacement()[0] for sc in scs]))
+        for sc in scs:
+            sc.close()
+    (stats, u), (stats1, u1) = out
+    first = [a[0] for _, a in stats]
+    assert [bool(a["ind"]) for a in first] == [True, True, False, False]
+    assert first[2]["cg_iters"] == 5 and first[3]["cg_iters"] > 5
+    assert repr(stats) == repr(stats1)
+    assert all(np.array_equal(a, b) for a, b in zip(u, u1))
