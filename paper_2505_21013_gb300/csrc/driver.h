@@ -468,6 +468,9 @@ struct Driver {
             U.bar = G.d_bar;
             U.words = reinterpret_cast<float4*>(G.h_desc[sl[0]].pword);
             U.smem_bytes = G.rd_smem_bytes;
+            // (PPN_PCG_WAIT_LIMIT: a short limit that runs out; tests)
+            const char* limit = std::getenv("PPN_PCG_WAIT_LIMIT");
+            U.wait_limit = limit ? (unsigned)std::min<long>(std::max<long>(std::atol(limit), 0), PCG_WAIT_LIMIT) : PCG_WAIT_LIMIT;
             err = launch_pcg_su(U, G.st);
             return;
           }

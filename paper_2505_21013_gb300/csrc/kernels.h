@@ -54,14 +54,15 @@ struct GridBar {
   int to_site;         // (1 neighbour flags, 2 reduction words, 3 halo w words, 4 progress flags, 6 seats of a team;
                        // 0 not recorded)
   unsigned to_seen;    // the stamp the wait last saw, on the word it waited for (site 6: the seats taken)
-  int to_slot;         // that word's scene slot and tile (site 2) or row (site 3)
-  int to_index;
+  int to_slot;         // that word's scene slot,
+  int to_index;        // and its tile (site 2; k_pcg_su: post) or row (site 3); k_pcg_su: -1 if it came just after
   int to_cta;
   unsigned beat;       // team launches: counts on while any team iterates
   int unused;
 };
 static_assert(sizeof(GridBar) % 8 == 0, "cleared in 8-byte words");
 
+constexpr unsigned PCG_WAIT_LIMIT = 1u << 20;  // bound of one wait, in polling rounds
 constexpr int PCG_MAX_SCENES = 64;      // scenes per PCG launch (per-CTA scalar state in shared memory)
 constexpr int XCH_MAX_CTAS_HOST = 1024;  // CTAs of one resident PCG launch
 constexpr int HALO_MAX_SCENES = 8;       // scenes of one set of halo tables (SR_HALO launches take one)
@@ -193,6 +194,7 @@ struct SuLaunch {
   GridBar* bar;
   float4* words;                 // 16 words of 16 bytes per post
   size_t smem_bytes;
+  unsigned wait_limit;           // of each wait, in polls
 };
 size_t pcg_su_smem_bytes(const RdPlan& p, int slots, int halo);
 int pcg_su_hpt(const RdPlan& p, int halo);  // halo rows per thread; 0: does not fit

@@ -160,8 +160,8 @@ __device__ __forceinline__ float* rec_ptr(float* base, int nv, int parity, int i
   return base + ((size_t)parity * nv + i) * 8;
 }
 
-// bound of one wait, in polling rounds; a CTA that gives up flags a timeout
-constexpr unsigned kWaitSpins = 1u << 20;
+// bound of one wait; a CTA that gives up flags a timeout
+constexpr unsigned kWaitSpins = PCG_WAIT_LIMIT;
 
 // One warp polls the stamped words W[LO..HI] (four per lane per round, LANE the
 // lane index) until each is >= STAMP.  It gives up after LIMIT rounds on some

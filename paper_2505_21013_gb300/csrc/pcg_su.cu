@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
   extern __shared__ __align__(16) char dyn[];
   __shared__ SceneLite<float> S;
   __shared__ SState<float> st;
-  __shared__ int s_to, s_nh;
+  __shared__ int s_to, s_nh, s_widx;
+  __shared__ unsigned s_seen;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_posts = A.plan.n_posts, n_tiles = (A.plan.nv + PCG_TILE - 1) / PCG_TILE;
   constexpr int rows = ROWS, per_tile = PCG_TILE / rows, ng = rows / 16;
@@ -93,6 +94,8 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
   if (tid == 0) {
     load_lite(S, *A.scene);
     s_to = s_nh = 0;
+    s_widx = -1;
+    s_seen = 0;
     st.done = 0;
   }
   for (int h = tid; h < hs; h += SU_NT) L.hkey[h] = -1;
@@ -215,6 +218,13 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
   const int max_iter = S.max_iter;
   float4* const zw = reinterpret_cast<float4*>(S.zrec);
   float4* const my_line = A.words + (size_t)blockIdx.x * 2 * SU_LINE;
+  // after a wait ran out: the first word found without stamp s, for the timeout record (looked for here, as
+  // the waits' loops are the kernel's pace: 2.18 -> 2.27 us per CG iteration when they kept it)
+  auto note_missing = [&](const float4* q, unsigned s, int index) {
+    unsigned long long a, b;
+    ld_word4(q, a, b);
+    if (word4_stamp(b) != s && atomicCAS(&s_widx, -1, index) == -1) s_seen = word4_stamp(b);
+  };
 
   for (int it = 0;; ++it) {
     const unsigned s = (unsigned)it + 1;
@@ -281,7 +291,7 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
           unsigned long long va, vb;
           ld_word4(wpar + hrow[k], va, vb);
           for (unsigned spins = 0; word4_stamp(vb) != s; ++spins) {
-            if (spins > kWaitSpins || *(volatile int*)&s_to) {
+            if (spins > A.wait_limit || *(volatile int*)&s_to) {
               s_to = 3;
               break;
             }
@@ -298,7 +308,7 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
           const float4* q = z ? line + 1 : line + par * SU_LINE;
           ld_word4(q, va, vb);
           for (unsigned spins = 0; word4_stamp(vb) != s; ++spins) {
-            if (spins > kWaitSpins || *(volatile int*)&s_to) {
+            if (spins > A.wait_limit || *(volatile int*)&s_to) {
               s_to = 2;
               break;
             }
@@ -316,9 +326,22 @@ __global__ void __launch_bounds__(SU_NT, 1) k_pcg_su(SuLaunch A) {
     }
     __syncthreads();
     if (s_to) {
+      const int site = s_to;  // (a halo row's word and a post's may both be missing: the one noted last names the wait)
+      if (halo_thr) {
+        if (site == 3) {
+          for (int k = 0; k < HPT; ++k)
+            if (hrow[k] >= 0) note_missing(wpar + hrow[k], s, hrow[k]);
+        } else {
+          for (int un = SU_NT - 1 - tid; un < n_posts; un += n_halo_thr)
+            note_missing(A.words + (size_t)un * 2 * SU_LINE + par * SU_LINE, s, un);
+        }
+      }
+      __syncthreads();
       if (tid == 0) {
         if (atomicCAS(&A.bar->to_site, 0, s_to) == 0) {
           A.bar->to_iter = (unsigned)it;
+          A.bar->to_seen = s_seen;
+          A.bar->to_index = s_widx;
           A.bar->to_cta = (int)blockIdx.x;
         }
         atomicExch(&A.bar->timeout, 1);
