@@ -4,6 +4,9 @@ mixed scenes of at most a tile per SM against the halo layout, the allocation-fr
 against the global-memory kernel.  Same sums in the same order, so the iterates are equal bit for bit at every size: fewer rows than a unit,
 exact and ragged units and tiles, one and several units per CTA, more tiles than lanes."""
 
+import dataclasses
+import time
+
 import numpy as np
 import pytest
 
@@ -158,3 +161,69 @@ def test_allocation_free_solve_runs_the_unit_kernel():
         P.ppn.pcg_solve_static(d_rp.data_ptr(), d_col.data_ptr(), d_val.data_ptr(), n, len(col), d_x.data_ptr(),
                                d_x.data_ptr(), max_iter=2)
         assert P.ppn.pcg_static_solver() == want, dims
+
+
+def shuffled(dims, seed):
+    """A mesh whose vertices are numbered at random: every CTA's halo is spread over all the others."""
+    spec = twisting_beam_scene(*dims, h=0.1, seed=3)
+    X, rp, col, K, b = springs(dims, seed)
+    n = len(X)
+    inv = np.random.default_rng(seed).permutation(n)
+    i, j = inv[np.repeat(np.arange(n), np.diff(rp))], inv[col]
+    order = np.lexsort((j, i))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(i, minlength=n))])
+    back = np.argsort(inv)
+    spec = dataclasses.replace(spec, rest=spec.rest[back], tets=inv[spec.tets].astype(np.int32),
+                               fixed=np.sort(inv[spec.fixed]).astype(np.int32), targets=None)
+    return spec, rp, j[order].astype(np.int32), K[order], b
+
+
+def on_device(rp, col, K, b):
+    dev = torch.device("cuda", 0)
+    return [torch.tensor(a, device=dev) for a in (
+        rp.astype(np.int32), col, np.ascontiguousarray(K.reshape(-1, 9).T.astype(np.float32)),
+        np.pad(b, ((0, 0), (0, 1))).astype(np.float32), np.zeros((len(b), 4), np.float32))]
+
+
+def solve_static(t, **kw):
+    return P.ppn.pcg_solve_static(t[0].data_ptr(), t[1].data_ptr(), t[2].data_ptr(), len(t[3]), len(t[1]),
+                                  t[3].data_ptr(), t[4].data_ptr(), **kw)
+
+
+# the halo rows' sort: 0, 114, 333 and 420 rows of a CTA, 838 and 1571, 1654, and 2069 and 3191, in the three unit kernels
+@pytest.mark.parametrize("dims", [(2, 4, 4), (3, 4, 13), (8, 8, 16), (16, 16, 19), (16, 16, 38), (16, 19, 64), (20, 20, 60)])
+def test_meshes_without_an_order(dims, monkeypatch):
+    spec, rp, col, K, b = shuffled(dims, 9)
+    t = on_device(rp, col, K, b)
+    info = solve_static(t, rel_tol=1e-5)
+    assert P.ppn.pcg_static_solver() in ("rd", "rd_read")
+    runs = []
+    for prec, env, tol in ((P.PREC_MIXED, "PPN_PCG_GLOBAL", 1e-5), (P.PREC_MIXED, None, 1e-5), (P.PREC_MIXED, "PPN_PCG_NO_HALO", 1e-5),
+                           (P.PREC_FP64, None, 1e-7), (P.PREC_FP64, "PPN_PCG_NO_UNITS", 1e-7)):
+        with monkeypatch.context() as m:
+            if env:
+                m.setenv(env, "1")
+            sc = P.Scene.from_spec(spec, precision=prec)
+            p_rp, p_col = sc.probe_pattern()
+            assert np.array_equal(p_rp, rp) and np.array_equal(p_col, col)
+            runs.append((*sc.probe_pcg(K, b, rel_tol=tol), sc.probe_solver()))
+            sc.close()
+    if len(b) <= 1024:  # (more halo rows than threads take in the mixed scenes, or than fit in FP64)
+        assert runs[1][2] == "su" and runs[3][2] == "rd"
+    assert info == runs[0][1] and np.array_equal(t[4][:, :3].cpu().numpy().astype(np.float64), runs[0][0])
+    for a, c in ((1, 2), (3, 4)):
+        assert runs[a][1] == runs[c][1] and np.array_equal(runs[a][0], runs[c][0])
+
+
+def test_a_mesh_without_an_order_sets_up_as_fast():
+    # 24000 rows, some 3300 halo rows per CTA: the set-up and one iteration, against the ordered mesh
+    best = []
+    for system in (springs((20, 20, 60), 9)[1:], shuffled((20, 20, 60), 9)[1:]):
+        t = on_device(*system)
+        times = []
+        for _ in range(30):
+            t0 = time.perf_counter()
+            solve_static(t, max_iter=1)
+            times.append(time.perf_counter() - t0)
+        best.append(min(times))
+    assert best[1] < 3 * best[0], best
