@@ -1283,13 +1283,14 @@ int pcg_team_max_grid(int device, size_t smem) {
 }
 
 // before a team launch: the barrier, and every job's seats, exchange words and w records, which carry
-// stamps of one launch only, in one launch (blocks (*, j): job j) instead of two memsets per scene
+// stamps of one launch only, in one launch (blocks (j, *): job j; a grid's y stops at 65535, and a batch may
+// have more scenes) instead of two memsets per scene
 constexpr int CLEAR_BLOCKS = 8;
 __global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* jobs, unsigned* seats, GridBar* bar) {
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *bar = GridBar{};
-  if (blockIdx.x == 0 && threadIdx.x == 0) seats[blockIdx.y] = 0;
-  const SceneDev<float>& S = scenes[jobs[blockIdx.y].scene];
-  const int n_thr = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.y == 0 && threadIdx.x == 0) seats[blockIdx.x] = 0;
+  const SceneDev<float>& S = scenes[jobs[blockIdx.x].scene];
+  const int n_thr = gridDim.y * blockDim.x, t0 = blockIdx.y * blockDim.x + threadIdx.x;
   ulonglong2* w = reinterpret_cast<ulonglong2*>(S.pword);
   ulonglong2* z = reinterpret_cast<ulonglong2*>(S.zrec);
   const int nw = 4 * S.n_ptiles * pword_stride(S.n_ptiles), nz = 2 * S.nv;  // 16-byte pieces
@@ -1299,7 +1300,7 @@ __global__ void k_pcg_team_clear(const SceneDev<float>* scenes, const TeamJob* j
 
 cudaError_t launch_pcg_team(const SceneDev<float>* scenes, const TeamLaunch& L, cudaStream_t st) {
   if (!L.jobs || L.n_jobs <= 0 || L.grid <= 0 || !L.bar || !L.seats) return cudaErrorInvalidValue;
-  k_pcg_team_clear<<<dim3(CLEAR_BLOCKS, L.n_jobs), 256, 0, st>>>(scenes, L.jobs, L.seats, L.bar);
+  k_pcg_team_clear<<<dim3(L.n_jobs, CLEAR_BLOCKS), 256, 0, st>>>(scenes, L.jobs, L.seats, L.bar);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = allow_shared((const void*)k_pcg_team, L.smem_bytes);
