@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <limits>
 #include <map>
@@ -113,7 +114,6 @@ struct Group {
   int* d_ids = nullptr;
   TileRef* d_pcgtiles = nullptr;
   TileRef* d_touchtiles = nullptr;  // (selected element, corner pair) tiles of the touched-block update
-  unsigned pcg_launch_seq = 0;
   std::vector<int> pcg_ids;  // slots of the tile table currently on the device
   int pcg_ntiles = 0;
   size_t pcg_smem_bytes = 0;  // > 0: resident PCG layout chosen for that table
@@ -447,7 +447,6 @@ struct Driver {
                               : L.smem_bytes  ? SOLVER_S
                                               : SOLVER_GLOBAL;
       }
-      L.launch_seq = ++G.pcg_launch_seq;
       L.flags = G.d_flags;
       L.n_pword = (int)sl.size();
       for (size_t k = 0; k < sl.size(); ++k) {

@@ -93,7 +93,6 @@ struct PcgLaunch {
   int halo_cap;          // most halo rows of one CTA
   void* zrec;            // SR_HALO: the scene's w words (zeroed before the launch)
   size_t zrec_bytes;
-  unsigned launch_seq;
   unsigned long long* flags;  // single-reduction kernel: per-CTA publication and progress flags (grid words)
   int n_pword;           // stamped partial arrays to clear before the launch
   void* pword[PCG_MAX_SCENES];

@@ -1333,14 +1333,14 @@ cudaError_t launch_pcg_sr(const SceneDev<float>* scenes, const PcgLaunch& L, cud
       (halo && (L.n_scenes != 1 || !L.zrec || L.n_tiles > NTP || !L.halo_off || !L.halo_col || !L.halo_ref || L.halo_cap < 0 ||
                 (L.n_tiles + L.grid - 1) / L.grid * PCG_TILE > SR_HALO_MAX_ROWS)))
     return cudaErrorInvalidValue;
-  // the barrier; flags, exchange words and w records carry stamps of this launch only
+  // the barrier; flags (not of the halo layout), exchange words and w records carry stamps of this launch only
   ClearList c{};
   auto clear = [&](void* p, size_t bytes) {
     c.p[c.n] = p;
     c.words[c.n++] = bytes / 8;
   };
   clear(L.bar, sizeof(GridBar));
-  clear(L.flags, sizeof(unsigned long long) * L.grid);
+  if (!halo) clear(L.flags, sizeof(unsigned long long) * L.grid);
   for (int k = 0; k < L.n_pword; ++k) clear(L.pword[k], L.pword_bytes[k]);
   if (halo) clear(L.zrec, L.zrec_bytes);
   k_sr_clear<<<dim3(halo ? 64 : 8, c.n), 256, 0, st>>>(c);

@@ -37,13 +37,6 @@ __device__ __forceinline__ void upd_px(float a, float b, float u, float& p, floa
   p = __fmaf_rn(b, p, u);
   x = __fmaf_rn(a, p, x);
 }
-__device__ __forceinline__ void st_relaxed_v2_u64(unsigned long long* p, unsigned long long a, unsigned long long b) {
-  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1,%2};" ::"l"(p), "l"(a), "l"(b) : "memory");
-}
-__device__ __forceinline__ void ld_relaxed_v2_u64(const unsigned long long* p, unsigned long long& a,
-                                                  unsigned long long& b) {
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-}
 
 // scalar step after the reduction of iteration `it` (it updates done so far):
 // stopping tests, then alpha and beta of the next direction, or the exits
