@@ -1183,8 +1183,8 @@ void launch_obst_gap(const SceneDev<T>* s, const TileRef* t, int n, int k0, cuda
 template <typename T>
 void launch_element(const SceneDev<T>* s, const TileRef* t, int n, int probe, cudaStream_t st) {
   if (!n) return;
-  // FP64: parts while the 4 sub-partitions of each of 152 SMs outnumber the warps
-  const int warps = n * EL_CTAS, fit = sizeof(T) == 8 ? 4 * 152 / warps : 1;
+  // FP64: parts while the 4 sub-partitions of all SMs outnumber the warps
+  const int warps = n * EL_CTAS, fit = sizeof(T) == 8 ? 4 * sm_count() / warps : 1;
   const int parts = fit >= 12 ? 12 : fit >= 6 ? 6 : fit >= 1 ? std::min(fit, 4) : 1;
   k_element<T><<<dim3(warps, parts), 32, 0, st>>>(s, t, probe);
 }
@@ -1198,7 +1198,7 @@ void launch_assemble(const SceneDev<T>* s, const TileRef* bt, int nb, const Tile
   if constexpr (sizeof(T) == 8) {
     if (nb + nv) k_assemble_seq<T><<<(nb + nv) * EL_CTAS, 32, 0, st>>>(s, bt, nb, vt, nv);
   } else {
-    if (nb && nb * EL_CTAS <= 32 * 152)
+    if (nb && nb * EL_CTAS <= 32 * sm_count())
       k_assemble<T, 32><<<nb * EL_CTAS, 32, 0, st>>>(s, bt, use_probe);
     else if (nb)
       k_assemble<T, TILE><<<nb, TILE, 0, st>>>(s, bt, use_probe);

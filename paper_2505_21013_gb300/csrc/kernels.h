@@ -7,6 +7,17 @@
 
 namespace ppn {
 
+// SMs of the current device
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return 1;
+  }
+  return n;
+}
+
 constexpr int PROJ_CTA = 128;  // threads per CTA of the projection kernel (register heavy)
 constexpr int PROJW_CTA = 128;  // threads per CTA of its warp form: 4 warps of 3 tets
 constexpr int PROJW_TETS = 3 * PROJW_CTA / 32;  // tets per CTA of the warp form

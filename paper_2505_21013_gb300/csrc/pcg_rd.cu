@@ -811,7 +811,7 @@ cudaError_t launch_pcg_rd(const RdLaunch<T>& L, cudaStream_t st) {
       p.n_posts != (nv + p.post_rows - 1) / p.post_rows || p.grid < 1 || p.grid > p.n_posts ||
       p.rows() > (sizeof(T) == 8 ? RD_ROWS_MAX_F64 : RD_NT) || (sizeof(T) == 4 && !L.z_words))
     return cudaErrorInvalidValue;
-  k_rd_clear<T><<<std::min(152, 1 + nv / 128), 256, 0, st>>>(L, nv);
+  k_rd_clear<T><<<std::min(sm_count(), 1 + nv / 128), 256, 0, st>>>(L, nv);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const void* k = rd_kernel<T>(L.resident);

@@ -50,10 +50,6 @@ namespace {
 constexpr int kMaxRows = PPN_PCG_STATIC_MAX_ROWS;
 constexpr int kMaxTiles = (kMaxRows + PCG_TILE - 1) / PCG_TILE;
 constexpr int kMaxDevices = 64;
-// rows up to which the unit kernel posts 32-row units (a CTA each up to the SM count): more CTAs for
-// the rows (2000 rows 7.5 -> 6.6 us per CG iteration against tiles); beyond, whole tiles: fewer words
-// for every CTA to poll (32000 rows 13.2 -> 10.1)
-constexpr int kUnitPostRows = 4864;
 constexpr int kErrPattern = 4;  // Ctl::error bit: the caller's BSR pattern is malformed
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -241,7 +237,10 @@ PPN_API ppn_status ppn_pcg_solve_static(const int32_t* row_ptr, const int32_t* c
   k_static_prep<<<nb, 256, 0, st>>>(row_ptr, col, n_rows, nnzb, A.diag, A.tiles, n_tiles, A.ctl);
   PPN_STATIC_CU(cudaGetLastError());
   // the unit kernel's shared-memory needs for this pattern (two counters of the control block)
-  const RdPlan plan = rd_plan(n_rows, n_rows <= kUnitPostRows ? 32 : PCG_TILE, D.n_sm);
+  // Posts of 32-row units while there is an SM for each: more CTAs for the rows (2000 rows 7.5 -> 6.6 us
+  // per CG iteration against tiles); beyond, of whole tiles: fewer words for every CTA to poll (32000 rows
+  // 13.2 -> 10.1).
+  const RdPlan plan = rd_plan(n_rows, n_rows <= 32 * D.n_sm ? 32 : PCG_TILE, D.n_sm);
   PPN_STATIC_CU(launch_rd_plan(row_ptr, col, plan, &A.ctl->error, &A.ctl->n_new, &A.ctl->n_touched, st));
   Ctl c{};
   PPN_STATIC_CU(cudaMemcpyAsync(&c, A.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));

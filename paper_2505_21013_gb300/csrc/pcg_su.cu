@@ -442,7 +442,7 @@ cudaError_t launch_pcg_su(const SuLaunch& L, cudaStream_t st) {
       (p.post_rows != 32 && p.post_rows != 64 && p.post_rows != PCG_TILE) ||
       p.n_posts != (p.nv + p.post_rows - 1) / p.post_rows || p.grid != p.n_posts || !hpt)
     return cudaErrorInvalidValue;
-  k_su_clear<<<std::min(152, 1 + p.nv / 64), 256, 0, st>>>(L);
+  k_su_clear<<<std::min(sm_count(), 1 + p.nv / 64), 256, 0, st>>>(L);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const void* k = su_kernel(p.post_rows, hpt);
