@@ -508,9 +508,9 @@ struct Driver {
   }
 
   // A group of scenes: those whose rows fit a team of CTAs go into one team launch (k_pcg_team) and
-  // leave `ids`.  Two tiles per CTA use an SM's time best (4.5 us per iteration of two tiles, 3.1
-  // of one); one tile per CTA is taken while all scenes' tiles fit the device at once (9 scenes of
-  // 1k to 13k tets: 10.2 -> 7.1 ms per step against the lockstep form).  The jobs run longest
+  // leave `ids`.  Two tiles per CTA use an SM's time best (3.6 us per iteration of two tiles, 2.5 to
+  // 2.8 of one); one tile per CTA is taken while all scenes' tiles fit the device at once (9 scenes of
+  // 1k to 13k tets: 10.2 -> 7.1 ms per step against the lockstep form when introduced).  The jobs run longest
   // first, by the scenes' last iteration counts.  A layout switch in the environment
   // (tests) keeps the lockstep forms.
   ppn_status solve_teams(std::vector<int>& ids, int b_from_g) {
@@ -741,7 +741,8 @@ struct Driver {
   // layout (FP32: pcg_su.cu), with the same bits, when their layout fits.
   // FP64: rows in 32-row units over all SMs, where 128-row tiles leave most SMs idle and 5.4 us of FP64
   // work per SpMV on the others.  125 rows: 22 -> 8.9 us per CG iteration, 6480 rows: 23.2 -> 10.6.
-  // FP32: scenes of at most one 128-row tile per SM; 756 rows 3.11 -> 2.20 us, 15840 rows 3.39 -> 2.54.
+  // FP32: scenes of at most one 128-row tile per SM; 756 rows 2.53 us in the halo layout, 2.17 here,
+  // 15872 rows 2.78 and 2.55.
   // PPN_PCG_NO_UNITS=1 keeps the other kernels (tests).
   bool plan_units(const SceneImpl<T>& s, int dev, int n_sm) {
     constexpr bool D = sizeof(T) == sizeof(double);

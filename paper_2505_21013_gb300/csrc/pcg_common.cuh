@@ -1,6 +1,6 @@
-// Helpers shared by the two cooperative PCG kernels (global-memory and
-// shared-memory-resident variants): bounded grid barrier, L2-only vector
-// loads, fixed-order reductions and the per-scene CG state.
+// Helpers shared by the cooperative PCG kernels (in global memory: pcg.cu; resident: pcg_smem.cu, pcg_sr.cu,
+// pcg_su.cu, pcg_rd.cu): bounded grid barrier, L2-only vector loads, fixed-order reductions and the
+// per-scene CG state.
 #pragma once
 
 #include <algorithm>

@@ -99,7 +99,7 @@ struct SrLayout {
   int* lrp;      // SR_RES, SR_HALO: [ni + 1] local row pointers (blocks in CTA order)
   int* lgb;      // SR_RES, SR_HALO: [ni / 16 + 1] first slot step of each 16-row group
   int* lcol;     // SR_RES: [nb] columns; SR_HALO: [nb] local columns (own item, or ni + halo index); by slot
-  float* lval;   // SR_RES, SR_HALO: [nb * 9] by slot step: nine runs of 32 values
+  float* lval;   // SR_RES, SR_HALO: [nb * 9] by slot step, as slot_val
   float* lP;     // SR_RES, SR_STREAM: [ni * 6] inverse (00 01 02 11 12 22 of the symmetric block)
   float *lx, *lr, *lu, *lw, *lp, *ls;  // SR_RES, SR_STREAM: [ni * 3] each (SR_HALO: in registers)
   float4* lu4;   // SR_HALO: [ni + nh] u of the own rows, then of the halo rows (w while it arrives)
@@ -220,8 +220,8 @@ __device__ __forceinline__ bool sr_solve(
   constexpr int GP = SP_GP;             // lanes per BSR row in the SpMV
   constexpr int RPP = NTP / GP;         // rows per SpMV pass
   // blocks per lane per gather round: from shared memory four (more in flight lengthen the
-  // register-bound loop: 4.73 against 4.58 us per CG iteration on the beam), from global
-  // memory eight (the streamed SpMV waits on memory latency)
+  // register-bound loop: eight 4.00 against 3.62 us per CG iteration on the beam, two 3.58),
+  // row by row from global memory eight (that SpMV waits on memory latency)
   constexpr int U = RES ? 8 / GP : 16 / GP;
   constexpr int NW = NTP / 32;          // warps
   static_assert(RPP % PCG_TILE == 0 && NTP % PCG_TILE == 0, "passes cover whole tiles");
@@ -1184,8 +1184,9 @@ __global__ void __launch_bounds__(NTP, 1)
 // member that waits for its team waits for jobs that finish; all CTAs are co-resident
 // (cooperative launch).  That wait (sr_solve's for the seats) is the only one that spans other scenes'
 // solves.  After a timeout no further ticket is taken.
-// Bound, as the halo layout, by an iteration's latency; 64 scenes of 1k to 50k tets (150k rows,
-// 60 to 400 iterations each): 11.9 -> 2.8 ms per solve, 36.6 -> 18.1 ms per time step.
+// Bound, as the halo layout, by an iteration's latency; 64 scenes of 1k to 50k tets (163k rows,
+// 60 to 400 iterations each): 11.9 -> 2.8 ms per solve when introduced, 36.6 -> 14.8 ms per time step
+// with all that has changed since.
 __global__ void __launch_bounds__(NTP, 1)
     k_pcg_team(const SceneDev<float>* scenes, const TeamJob* jobs, int n_jobs, unsigned* seats, GridBar* bar,
                int b_from_g) {

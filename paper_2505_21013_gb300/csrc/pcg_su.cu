@@ -6,8 +6,9 @@
 // 6200 cycles per iteration: 2600 for the SpMV of 128 rows with its sums and posts, 1900 for the
 // grid's reduction, 740 for the scalar step of one thread between two barriers, 750 for updates
 // through shared memory and their barriers.  One way between two SMs through L2 is 500 to 850
-// cycles, so a reduction cannot take less than about 1000.  Here (756 rows 3.11 -> 2.20 us per CG
-// iteration, 4000 rows 3.27 -> 2.36, 15840 rows 3.39 -> 2.54; about 4300 cycles: SpMV 900, its sums
+// cycles, so a reduction cannot take less than about 1000.  Here (756 rows 3.11 -> 2.17 us per CG
+// iteration, 4096 rows 3.27 -> 2.35, 15872 rows 3.39 -> 2.55, where the halo layout, which has had some
+// of this since, takes 2.53, 2.75 and 2.78; about 4300 cycles: SpMV 900, its sums
 // 390, post and wait 1700, the scene's sums 400, scalar step 440, update and barriers 400):
 //   - a CTA has 32, 64 or 128 rows, as few as the SMs allow: the tile sum
 //     ((w0 + w1) + (w2 + w3)) + ((w4 + w5) + (w6 + w7)) of eight 16-row groups splits there, so that
