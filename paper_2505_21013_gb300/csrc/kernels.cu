@@ -63,7 +63,7 @@ __device__ __forceinline__ void load_u(const double4* U, int v, double* out) {
 // and g^e: a branch around g^e would save a few microseconds there, but changes the
 // compiler's choice of fused operations, and with it the FP64 bits of every scene.
 // One launch, 256-thread CTAs -> this: 384 tets FP64 57 -> 18.5 us; mixed, 4,350 tets 29 ->
-// 18.7 us, 171,114 tets 87 -> 75 us (the waves end more evenly).
+// 18.7 us, 171,114 tets 87 -> 74 us (the waves end more evenly).
 constexpr int EL_CTAS = TILE / 32;
 template <typename T>
 __global__ void __launch_bounds__(32) k_element(const SceneDev<T>* scenes, const TileRef* tiles,
