@@ -22,7 +22,8 @@
  *     inside kernels are bounded and report PPN_ERR_TIMEOUT.
  *   - A scene owns its device memory (cudaMalloc at creation, or the allocator
  *     installed with ppn_set_allocator; freed at destruction) and runs on its own
- *     stream unless ppn_set_stream is called.
+ *     stream unless ppn_set_stream is called.  It also pins 48 bytes of host memory
+ *     per vertex, at most 768 KB, for state in and out (not in device_bytes).
  *   - Not thread-safe per scene: calls on one scene must not overlap.
  */
 #ifndef PPN_H
